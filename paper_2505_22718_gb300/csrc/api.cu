@@ -368,8 +368,10 @@ int swcl_destroy(swcl_ctx* c) {
                     &c->bt_g32, &c->bt_kmu, &c->bt_himg, &c->bt_dimg, &c->ws_qpart, &c->bt_cmap_f,
                     &c->bt_cmap_a, &c->bt_lpos, &c->bt_wbase,
                     &c->ws_jin, &c->ws_dU, &c->ws_jout, &c->ws_fz, &c->ws_fsmall, &c->ws_lq,
-                    &c->ws_ltab, &c->hs_C, &c->hs_Cb, &c->hs_Pb, &c->hs_Ab, &c->hs_Wb};
+                    &c->ws_ltab, &c->ws_ckpart, &c->hs_C, &c->hs_Cb, &c->hs_Pb, &c->hs_Ab, &c->hs_Wb};
   for (DevBuf* b : bufs) swcl::release(c, *b);
+  for (auto& p : c->ck)
+    for (auto& d : p) swcl::release(c, d.tab);
   for (auto& t : c->tc) {
     swcl::release(c, t.bfwd);
     swcl::release(c, t.bvjp);
@@ -442,6 +444,7 @@ int swcl_set_grids(swcl_ctx* c, double chi_min, double chi_max, int N, const dou
   c->k_h = kh;
   c->knots_h = knh;
   c->ells_h = eh;
+  swcl::chirp_fit_grid(c);
   c->last_fwd_precision = -1;
   c->u_valid = false;
   SWCL_TRY(swcl::copy_in(c, c->d_k, kh.data(), sizeof(double) * N_k));
@@ -749,7 +752,7 @@ static int check_ready(swcl_ctx* c, int precision) {
 // Dbar (and, in basis mode, the per-call GEMM operands) for every multipole at once.  Then the
 // forward pass contracts and integrates chunk by chunk, and the VJP recomputes each chunk's
 // Delta before its reverse mode.  Returns 0 when not even 8 multipoles fit.
-static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need) {
+static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need, bool whole_part) {
   // n_need: the multipoles that take the FFTLog path (all but the Limber rows)
   if (n_need <= 0) return c->N_ell;
   const int N_ell = c->N_ell;
@@ -771,9 +774,10 @@ static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need) {
                  + swcl::delta_bar_scratch_bytes(c->n_walk, c->N_k, N_ell)
                  + sizeof(double) * (nw * c->N_k + nrow);
   if (basis) fixed += swcl::basis_fixed_bytes(c);
+  fixed += swcl::chirp_part_bytes(c, precision, n_need, whole_part);
   const DevBuf* ws[] = {&c->ws_coef, &c->ws_delta, &c->ws_U, &c->ws_C, &c->ws_cbar, &c->ws_dbar,
                         &c->ws_Cbar, &c->ws_outP, &c->ws_outA, &c->ws_outW, &c->ws_pbpart,
-                        &c->ws_qpart, &c->bt_eimg_f, &c->bt_eimg_a, &c->bt_gdf, &c->bt_g32, &c->bt_kmu,
+                        &c->ws_qpart, &c->ws_ckpart, &c->bt_eimg_f, &c->bt_eimg_a, &c->bt_gdf, &c->bt_g32, &c->bt_kmu,
                         &c->bt_himg, &c->bt_dimg};
   size_t ws_now = 0;
   for (const DevBuf* b : ws) ws_now += b->bytes;
@@ -784,10 +788,28 @@ static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need) {
   return (int)std::min<size_t>(n_need, std::max<size_t>(8, n / 8 * 8));
 }
 
+// The same with the tables of the chirp transforms built first.  Where the budget has no room for 8
+// multipoles beside them, their partial sums are planned at the least, then they are given up.
+static int plan_chunk(swcl_ctx* c, int precision, int n_need, int& n_lc) {
+  SWCL_TRY(swcl::chirp_prepare(c, precision));
+  n_lc = plan_ell_chunk(c, precision, n_need, true);
+  if (n_lc == 0 && swcl::chirp_use(c, precision)) {
+    n_lc = plan_ell_chunk(c, precision, n_need, false);
+    if (n_lc == 0) {
+      swcl::chirp_drop(c);
+      n_lc = plan_ell_chunk(c, precision, n_need, true);
+    }
+  }
+  if (n_lc == 0)
+    return swcl::fail(c, SWCL_ERR_OOM_BUDGET, "memory budget too small for 8 multipoles of Delta");
+  return SWCL_OK;
+}
+
 // Delta for multipoles [l_lo, l_lo + n_l) into ws_delta ([n_walk][n_l][N_tr][N_k])
 static int contract_chunk(swcl_ctx* c, int precision, int l_lo, int n_l) {
   const swcl::Stencil sv = swcl::stencil(c);
   if (!use_basis_gemm(c, precision)) c->bt_delta_clean = false;   // every row rewritten
+  if (precision == SWCL_FP64 && swcl::chirp_use(c, precision)) return swcl::chirp_forward(c, precision, l_lo, n_l);
   if (precision == SWCL_FP64) {
     SWCL_LAUNCH(c, swcl::launch_contract_fp64((double*)c->ws_delta.p, (const cplx*)c->ws_coef.p,
                                               (const cplx*)c->d_phase.p, (const cplx*)c->d_gtab.p,
@@ -891,9 +913,8 @@ int swcl_compute_cl(swcl_ctx* c, int precision, double* C_out) {
   // the Limber table and scratch first, so that the multipole chunks are planned around them
   swcl::LimberTable lt;
   if (lim.n_lim > 0) SWCL_TRY(limber_prepare(c, lim, nw, lt));
-  const int n_lc = plan_ell_chunk(c, precision, n_fft);
-  if (n_lc == 0)
-    return swcl::fail(c, SWCL_ERR_OOM_BUDGET, "memory budget too small for 8 multipoles of Delta");
+  int n_lc = 0;
+  SWCL_TRY(plan_chunk(c, precision, n_fft, n_lc));
   SWCL_TRY(swcl::ensure(c, c->ws_coef, sizeof(cplx) * nrow * N_I * n_h));
   SWCL_TRY(swcl::ensure(c, c->ws_delta, nrow * n_lc * N_k * (fp64 ? sizeof(double) : sizeof(float))));
   SWCL_TRY(swcl::ensure(c, c->ws_U, sizeof(double) * nw * (size_t)N_ell * N_tr * N_tr));
@@ -1062,7 +1083,9 @@ int swcl_vjp(swcl_ctx* c, int precision, const double* C_bar, double* P_bar, dou
                                                    c->pdl && !c->prof),
                   "delta_bar f32");
     if (!W_bar) continue;
-    if (fp64) {
+    if (fp64 && swcl::chirp_use(c, precision)) {
+      SWCL_TRY(swcl::chirp_adjoint(c, precision, l_lo, n_l, accumulate));
+    } else if (fp64) {
       SWCL_LAUNCH(c, swcl::launch_contract_fp64_adj((cplx*)c->ws_cbar.p, (const double*)c->ws_dbar.p,
                                                     (const cplx*)c->d_phase.p,
                                                     (const cplx*)c->d_gtab.p,
@@ -1451,9 +1474,8 @@ int swcl_jvp(swcl_ctx* c, int precision, int n_dir, const double* P_dot, const d
   c->u_valid = false;
   {
     WalkScope scope(c, nw2);
-    const int n_lc = plan_ell_chunk(c, precision, n_fft);
-    if (n_lc == 0)
-      return swcl::fail(c, SWCL_ERR_OOM_BUDGET, "memory budget too small for 8 multipoles of Delta");
+    int n_lc = 0;
+    SWCL_TRY(plan_chunk(c, precision, n_fft, n_lc));
     c->ell_chunk = n_lc;
     c->ell_fft = n_fft;
     SWCL_TRY(swcl::ensure(c, c->ws_coef, sizeof(cplx) * nw2 * N_tr * N_I * n_h));

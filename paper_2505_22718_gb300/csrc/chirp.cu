@@ -1,0 +1,162 @@
+// Chirp transforms of the contraction (chirp.cuh): when they apply, their tables, and how the rows
+// are split over CTAs.
+#include <algorithm>
+#include <cmath>
+
+#include "swcl_internal.h"
+
+namespace swcl {
+
+// ln k_q = x0 + q d to rounding: the line through the end points (their logarithms in extended
+// precision), with no point further off than a few rounding errors of ln k.  The phases
+// e^{-i eta_n ln k_q} of the line then differ from those of the grid by no more than a
+// double-precision ln k does.  Grids that geomspace, logspace or an exponential of a linspace give
+// pass; one rounded to seven digits, or perturbed by 1e-12, does not (tests/test_gpu_chirp.py).
+void chirp_fit_grid(swcl_ctx* c) {
+  c->ck_uniform = false;
+  c->ck_off = false;
+  for (auto& p : c->ck)
+    for (auto& d : p) d.ready = false;
+  const int n = c->N_k;
+  if (n < 3) return;
+  const long double x0 = logl((long double)c->k_h[0]);
+  const long double d = (logl((long double)c->k_h[n - 1]) - x0) / (n - 1);
+  const double x0d = (double)x0, dd = (double)d;
+  const double tol = 4.0 * 2.220446e-16 * std::max({4.0, std::fabs(std::log(c->k_h[0])),
+                                                   std::fabs(std::log(c->k_h[n - 1]))});
+  for (int q = 0; q < n; ++q)
+    if (std::fabs(std::log(c->k_h[q]) - std::fma(dd, (double)q, x0d)) > tol) return;
+  const long double cc = d / (2.0L * (long double)c->L), xx = x0 / (long double)c->L;
+  c->ck_c[0] = (double)cc;
+  c->ck_c[1] = (double)(cc - (long double)c->ck_c[0]);
+  c->ck_x[0] = (double)xx;
+  c->ck_x[1] = (double)(xx - (long double)c->ck_x[0]);
+  c->ck_uniform = true;
+}
+
+namespace {
+
+// smallest M = 2^m, m = 9..13, that holds the linear convolution; 0 = none
+int log_size(int n_in, int n_out) {
+  for (int m = 9; m <= 13; ++m)
+    if (n_in + n_out - 1 <= (1 << m)) return m;
+  return 0;
+}
+
+constexpr int kFirst64 = 1;    // FP64: the term n = 0 (phase 1) is added beside the transform
+
+}  // namespace
+
+// Transforms per (walker, tracer, multipole): the profile rows of basis mode, or up to four knots.
+int chirp_rank(const swcl_ctx* c) { return c->lr_basis ? c->lr_true_rank : c->N_I <= 4 ? c->N_I : 0; }
+
+bool chirp_use(const swcl_ctx* c, int precision) {
+  if (!c->ck_uniform || c->ck_off || precision != SWCL_FP64) return false;
+  const int r = chirp_rank(c), mf = log_size(c->n_h - kFirst64, c->N_k), ma = log_size(c->N_k, c->n_h);
+  if (r <= 0 || !mf || !ma) return false;
+  // FP64 operations: about 75 per point and pair of FFTs, against 2 per (frequency, k point) of the
+  // direct sum (four profile rows cost four transforms but one direct sum).  Both sides are bound by
+  // the FP64 pipe: forward + VJP at N = 2048, N_k = 1024, 103 multipoles, 15 tracers 1.01 ms against
+  // 12.8 ms; N = N_k = 256, 20 multipoles, 2 tracers (three quarters of the line) 0.24 against 0.79 ms.
+  return 75.0 * r * (double)(1 << std::max(mf, ma)) < 2.0 * c->n_h * (double)c->N_k;
+}
+
+void chirp_drop(swcl_ctx* c) {
+  for (auto& p : c->ck)
+    for (auto& d : p) {
+      release(c, d.tab);
+      d.ready = false;
+    }
+  release(c, c->ws_ckpart);
+  c->ck_off = true;
+}
+
+int chirp_prepare(swcl_ctx* c, int precision) {
+  if (!chirp_use(c, precision)) return SWCL_OK;
+  for (int dir = 0; dir < 2; ++dir) {
+    ChirpDir& d = c->ck[0][dir];
+    if (d.ready) continue;
+    if (c->capturing) return fail(c, SWCL_ERR_STATE, "chirp tables built during capture");
+    d.n0 = dir == 0 ? kFirst64 : 0;
+    const int n_freq = c->n_h - d.n0;
+    d.logm = dir == 0 ? log_size(n_freq, c->N_k) : log_size(c->N_k, n_freq);
+    const int M = 1 << d.logm;
+    d.half = c->N_k <= M / 2 && n_freq <= M / 2 + (dir == 0 ? 0 : 1);
+    const int st = ensure(c, d.tab, chirp64_table_bytes(d.logm, n_freq, c->N_k));
+    if (st == SWCL_ERR_OOM_BUDGET) {   // the direct sums need no tables
+      chirp_drop(c);
+      c->err.clear();
+      return SWCL_OK;
+    }
+    if (st) return st;
+    const int t_lo = dir == 0 ? n_freq - 1 : c->N_k - 1, t_hi = dir == 0 ? c->N_k - 1 : n_freq - 1;
+    const cudaError_t e = chirp64_build(d.tab.p, d.logm, d.n0, n_freq, c->N_k, t_lo, t_hi, c->ck_c, c->ck_x,
+                                        c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "chirp tables");
+    d.ready = true;
+  }
+  return SWCL_OK;
+}
+
+// CTAs per row (each takes an equal share of the row's multipoles): enough CTAs for several turns of
+// what the GPU holds at once, so that the last turn is a small part, and no more, since each CTA
+// loads its row's coefficients and weights once.
+static int row_chunks(const swcl_ctx* c, long rows, int n_l, int logm) {
+  const int threads = logm == 13 ? 256 : (1 << logm) / 16;
+  const long slots = (long)c->num_sms * std::max(1, 256 / threads);
+  const long per = std::max<long>(1, rows * n_l / (8 * slots));
+  return (int)std::min<long>(n_l, (n_l + per - 1) / per);
+}
+
+// Bytes of the adjoint's partial sums over n_l multipoles (whole: with every CTA of a row its own)
+size_t chirp_part_bytes(const swcl_ctx* c, int precision, int n_l, bool whole) {
+  if (!chirp_use(c, precision)) return 0;
+  const long rows = (long)c->n_walk * c->N_tr;
+  const int n = whole ? row_chunks(c, rows, n_l, log_size(c->N_k, c->n_h)) : 1;
+  return sizeof(cplx) * rows * chirp_rank(c) * c->n_h * n;
+}
+
+int chirp_forward(swcl_ctx* c, int precision, int l_lo, int n_l) {
+  (void)precision;
+  const ChirpDir& d = c->ck[0][0];
+  const Stencil sv = stencil(c);
+  const long rows = (long)c->n_walk * c->N_tr;
+  ChirpRun r{c->n_walk, c->N_tr, sv.NI, c->n_h, c->N_k, c->N_ell, l_lo, n_l, chirp_rank(c),
+             row_chunks(c, rows, n_l, d.logm), nullptr, nullptr};
+  ++c->last_launches;
+  prof_begin(c);
+  const cudaError_t e = chirp64_forward(d, (double*)c->ws_delta.p, (const cplx*)c->ws_coef.p,
+                                        (const cplx*)c->d_gtab.p, (const int*)c->d_cls_of.p, sv.w, sv.w_ts,
+                                        (const double*)c->d_kpow.p, r, c->stream);
+  prof_end(c, "chirp fwd fp64");
+  return e == cudaSuccess ? SWCL_OK : cuda_fail(c, e, "chirp fwd fp64");
+}
+
+int chirp_adjoint(swcl_ctx* c, int precision, int l_lo, int n_l, bool accumulate) {
+  (void)precision;
+  const ChirpDir& d = c->ck[0][1];
+  const Stencil sv = stencil(c);
+  const long rows = (long)c->n_walk * c->N_tr;
+  const int rank = chirp_rank(c);
+  ChirpRun r{c->n_walk, c->N_tr, sv.NI, c->n_h, c->N_k, c->N_ell, l_lo, n_l, rank,
+             row_chunks(c, rows, n_l, d.logm), nullptr, nullptr};
+  // partial sums of the CTAs of a row; under a tight budget one CTA per row
+  const size_t per = chirp_part_bytes(c, precision, n_l, false);
+  if (c->budget && c->held - c->ws_ckpart.bytes + per * r.n_chunk > c->budget) r.n_chunk = 1;
+  const int st = ensure(c, c->ws_ckpart, per * r.n_chunk);
+  if (st) return st;
+  ++c->last_launches;
+  prof_begin(c);
+  cudaError_t e = chirp64_adjoint(d, c->ws_ckpart.p, (const double*)c->ws_dbar.p, (const cplx*)c->d_gtab.p,
+                                  (const int*)c->d_cls_of.p, sv.w, sv.w_ts, (const double*)c->d_kpow.p, r,
+                                  c->stream);
+  prof_end(c, "chirp adj fp64");
+  if (e != cudaSuccess) return cuda_fail(c, e, "chirp adj fp64");
+  ++c->last_launches;
+  prof_begin(c);
+  e = chirp64_sum((cplx*)c->ws_cbar.p, c->ws_ckpart.p, d, r, accumulate, c->stream);
+  prof_end(c, "chirp adj sum");
+  return e == cudaSuccess ? SWCL_OK : cuda_fail(c, e, "chirp adj sum");
+}
+
+}  // namespace swcl

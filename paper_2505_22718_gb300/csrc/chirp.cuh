@@ -1,0 +1,741 @@
+// The contraction over the FFTLog frequencies as a chirp transform (a3 and its transpose), for k
+// grids that are uniform in ln k:  ln k_q = x0 + q d.
+//
+// With eta_n = 2 pi n/L and beta = 2 pi d/L the phase of Eq. 3.4-3.5 is e^{-i eta_n ln k_q} =
+// e^{-i eta_n x0} e^{-i beta n q}, and with n = n0 + m, m q = (m^2 + q^2 - (m - q)^2)/2 (Bluestein):
+//   sum_{n >= n0} F_n G_n e^{-i eta_n ln k_q} = b_q sum_m [F_n G_n a_n] h_{q - m},
+//   a_n = e^{-i eta_n x0 - i beta m^2/2},  b_q = e^{-i beta (n0 q + q^2/2)},  h_t = e^{+i beta t^2/2},
+// a linear convolution with one fixed filter: two FFTs of M >= (frequencies) + N_k - 1 points per
+// row (walker, tracer, multipole) instead of 4 n_h N_k operations.  The transpose is the same
+// convolution with the roles of m and q exchanged:
+//   sum_q d_q e^{-i eta_n ln k_q} = a_n sum_q [d_q b_q] h_{n - q}                  (n0 = 0),
+// multiplied by G[l][n] and summed over the multipoles before the factor a_n.
+//
+// One CTA of M/16 threads (16 points each; 32 for M = 8192) runs one row at a time: a forward FFT
+// of passes 16 x 16 x M/256 with the frequencies left in digit-reversed order, the product with the
+// filter's spectrum (stored in that order), and the inverse passes in reverse.  Each pass works in
+// registers; passes exchange through shared memory in place (a thread writes back the places it has
+// read), so the second and third pass, which stay within 16 neighbouring threads, need a warp
+// barrier only and a row needs two CTA barriers.  The window of the frequencies and of the k points
+// is at most M/2 in the HALF form: half of the first pass's inputs are then zero and half of the
+// last pass's outputs unused.
+//
+// FP64: bound by the FP64 pipe (two FMA per clock and SM): about 1160 FP64 instructions per thread and
+// row of 2048 points, so the largest radix whose points fit the registers (fewest twiddle products)
+// and eight resident warps are enough.  15 tracers x 103 multipoles, N = 2048, N_k = 1024: 484 us
+// forward and 463 us transposed (75 % of the pipe's rate; the last of six turns of two CTAs per SM is
+// nearly empty), against 5.9 ms each for the direct sums.
+#pragma once
+#include <algorithm>
+#include <type_traits>
+
+#include "swcl_internal.h"
+
+namespace swcl {
+namespace chirp {
+
+template <class T> struct Vec2;
+template <> struct Vec2<float> { using type = float2; };
+template <> struct Vec2<double> { using type = double2; };
+template <class T> using V2 = typename Vec2<T>::type;
+
+template <class T> __device__ __forceinline__ V2<T> mk(T x, T y) { V2<T> v; v.x = x; v.y = y; return v; }
+template <class V> __device__ __forceinline__ V add(V a, V b) { a.x += b.x; a.y += b.y; return a; }
+template <class V> __device__ __forceinline__ V sub(V a, V b) { a.x -= b.x; a.y -= b.y; return a; }
+// a b, and a conj(b)
+template <class V> __device__ __forceinline__ V mul(V a, V b) {
+  V r;
+  r.x = fma(a.x, b.x, -a.y * b.y);
+  r.y = fma(a.x, b.y, a.y * b.x);
+  return r;
+}
+template <class V> __device__ __forceinline__ V mulc(V a, V b) {
+  V r;
+  r.x = fma(a.x, b.x, a.y * b.y);
+  r.y = fma(a.y, b.x, -a.x * b.y);
+  return r;
+}
+// a times i S (S = +1 or -1)
+template <int S, class V> __device__ __forceinline__ V rot(V a) {
+  V r;
+  if constexpr (S > 0) { r.x = -a.y; r.y = a.x; } else { r.x = a.y; r.y = -a.x; }
+  return r;
+}
+
+// ---- DFTs in registers, X_k = sum_n v_n e^{2 pi i S n k / R}, natural order in and out ----
+
+template <int S, class V> __device__ __forceinline__ void dft4(V& a, V& b, V& c, V& d) {
+  const V s0 = add(a, c), d0 = sub(a, c), s1 = add(b, d), d1 = rot<S>(sub(b, d));
+  a = add(s0, s1);
+  b = add(d0, d1);
+  c = sub(s0, s1);
+  d = sub(d0, d1);
+}
+// c = d = 0
+template <int S, class V> __device__ __forceinline__ void dft4_half(V& a, V& b, V& c, V& d) {
+  const V a0 = a, b0 = b, r = rot<S>(b);
+  a = add(a0, b0);
+  b = add(a0, r);
+  c = sub(a0, b0);
+  d = sub(a0, r);
+}
+
+// cos and sin of 2 pi j/32 (j mod 32; the quadrant's nine values, the rest by symmetry)
+__host__ __device__ constexpr double cos32(int j) {
+  constexpr double c[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613,
+                           0.83146961230254523708, 0.70710678118654752440,
+                           0.55557023301960222474, 0.38268343236508977173,
+                           0.19509032201612826785, 0.0};
+  j &= 31;
+  if (j > 16) j = 32 - j;
+  return j <= 8 ? c[j] : -c[16 - j];
+}
+__host__ __device__ constexpr double sin32(int j) { return cos32(j + 24); }   // cos(x - pi/2)
+
+// v e^{2 pi i S j / 32}, J a compile-time constant
+template <int S, int J, class V> __device__ __forceinline__ V tw32(V v) {
+  constexpr int j = J & 31;
+  if constexpr (j == 0) {
+    return v;
+  } else if constexpr (j == 8) {
+    return rot<S>(v);
+  } else if constexpr (j == 16) {
+    V r;
+    r.x = -v.x;
+    r.y = -v.y;
+    return r;
+  } else {
+    using T = decltype(v.x);
+    constexpr T c = (T)cos32(j), s = (T)(S * sin32(j));
+    V r;
+    if constexpr (j == 4) {
+      const T h = c;
+      if constexpr (S > 0) { r.x = (v.x - v.y) * h; r.y = (v.x + v.y) * h; }
+      else { r.x = (v.x + v.y) * h; r.y = (v.y - v.x) * h; }
+    } else if constexpr (j == 12) {
+      const T h = -c;
+      if constexpr (S > 0) { r.x = -(v.x + v.y) * h; r.y = (v.x - v.y) * h; }
+      else { r.x = (v.y - v.x) * h; r.y = -(v.x + v.y) * h; }
+    } else {
+      r.x = fma(v.x, c, -v.y * s);
+      r.y = fma(v.x, s, v.y * c);
+    }
+    return r;
+  }
+}
+
+template <int S, class V> __device__ __forceinline__ void dft2(V* v) {
+  const V a = v[0];
+  v[0] = add(a, v[1]);
+  v[1] = sub(a, v[1]);
+}
+template <int S, class V> __device__ __forceinline__ void dft8(V* v) {
+  V u[4], w[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    u[j] = add(v[j], v[j + 4]);
+    w[j] = sub(v[j], v[j + 4]);
+  }
+  w[1] = tw32<S, 4>(w[1]);
+  w[2] = tw32<S, 8>(w[2]);
+  w[3] = tw32<S, 12>(w[3]);
+  dft4<S>(u[0], u[1], u[2], u[3]);
+  dft4<S>(w[0], w[1], w[2], w[3]);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    v[2 * j] = u[j];
+    v[2 * j + 1] = w[j];
+  }
+}
+// the same with v[4..7] = 0
+template <int S, class V> __device__ __forceinline__ void dft8_half(V* v) {
+  V u[4] = {v[0], v[1], v[2], v[3]};
+  V w[4] = {v[0], tw32<S, 4>(v[1]), tw32<S, 8>(v[2]), tw32<S, 12>(v[3])};
+  dft4<S>(u[0], u[1], u[2], u[3]);
+  dft4<S>(w[0], w[1], w[2], w[3]);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    v[2 * j] = u[j];
+    v[2 * j + 1] = w[j];
+  }
+}
+// n = 4 n1 + n2, k = k1 + 4 k2
+template <int S, bool HALF, class V> __device__ __forceinline__ void dft16(V* v) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if constexpr (HALF) dft4_half<S>(v[j], v[j + 4], v[j + 8], v[j + 12]);
+    else dft4<S>(v[j], v[j + 4], v[j + 8], v[j + 12]);
+  }
+  // now v[4 k1 + n2]; times w16^{n2 k1}
+  v[5] = tw32<S, 2>(v[5]);
+  v[6] = tw32<S, 4>(v[6]);
+  v[7] = tw32<S, 6>(v[7]);
+  v[9] = tw32<S, 4>(v[9]);
+  v[10] = tw32<S, 8>(v[10]);
+  v[11] = tw32<S, 12>(v[11]);
+  v[13] = tw32<S, 6>(v[13]);
+  v[14] = tw32<S, 12>(v[14]);
+  v[15] = tw32<S, 18>(v[15]);
+#pragma unroll
+  for (int k1 = 0; k1 < 4; ++k1) dft4<S>(v[4 * k1], v[4 * k1 + 1], v[4 * k1 + 2], v[4 * k1 + 3]);
+  // v[4 k1 + k2] -> X[k1 + 4 k2]
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = a + 1; b < 4; ++b) {
+      const V t = v[4 * a + b];
+      v[4 * a + b] = v[4 * b + a];
+      v[4 * b + a] = t;
+    }
+}
+template <int S, int K1, class V> __device__ __forceinline__ void tw_row32(V* r) {   // w32^{n2 k1}
+  r[1] = tw32<S, K1>(r[1]);
+  r[2] = tw32<S, 2 * K1>(r[2]);
+  r[3] = tw32<S, 3 * K1>(r[3]);
+}
+// n = 4 n1 + n2, n1 < 8, k = k1 + 8 k2
+template <int S, bool HALF, class V> __device__ __forceinline__ void dft32(V* v) {
+  V y[8][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    V c[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) c[a] = v[4 * a + j];
+    if constexpr (HALF) dft8_half<S>(c); else dft8<S>(c);
+#pragma unroll
+    for (int a = 0; a < 8; ++a) y[a][j] = c[a];
+  }
+  tw_row32<S, 1>(y[1]);
+  tw_row32<S, 2>(y[2]);
+  tw_row32<S, 3>(y[3]);
+  tw_row32<S, 4>(y[4]);
+  tw_row32<S, 5>(y[5]);
+  tw_row32<S, 6>(y[6]);
+  tw_row32<S, 7>(y[7]);
+#pragma unroll
+  for (int a = 0; a < 8; ++a) {
+    dft4<S>(y[a][0], y[a][1], y[a][2], y[a][3]);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) v[a + 8 * b] = y[a][b];
+  }
+}
+// R points; HALF: v[R/2 .. R-1] = 0 on input
+template <int R, int S, bool HALF = false, class V> __device__ __forceinline__ void dft(V* v) {
+  if constexpr (R == 2) dft2<S>(v);
+  else if constexpr (R == 4) dft4<S>(v[0], v[1], v[2], v[3]);
+  else if constexpr (R == 8) dft8<S>(v);
+  else if constexpr (R == 16) dft16<S, HALF>(v);
+  else dft32<S, HALF>(v);
+}
+
+// ---- the plan of one size ----
+
+template <int LOGM> struct Plan {
+  static constexpr int M = 1 << LOGM;
+  static constexpr int R1 = LOGM == 13 ? 32 : 16;   // points per thread = radix of the first pass
+  static constexpr int S1 = M / R1;                 // its stride = threads per CTA
+  static constexpr int S2 = S1 / 16;                // stride of the second pass (radix 16)
+  static constexpr int R3 = S2;                     // radix of the third pass (stride 1)
+  static constexpr int T = S1, E = R1;
+  static constexpr int C2 = E / 16;                 // second-pass columns per thread
+  static constexpr int KP = 16 / S2;                // third-pass columns per thread and column of the second
+  static constexpr int kSmem = M + M / 16;          // elements, padded by one in sixteen
+  static_assert(S2 >= 2 && S2 <= 16, "the exchange of passes 2 and 3 stays within a warp");
+};
+__device__ __forceinline__ int pad(int i) { return i + (i >> 4); }
+
+template <int LOGM> __device__ __forceinline__ void cta_sync() {
+  if constexpr (Plan<LOGM>::T <= 32) __syncwarp();
+  else __syncthreads();
+}
+
+// Tables of one size in global memory: tw1[(k1 - 1) S1 + t] = e^{-2 pi i t k1 / M}, k1 = 1..R1-1;
+// tw2[(k2 - 1) S2 + j] = e^{-2 pi i j k2 / S1}, k2 = 1..15.
+
+// v[j] = x[t + j S1] -> the spectrum in this thread's registers (digit-reversed order)
+template <int LOGM, bool HALF, class V>
+__device__ __forceinline__ void fft_fwd(V* v, V* sm, const V* __restrict__ tw1, const V* __restrict__ tw2) {
+  using P = Plan<LOGM>;
+  const int t = threadIdx.x;
+  dft<P::R1, -1, HALF>(v);
+  sm[pad(t)] = v[0];
+#pragma unroll
+  for (int k = 1; k < P::R1; ++k) sm[pad(k * P::S1 + t)] = mul(v[k], __ldg(tw1 + (k - 1) * P::S1 + t));
+  cta_sync<LOGM>();
+  const int g = t / P::S2, n3 = t % P::S2;
+#pragma unroll
+  for (int c = 0; c < P::C2; ++c) {
+    V* u = v + 16 * c;
+    const int b = (g + 16 * c) * P::S1 + n3;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) u[j] = sm[pad(b + j * P::S2)];
+    dft<16, -1>(u);
+    sm[pad(b)] = u[0];
+#pragma unroll
+    for (int k = 1; k < 16; ++k) sm[pad(b + k * P::S2)] = mul(u[k], __ldg(tw2 + (k - 1) * P::S2 + n3));
+  }
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < P::C2; ++c)
+#pragma unroll
+    for (int e = 0; e < P::KP; ++e) {
+      V* u = v + (c * P::KP + e) * P::R3;
+      const int b = (g + 16 * c) * P::S1 + (n3 * P::KP + e) * P::S2;
+#pragma unroll
+      for (int j = 0; j < P::R3; ++j) u[j] = sm[pad(b + j)];
+      dft<P::R3, -1>(u);
+    }
+}
+
+// the spectrum as fft_fwd leaves it -> v[j] = x[t + j S1] (unscaled inverse); the caller's next
+// fft_fwd may follow without a barrier (its first writes go to the places this thread read last)
+template <int LOGM, class V>
+__device__ __forceinline__ void fft_inv(V* v, V* sm, const V* __restrict__ tw1, const V* __restrict__ tw2) {
+  using P = Plan<LOGM>;
+  const int t = threadIdx.x;
+  const int g = t / P::S2, n3 = t % P::S2;
+#pragma unroll
+  for (int c = 0; c < P::C2; ++c)
+#pragma unroll
+    for (int e = 0; e < P::KP; ++e) {
+      V* u = v + (c * P::KP + e) * P::R3;
+      const int b = (g + 16 * c) * P::S1 + (n3 * P::KP + e) * P::S2;
+      dft<P::R3, 1>(u);
+#pragma unroll
+      for (int j = 0; j < P::R3; ++j) sm[pad(b + j)] = u[j];
+    }
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < P::C2; ++c) {
+    V* u = v + 16 * c;
+    const int b = (g + 16 * c) * P::S1 + n3;
+    u[0] = sm[pad(b)];
+#pragma unroll
+    for (int k = 1; k < 16; ++k) u[k] = mulc(sm[pad(b + k * P::S2)], __ldg(tw2 + (k - 1) * P::S2 + n3));
+    dft<16, 1>(u);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) sm[pad(b + j * P::S2)] = u[j];
+  }
+  cta_sync<LOGM>();
+  v[0] = sm[pad(t)];
+#pragma unroll
+  for (int k = 1; k < P::R1; ++k) v[k] = mulc(sm[pad(k * P::S1 + t)], __ldg(tw1 + (k - 1) * P::S1 + t));
+  dft<P::R1, 1>(v);
+}
+
+// x -> x * h (cyclic), filt[e T + t] = spectrum of h over M in the order of fft_fwd's registers
+template <int LOGM, bool HALF, class V>
+__device__ __forceinline__ void convolve(V* v, V* sm, const V* __restrict__ tw1,
+                                         const V* __restrict__ tw2, const V* __restrict__ filt) {
+  using P = Plan<LOGM>;
+  fft_fwd<LOGM, HALF>(v, sm, tw1, tw2);
+#pragma unroll
+  for (int e = 0; e < P::E; ++e) v[e] = mul(v[e], __ldg(filt + e * P::T + threadIdx.x));
+  fft_inv<LOGM>(v, sm, tw1, tw2);
+}
+
+// ---- kernels ----
+
+template <class T> struct ChirpArgs {
+  const V2<T>* tw1;
+  const V2<T>* tw2;
+  const V2<T>* filt;     // spectrum of h over M
+  const V2<T>* a;        // [n_in] a_{n0 + m} (forward)
+  const V2<T>* b;        // [N_k] b_q
+  const V2<T>* g;        // Gamma table [n_cls][N_ell][n_h]
+  const int* cls_of;
+  const T* kw;           // FP64: stencil weights [tracer stride lw_ts][N_k][4]; FP32: kpow mu [N_tr][4][N_k]
+  long lw_ts;
+  const double* kpow;    // FP64: [N_tr][N_k]
+  const int* off;        // ragged lists (null: multipoles l_lo .. l_lo + n_l - 1)
+  const int* idx;
+  int N_tr, NI, n_h, N_k, N_ell, l_lo, n_l, r, n0, n_chunk;
+};
+
+// FP64: kpow lw; FP32: the product is tabulated
+__device__ __forceinline__ double k_weight(const ChirpArgs<double>& A, int i, int s, int q) {
+  return A.kpow[(size_t)i * A.N_k + q] * A.kw[(size_t)i * A.lw_ts + (size_t)q * 4 + s];
+}
+__device__ __forceinline__ float k_weight(const ChirpArgs<float>& A, int i, int s, int q) {
+  return __ldg(A.kw + ((size_t)i * 4 + s) * A.N_k + q);
+}
+__device__ __forceinline__ double2 coef_at(const cplx* p) { return make_double2(p->x, p->y); }
+__device__ __forceinline__ float2 coef_at(const float4* p) {
+  return *reinterpret_cast<const float2*>(p);   // the high parts of a double-float pair
+}
+
+// the multipoles of walker w that this chunk of a row works on: positions [u0, u1) of its list
+__device__ __forceinline__ void chunk_range(int n, int n_chunk, int chunk, int& u0, int& u1) {
+  u0 = (int)((long)n * chunk / n_chunk);
+  u1 = (int)((long)n * (chunk + 1) / n_chunk);
+}
+
+template <class T, int LOGM> constexpr int min_blocks() {
+  constexpr int per_sm = sizeof(T) == 8 ? 256 : 512;   // resident threads the registers are cut for
+  return per_sm / Plan<LOGM>::T > 0 ? per_sm / Plan<LOGM>::T : 1;
+}
+
+// Delta[w][l - l_lo][i][q] (+)= sum_s kw_is[q] Re sum_{n >= n0} F_wisn G[l][n] e^{-i eta_n ln k_q}
+// FP64 (n0 = 1): the term n = 0, whose phase is 1, is added and Delta is written; FP32 (n0 > 0):
+// the terms below n0 are in Delta already.  CT: cplx (FP64) or float4 (double-float pairs, FP32).
+template <int LOGM, class T, class CT, bool HALF>
+__global__ void __launch_bounds__(Plan<LOGM>::T, min_blocks<T, LOGM>())
+k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) {
+  using P = Plan<LOGM>;
+  using V = V2<T>;
+  constexpr bool kDc = sizeof(T) == 8;
+  constexpr int NI = HALF ? P::E / 2 : P::E;     // inputs and outputs of a thread
+  extern __shared__ __align__(16) unsigned char chirp_sm[];
+  V* sm = reinterpret_cast<V*>(chirp_sm);
+  const int t = threadIdx.x;
+  const int chunk = blockIdx.x % A.n_chunk, wi = blockIdx.x / A.n_chunk;
+  const int i = wi % A.N_tr, w = wi / A.N_tr;
+  const int lo = A.off ? A.off[w] : 0;
+  int u0, u1;
+  chunk_range(A.off ? A.off[w + 1] - lo : A.n_l, A.n_chunk, chunk, u0, u1);
+  const V* G0 = A.g + (size_t)A.cls_of[i] * A.N_ell * A.n_h;
+  const int n_in = A.n_h - A.n0;
+  for (int s = 0; s < A.r; ++s) {
+    const CT* F = coef + ((size_t)wi * A.NI + s) * A.n_h;
+    V f[HALF ? NI : 1], cs[HALF ? NI : 1];
+    T km[kDc && HALF ? NI : 1];
+    if constexpr (HALF) {
+#pragma unroll
+      for (int e = 0; e < NI; ++e) {
+        const int m = t + e * P::S1;
+        f[e] = m < n_in ? mul(coef_at(F + A.n0 + m), A.a[m]) : mk<T>(0, 0);
+        const T k = m < A.N_k ? k_weight(A, i, s, m) : T(0);
+        const V b = m < A.N_k ? A.b[m] : mk<T>(0, 0);
+        cs[e] = mk<T>(k * b.x, k * b.y);
+        if constexpr (kDc) km[e] = k;
+      }
+    }
+    for (int u = u0; u < u1; ++u) {
+      const int l = A.off ? A.idx[lo + u] : A.l_lo + u;
+      const V* G = G0 + (size_t)l * A.n_h + A.n0;
+      V v[P::E];
+#pragma unroll
+      for (int e = 0; e < NI; ++e) {
+        const int m = t + e * P::S1;
+        if constexpr (HALF) {
+          v[e] = m < n_in ? mul(f[e], __ldg(G + m)) : mk<T>(0, 0);
+        } else {
+          v[e] = m < n_in ? mul(mul(coef_at(F + A.n0 + m), A.a[m]), __ldg(G + m)) : mk<T>(0, 0);
+        }
+      }
+#pragma unroll
+      for (int e = NI; e < P::E; ++e) v[e] = mk<T>(0, 0);
+      T dc = 0;
+      if constexpr (kDc) {
+        const V f0 = coef_at(F), g0 = __ldg(G - 1);
+        dc = fma(f0.x, g0.x, -f0.y * g0.y);
+      }
+      convolve<LOGM, HALF>(v, sm, A.tw1, A.tw2, A.filt);
+      T* out = delta + (((size_t)w * A.n_l + (l - A.l_lo)) * A.N_tr + i) * A.N_k;
+#pragma unroll
+      for (int e = 0; e < NI; ++e) {
+        const int q = t + e * P::S1;
+        if (q < A.N_k) {
+          T x;
+          if constexpr (HALF) {
+            x = fma(v[e].x, cs[e].x, -v[e].y * cs[e].y);
+            if constexpr (kDc) x = fma(km[e], dc, x);
+          } else {
+            const V b = A.b[q];
+            x = fma(v[e].x, b.x, -v[e].y * b.y);
+            if constexpr (kDc) x += dc;
+            x *= k_weight(A, i, s, q);
+          }
+          if (kDc && s == 0) out[q] = x;
+          else out[q] += x;
+        }
+      }
+    }
+  }
+}
+
+// The transpose: part[chunk][(w, i, s)][n] = sum over the chunk's multipoles of
+// G[l][n] sum_q [kw_is[q] Dbar q b_q] h_{n - q}; the FP32 form carries the rounding error of the
+// sum over multipoles in a second float (TwoSum).  n0 = 0 here.
+template <int LOGM, class T, bool HALF>
+__global__ void __launch_bounds__(Plan<LOGM>::T, min_blocks<T, LOGM>())
+k_chirp_adj(V2<T>* __restrict__ part, const T* __restrict__ dbar, ChirpArgs<T> A) {
+  using P = Plan<LOGM>;
+  using V = V2<T>;
+  constexpr bool kComp = sizeof(T) == 4;
+  constexpr int NI = HALF ? P::E / 2 : P::E;         // inputs of a thread
+  constexpr int NO = HALF ? P::E / 2 + 1 : P::E;     // outputs (n_h <= M/2 + 1)
+  extern __shared__ __align__(16) unsigned char chirp_sm[];
+  V* sm = reinterpret_cast<V*>(chirp_sm);
+  const int t = threadIdx.x;
+  const int chunk = blockIdx.x % A.n_chunk, wi = blockIdx.x / A.n_chunk;
+  const int i = wi % A.N_tr, w = wi / A.N_tr;
+  const int lo = A.off ? A.off[w] : 0;
+  int u0, u1;
+  chunk_range(A.off ? A.off[w + 1] - lo : A.n_l, A.n_chunk, chunk, u0, u1);
+  const V* G0 = A.g + (size_t)A.cls_of[i] * A.N_ell * A.n_h;
+  const size_t rows = (size_t)(gridDim.x / A.n_chunk) * A.r;
+  for (int s = 0; s < A.r; ++s) {
+    V cs[HALF ? NI : 1];
+    if constexpr (HALF) {
+#pragma unroll
+      for (int e = 0; e < NI; ++e) {
+        const int q = t + e * P::S1;
+        const T k = q < A.N_k ? k_weight(A, i, s, q) : T(0);
+        const V b = q < A.N_k ? A.b[q] : mk<T>(0, 0);
+        cs[e] = mk<T>(k * b.x, k * b.y);
+      }
+    }
+    V acc[NO], cmp[kComp ? NO : 1];
+#pragma unroll
+    for (int e = 0; e < NO; ++e) {
+      acc[e] = mk<T>(0, 0);
+      if constexpr (kComp) cmp[e] = mk<T>(0, 0);
+    }
+    for (int u = u0; u < u1; ++u) {
+      const int l = A.off ? A.idx[lo + u] : A.l_lo + u;
+      const T* d = dbar + (((size_t)w * A.n_l + (l - A.l_lo)) * A.N_tr + i) * A.N_k;
+      V v[P::E];
+#pragma unroll
+      for (int e = 0; e < NI; ++e) {
+        const int q = t + e * P::S1;
+        const T x = q < A.N_k ? d[q] : T(0);
+        if constexpr (HALF) {
+          v[e] = mk<T>(x * cs[e].x, x * cs[e].y);
+        } else {
+          const V b = q < A.N_k ? A.b[q] : mk<T>(0, 0);
+          const T k = q < A.N_k ? x * k_weight(A, i, s, q) : T(0);
+          v[e] = mk<T>(k * b.x, k * b.y);
+        }
+      }
+#pragma unroll
+      for (int e = NI; e < P::E; ++e) v[e] = mk<T>(0, 0);
+      convolve<LOGM, HALF>(v, sm, A.tw1, A.tw2, A.filt);
+      const V* G = G0 + (size_t)l * A.n_h;
+#pragma unroll
+      for (int e = 0; e < NO; ++e) {
+        const int n = t + e * P::S1;
+        if (n < A.n_h) {
+          const V g = __ldg(G + n);
+          if constexpr (kComp) {
+            const V x = mul(v[e], g);
+            const T sx = acc[e].x + x.x, bx = sx - acc[e].x;
+            cmp[e].x += (acc[e].x - (sx - bx)) + (x.x - bx);
+            acc[e].x = sx;
+            const T sy = acc[e].y + x.y, by = sy - acc[e].y;
+            cmp[e].y += (acc[e].y - (sy - by)) + (x.y - by);
+            acc[e].y = sy;
+          } else {
+            acc[e].x = fma(v[e].x, g.x, fma(-v[e].y, g.y, acc[e].x));
+            acc[e].y = fma(v[e].x, g.y, fma(v[e].y, g.x, acc[e].y));
+          }
+        }
+      }
+    }
+    V* out = part + ((size_t)chunk * rows + (size_t)wi * A.r + s) * A.n_h;
+#pragma unroll
+    for (int e = 0; e < NO; ++e) {
+      const int n = t + e * P::S1;
+      if (n < A.n_h) {
+        V x = acc[e];
+        if constexpr (kComp) { x.x += cmp[e].x; x.y += cmp[e].y; }
+        out[n] = x;
+      }
+    }
+  }
+}
+
+// cbar[(w, i, s)][n] (+)= conj(a_n sum_chunk part[chunk][(w, i, s)][n]) in FP64; rows s >= r
+// (padding of the profile rows) are zeros.  Grid: rows x (n_h / 32); thread (n, group) adds the
+// chunks group, group + 8, ... in order, then the eight groups are added in order, so that a row's
+// hundred or so chunks are not one serial chain of loads.
+constexpr int kSumN = 32, kSumG = 8;
+template <class T>
+__global__ void __launch_bounds__(kSumN * kSumG)
+k_chirp_sum(cplx* __restrict__ cbar, const V2<T>* __restrict__ part, const double2* __restrict__ a,
+            int n_rows, int NI, int r, int n_h, int n_chunk, bool accumulate) {
+  __shared__ double2 red[kSumG][kSumN];
+  const int nb = (n_h + kSumN - 1) / kSumN;
+  const int nl = threadIdx.x % kSumN, grp = threadIdx.x / kSumN;
+  const int n = (blockIdx.x % nb) * kSumN + nl;
+  const int row = blockIdx.x / nb, wi = row / NI, s = row % NI;
+  double x = 0.0, y = 0.0;
+  if (n < n_h && s < r) {
+    const size_t per = (size_t)n_rows * r * n_h;
+    const V2<T>* p = part + ((size_t)wi * r + s) * n_h + n;
+#pragma unroll 4
+    for (int c = grp; c < n_chunk; c += kSumG) {
+      const V2<T> v = p[(size_t)c * per];
+      x += (double)v.x;
+      y += (double)v.y;
+    }
+  }
+  red[grp][nl] = make_double2(x, y);
+  __syncthreads();
+  if (grp || n >= n_h) return;
+#pragma unroll
+  for (int g = 1; g < kSumG; ++g) {
+    x += red[g][nl].x;
+    y += red[g][nl].y;
+  }
+  cplx* out = cbar + (size_t)row * n_h + n;
+  if (s >= r) {
+    if (!accumulate) *out = {0.0, 0.0};
+    return;
+  }
+  const double2 f = a[n];
+  cplx o = {fma(x, f.x, -y * f.y), -fma(x, f.y, y * f.x)};
+  if (accumulate) { o.x += out->x; o.y += out->y; }
+  *out = o;
+}
+
+// ---- tables ----
+
+// e^{2 pi i S f}, f = frac(n (ch + cl)) with the product's rounding error kept
+__device__ __forceinline__ double dd_cycles(double n, double ch, double cl) {
+  const double p = n * ch;
+  return (p - rint(p)) + fma(n, ch, -p) + n * cl;
+}
+__device__ __forceinline__ double2 unit(double cycles) {
+  double s, c;
+  sincospi(2.0 * cycles, &s, &c);
+  return make_double2(c, s);
+}
+template <class T> __device__ __forceinline__ V2<T> cast2(double2 v) { return mk<T>((T)v.x, (T)v.y); }
+
+// tw1, tw2 of the plan, a_{n0 + m} (m < n_in, type TA) and b_q (q < N_k).  cc = d/(2 L) and
+// xx = x0/L in double-double: beta m^2/2 = 2 pi cc m^2 and eta_n x0 = 2 pi n xx.
+template <int LOGM, class T, class TA>
+__global__ void k_chirp_tables(V2<T>* __restrict__ tw1, V2<T>* __restrict__ tw2, V2<TA>* __restrict__ a,
+                               V2<T>* __restrict__ b, int n0, int n_in, int N_k, double2 cc, double2 xx) {
+  using P = Plan<LOGM>;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < (P::R1 - 1) * P::S1) {
+    const long k1 = e / P::S1 + 1, t = e % P::S1;
+    tw1[e] = cast2<T>(unit(-(double)((k1 * t) & (P::M - 1)) / P::M));
+  }
+  if (e < 15 * P::S2) {
+    const int k2 = e / P::S2 + 1, j = e % P::S2;
+    tw2[e] = cast2<T>(unit(-(double)((k2 * j) & (P::S1 - 1)) / P::S1));
+  }
+  if (e < n_in) {
+    const double m = e, n = n0 + e;
+    a[e] = cast2<TA>(unit(-(dd_cycles(n, xx.x, xx.y) + dd_cycles(m * m, cc.x, cc.y))));
+  }
+  if (e < N_k) {
+    const double q = e;
+    b[e] = cast2<T>(unit(-dd_cycles(q * q + 2.0 * n0 * q, cc.x, cc.y)));
+  }
+}
+
+// spectrum of h_t/M, t = -t_lo .. t_hi (t_lo + t_hi < M, the rest zero), in FP64, one CTA
+template <int LOGM, class T>
+__global__ void __launch_bounds__(Plan<LOGM>::T)
+k_chirp_filter(V2<T>* __restrict__ filt, int t_lo, int t_hi, double2 cc, const double2* __restrict__ tw1,
+               const double2* __restrict__ tw2) {
+  using P = Plan<LOGM>;
+  extern __shared__ __align__(16) unsigned char chirp_sm[];
+  double2 v[P::E];
+#pragma unroll
+  for (int e = 0; e < P::E; ++e) {
+    const int p = threadIdx.x + e * P::S1;
+    const int x = p <= t_hi ? p : p - P::M;
+    v[e] = make_double2(0.0, 0.0);
+    if (x >= -t_lo) {
+      v[e] = unit(dd_cycles((double)x * x, cc.x, cc.y));
+      v[e].x *= 1.0 / P::M;
+      v[e].y *= 1.0 / P::M;
+    }
+  }
+  fft_fwd<LOGM, false>(v, reinterpret_cast<double2*>(chirp_sm), tw1, tw2);
+#pragma unroll
+  for (int e = 0; e < P::E; ++e) filt[e * P::T + threadIdx.x] = cast2<T>(v[e]);
+}
+
+// ---- host side of one precision (instantiated in chirp_f64.cu and chirp_f32.cu) ----
+
+template <class T> size_t smem_bytes(int logm) { return sizeof(V2<T>) * (((size_t)1 << logm) + ((size_t)1 << logm) / 16); }
+
+template <class F> cudaError_t with_smem(F kern, size_t smem) {
+  return smem > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                          : cudaSuccess;
+}
+
+// Elements of a direction's tables: tw1 and tw2 (FP64 ones first, for the filter), filt, b, a
+struct TabLayout {
+  size_t tw1d, tw2d, tw1, tw2, filt, b, a, bytes;
+};
+template <class T> TabLayout tab_layout(int logm, int n_in, int N_k, size_t a_elem) {
+  const size_t M = (size_t)1 << logm, R1 = logm == 13 ? 32 : 16, S1 = M / R1, S2 = S1 / 16;
+  TabLayout L;
+  size_t o = 0;
+  auto put = [&](size_t bytes) { const size_t at = o; o += (bytes + 255) & ~size_t(255); return at; };
+  L.tw1d = put(16 * (R1 - 1) * S1);
+  L.tw2d = put(16 * 15 * S2);
+  L.tw1 = sizeof(T) == 8 ? L.tw1d : put(8 * (R1 - 1) * S1);
+  L.tw2 = sizeof(T) == 8 ? L.tw2d : put(8 * 15 * S2);
+  L.filt = put(sizeof(V2<T>) * M);
+  L.b = put(sizeof(V2<T>) * N_k);
+  L.a = put(a_elem * n_in);
+  L.bytes = o;
+  return L;
+}
+
+template <int LOGM, class T, class TA>
+cudaError_t build_tables(uint8_t* p, const TabLayout& L, int n0, int n_in, int N_k, int t_lo, int t_hi,
+                         double2 cc, double2 xx, cudaStream_t s) {
+  using P = Plan<LOGM>;
+  const int n = std::max({(P::R1 - 1) * P::S1, 15 * P::S2, n_in, N_k});
+  const unsigned grid = (unsigned)((n + 255) / 256);
+  double2 *tw1d = (double2*)(p + L.tw1d), *tw2d = (double2*)(p + L.tw2d);
+  k_chirp_tables<LOGM, T, TA><<<grid, 256, 0, s>>>((V2<T>*)(p + L.tw1), (V2<T>*)(p + L.tw2), (V2<TA>*)(p + L.a),
+                                                   (V2<T>*)(p + L.b), n0, n_in, N_k, cc, xx);
+  if (sizeof(T) == 4)
+    k_chirp_tables<LOGM, double, double><<<grid, 256, 0, s>>>(tw1d, tw2d, nullptr, nullptr, 0, 0, 0, cc, xx);
+  const size_t smem = smem_bytes<double>(LOGM);
+  cudaError_t e = with_smem(k_chirp_filter<LOGM, T>, smem);
+  if (e != cudaSuccess) return e;
+  k_chirp_filter<LOGM, T><<<1, P::T, smem, s>>>((V2<T>*)(p + L.filt), t_lo, t_hi, cc, tw1d, tw2d);
+  return cudaGetLastError();
+}
+
+template <class T, class F> cudaError_t by_size(int logm, F f) {
+  switch (logm) {
+    case 9: return f(std::integral_constant<int, 9>());
+    case 10: return f(std::integral_constant<int, 10>());
+    case 11: return f(std::integral_constant<int, 11>());
+    case 12: return f(std::integral_constant<int, 12>());
+    case 13: return f(std::integral_constant<int, 13>());
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <class T, class CT>
+cudaError_t launch_fwd(int logm, bool half, T* delta, const CT* coef, const ChirpArgs<T>& A, int n_rows,
+                       cudaStream_t s) {
+  return by_size<T>(logm, [&](auto lm) {
+    constexpr int LM = decltype(lm)::value;
+    auto kern = half ? k_chirp_fwd<LM, T, CT, true> : k_chirp_fwd<LM, T, CT, false>;
+    const size_t smem = smem_bytes<T>(LM);
+    cudaError_t e = with_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((long)n_rows * A.n_chunk), Plan<LM>::T, smem, s>>>(delta, coef, A);
+    return cudaGetLastError();
+  });
+}
+template <class T>
+cudaError_t launch_adj(int logm, bool half, V2<T>* part, const T* dbar, const ChirpArgs<T>& A, int n_rows,
+                       cudaStream_t s) {
+  return by_size<T>(logm, [&](auto lm) {
+    constexpr int LM = decltype(lm)::value;
+    auto kern = half ? k_chirp_adj<LM, T, true> : k_chirp_adj<LM, T, false>;
+    const size_t smem = smem_bytes<T>(LM);
+    cudaError_t e = with_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((long)n_rows * A.n_chunk), Plan<LM>::T, smem, s>>>(part, dbar, A);
+    return cudaGetLastError();
+  });
+}
+
+}  // namespace chirp
+}  // namespace swcl

@@ -115,6 +115,21 @@ struct LimberTable {
   double* lnnu = nullptr;
 };
 
+// Chirp transforms of the contraction (chirp.cuh): one direction's size and tables
+struct ChirpDir {
+  bool ready = false;
+  int logm = 0;         // FFT points M = 2^logm
+  bool half = false;    // frequencies and k points both fit M/2
+  int n0 = 0;           // first frequency of the transform
+  DevBuf tab;
+};
+// one launch: shapes, multipoles, transforms per row, CTAs per row, ragged lists (null: all)
+struct ChirpRun {
+  int n_walk, N_tr, NI, n_h, N_k, N_ell, l_lo, n_l, rank, n_chunk;
+  const int* off;
+  const int* idx;
+};
+
 }  // namespace swcl
 
 struct swcl_ctx {
@@ -170,6 +185,14 @@ struct swcl_ctx {
   int lr_rank = 0;            // stencil rows used in basis mode
   int lr_true_rank = 0;
   swcl::DevBuf lr_res, lr_norms, lr_Q, lr_coef, lr_w, lr_j0, lr_ones;
+
+  // chirp transforms (chirp.cu): set by the grids
+  bool ck_uniform = false;     // ln k_q = x0 + q d
+  bool ck_off = false;         // given up (memory budget)
+  double ck_c[2] = {0, 0};     // d/(2 L) in double-double
+  double ck_x[2] = {0, 0};     // x0/L
+  swcl::ChirpDir ck[1][2];     // [FP64][forward, adjoint]
+  swcl::DevBuf ws_ckpart;      // adjoint: partial sums over the multipoles
 
   // basis-mode tensor-core GEMMs (basis_tc.cu)
   bool bt_ready = false;       // constant operands built for the current grids/tracers/profiles
@@ -355,6 +378,25 @@ cudaError_t launch_contract_fp64_adj(cplx* cbar, const double* dbar, const cplx*
                                      const int* j0, const double* lw, long lw_ts, int n_walk,
                                      int N_tr, int N_I, int n_h, int N_k, int N_ell, int l_lo,
                                      int n_l, bool accumulate, cudaStream_t s);
+
+// a3 as chirp transforms on k grids uniform in ln k (chirp.cu, chirp_f64.cu)
+void chirp_fit_grid(swcl_ctx* c);
+bool chirp_use(const swcl_ctx* c, int precision);
+int chirp_rank(const swcl_ctx* c);
+int chirp_prepare(swcl_ctx* c, int precision);      // tables; gives the transforms up on a full budget
+void chirp_drop(swcl_ctx* c);
+size_t chirp_part_bytes(const swcl_ctx* c, int precision, int n_l, bool whole);
+int chirp_forward(swcl_ctx* c, int precision, int l_lo, int n_l);
+int chirp_adjoint(swcl_ctx* c, int precision, int l_lo, int n_l, bool accumulate);
+size_t chirp64_table_bytes(int logm, int n_in, int N_k);
+cudaError_t chirp64_build(void* tab, int logm, int n0, int n_in, int N_k, int t_lo, int t_hi, const double* cc,
+                          const double* xx, cudaStream_t s);
+cudaError_t chirp64_forward(const ChirpDir& d, double* delta, const cplx* coef, const cplx* g, const int* cls_of,
+                            const double* w, long w_ts, const double* kpow, const ChirpRun& r, cudaStream_t s);
+cudaError_t chirp64_adjoint(const ChirpDir& d, void* part, const double* dbar, const cplx* g, const int* cls_of,
+                            const double* w, long w_ts, const double* kpow, const ChirpRun& r, cudaStream_t s);
+cudaError_t chirp64_sum(cplx* cbar, const void* part, const ChirpDir& d, const ChirpRun& r, bool accumulate,
+                        cudaStream_t s);
 
 // a4 k-quadrature and VJP reductions (quad.cu).  Delta and Dbar buffers hold the multipoles
 // l_lo .. l_lo + n_l - 1 ([n_walk][n_l][N_tr][N_k]); U and Cbar_full all N_ell.
