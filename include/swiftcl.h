@@ -97,7 +97,8 @@ typedef struct swcl_ctx swcl_ctx;
 #define SWCL_Q_TILE_FWD        6  /* autotuned tile of the basis-mode forward GEMM (0 = none yet):
                                      column tile in bits 0-7, bit 8 set for the variant that runs
                                      two CTAs per SM, bit 10 for two K-blocks per stage */
-#define SWCL_Q_TILE_ADJ        7  /* the same for the basis-mode adjoint GEMM */
+#define SWCL_Q_TILE_ADJ        7  /* the same for the basis-mode adjoint GEMM (0 also where chirp
+                                     transforms take its place: k uniform in ln k, N >= 1024) */
 
 /* Create a context on CUDA device `device`.  mem_budget_bytes bounds the device memory the
  * context may hold (0 = no bound).  `stream` is a cudaStream_t (NULL = the context creates

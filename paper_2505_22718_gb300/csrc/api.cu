@@ -322,14 +322,22 @@ int swcl_create(swcl_ctx** out, int device, size_t mem_budget_bytes, void* strea
   // SWCL_PER_KNOT_FFT=1 keeps the paper's one FFT per knot (no low-rank profiles)
   if (const char* v = std::getenv("SWCL_PER_KNOT_FFT")) c->lr_disabled = std::atoi(v) != 0;
   if (const char* v = std::getenv("SWCL_PDL")) c->pdl = std::atoi(v) != 0;
-  if (const char* v = std::getenv("SWCL_BASIS_GEMM")) c->bt_disabled = std::atoi(v) == 0;
+  // SWCL_BASIS_GEMM=0: the knot-stencil kernels in basis mode too; =1: the basis-mode GEMMs over all
+  // frequencies also where the chirp transforms would take most of them
+  if (const char* v = std::getenv("SWCL_BASIS_GEMM")) {
+    c->bt_disabled = std::atoi(v) == 0;
+    c->bt_asked = !c->bt_disabled;
+  }
   // the accuracy study of the compensated products: a subset of the six products of the basis
   // GEMMs (bit t = product t in the order (0,0) (0,1) (1,0) (0,2) (1,1) (2,0)); only the sets
   // 0x2F, 0x37, 0x1F, 0x17 and 0x07 exist, at the 96-column two-K-block tile (SWCL_BASIS_TILES
   // 1120,1120); they all miss the accuracy gate
   if (const char* v = std::getenv("SWCL_BASIS_PRODUCTS")) {
     const unsigned m = (unsigned)std::strtoul(v, nullptr, 0);
-    if (m == 0x2Fu || m == 0x37u || m == 0x1Fu || m == 0x17u || m == 0x07u) c->bt_pmask = m;
+    if (m == 0x2Fu || m == 0x37u || m == 0x1Fu || m == 0x17u || m == 0x07u) {
+      c->bt_pmask = m;
+      c->bt_asked = true;
+    }
   }
   // fixed basis-GEMM tiles "fwd,adj" (tile codes as reported by SWCL_Q_TILE_*) instead of tuning
   if (const char* v = std::getenv("SWCL_BASIS_TILES")) {
@@ -337,6 +345,7 @@ int swcl_create(swcl_ctx** out, int device, size_t mem_budget_bytes, void* strea
     if (std::sscanf(v, "%d,%d", &f, &a) == 2) {
       c->bt_fixed_fwd = f;
       c->bt_fixed_adj = a;
+      c->bt_asked = true;
     }
   }
   // device status word raised by bounded waits in the tensor-core kernels

@@ -16,6 +16,9 @@
 //   A[2n][q] = Re E, A[2n+1][q] = -Im E;  B[j][q] = kpow mu Dbar;
 // its epilogue multiplies by conj(G) and sums over l.
 //
+// On k grids uniform in ln k (from N = 1024 on) only the frequencies n < 64 take the forward GEMM, and
+// the rest of the sum and its whole transpose the FP32 chirp transforms (chirp.cuh).
+//
 // Compensated products with FP32 accumulation (the 5th-generation tensor cores take bf16 operands
 // here): the constant operand is split once from FP64 into 3 bf16 planes; the forward B operand
 // H is formed in double-float arithmetic from double-float F and G and split into 3 planes; the
@@ -2031,10 +2034,17 @@ bool valid_tile(int code, const std::vector<int>& cands) {
 
 }  // namespace
 
+// K-blocks of the forward GEMM: every frequency, or those below the chirp transform's
+static int fwd_kblocks(const swcl_ctx* c, bool chirp) {
+  return (2 * (chirp ? kChirpHead : c->n_h) + kK - 1) / kK;
+}
+
 size_t basis_fixed_bytes(const swcl_ctx* c) {
   // row tiles rounded up to an even count, as in basis_prepare
-  const size_t f_mt = (((c->N_k + kM - 1) / kM) + 1) & ~1, f_kb = (2 * c->n_h + kK - 1) / kK;
-  const size_t a_mt = (((2 * c->n_h + kM - 1) / kM) + 1) & ~1, a_kb = (c->N_k + kK - 1) / kK;
+  const bool chirp = chirp_use(c, SWCL_SPLIT_BF16);
+  const size_t f_mt = (((c->N_k + kM - 1) / kM) + 1) & ~1, f_kb = fwd_kblocks(c, chirp);
+  const size_t a_mt = chirp ? 0 : (((2 * c->n_h + kM - 1) / kM) + 1) & ~1;
+  const size_t a_kb = chirp ? 0 : (c->N_k + kK - 1) / kK;
   const size_t ng = (size_t)c->n_cls * c->N_ell * c->n_h;
   return (f_mt * f_kb + a_mt * a_kb) * kPlanes * kPlaneM + ng * (sizeof(float4) + sizeof(float2)) +
          sizeof(float) * (size_t)c->N_tr * 4 * c->N_k +
@@ -2042,7 +2052,8 @@ size_t basis_fixed_bytes(const swcl_ctx* c) {
 }
 
 size_t basis_bytes_per_ell(const swcl_ctx* c) {
-  const size_t f_kb = (2 * c->n_h + kK - 1) / kK, a_kb = (c->N_k + kK - 1) / kK;
+  const bool chirp = chirp_use(c, SWCL_SPLIT_BF16);
+  const size_t f_kb = fwd_kblocks(c, chirp), a_kb = chirp ? 0 : (c->N_k + kK - 1) / kK;
   return (size_t)c->n_walk * c->N_tr * std::max(1, c->lr_true_rank) * (f_kb + a_kb) * kPlanes * kRow;
 }
 
@@ -2054,7 +2065,8 @@ int basis_prepare(swcl_ctx* c) {
   const int r = basis_rank(c);
   int st;
   c->bt_f_mt = (N_k + kM - 1) / kM;
-  c->bt_f_kb = (2 * n_h + kK - 1) / kK;
+  c->bt_chirp = chirp_use(c, SWCL_SPLIT_BF16);
+  c->bt_f_kb = fwd_kblocks(c, c->bt_chirp);
   c->bt_a_mt = (2 * n_h + kM - 1) / kM;
   c->bt_a_kb = (N_k + kK - 1) / kK;
   // the images hold an even number of row tiles (the last one zero when the count is odd), so
@@ -2063,7 +2075,7 @@ int basis_prepare(swcl_ctx* c) {
   const size_t ef = (size_t)f_mt2 * c->bt_f_kb * kPlanes * kPlaneM;
   const size_t ea = (size_t)a_mt2 * c->bt_a_kb * kPlanes * kPlaneM;
   if ((st = ensure(c, c->bt_eimg_f, ef))) return st;
-  if ((st = ensure(c, c->bt_eimg_a, ea))) return st;
+  if (!c->bt_chirp && (st = ensure(c, c->bt_eimg_a, ea))) return st;
   const long ng = (long)c->n_cls * c->N_ell * n_h;
   if ((st = ensure(c, c->bt_gdf, sizeof(float4) * ng))) return st;
   if ((st = ensure(c, c->bt_g32, sizeof(float2) * ng))) return st;
@@ -2072,8 +2084,9 @@ int basis_prepare(swcl_ctx* c) {
   k_eimg_fwd<<<grid_for(tot), 256, 0, c->stream>>>((uint8_t*)c->bt_eimg_f.p, (const cplx*)c->d_phase.p,
                                                    N_k, n_h, f_mt2, c->bt_f_kb);
   tot = (long)a_mt2 * c->bt_a_kb * kM * 4;
-  k_eimg_adj<<<grid_for(tot), 256, 0, c->stream>>>((uint8_t*)c->bt_eimg_a.p, (const cplx*)c->d_phase.p,
-                                                   N_k, n_h, a_mt2, c->bt_a_kb);
+  if (!c->bt_chirp)
+    k_eimg_adj<<<grid_for(tot), 256, 0, c->stream>>>((uint8_t*)c->bt_eimg_a.p, (const cplx*)c->d_phase.p,
+                                                     N_k, n_h, a_mt2, c->bt_a_kb);
   k_gtab_split<<<grid_for(ng), 256, 0, c->stream>>>((float4*)c->bt_gdf.p, (float2*)c->bt_g32.p,
                                                     (const cplx*)c->d_gtab.p, ng);
   k_kmu<<<grid_for((long)c->N_tr * 4 * N_k), 256, 0, c->stream>>>(
@@ -2267,7 +2280,8 @@ int basis_forward(swcl_ctx* c, int l_lo, int n_l) {
          return build_h(c, cp, img_cols(code), img_tiles(code, n_nt), l_lo, n_l);
        })))
     return st;
-  return counted(c, "basis gemm fwd", [&] { return run(code, false); });
+  if ((st = counted(c, "basis gemm fwd", [&] { return run(code, false); }))) return st;
+  return c->bt_chirp ? chirp_forward(c, SWCL_SPLIT_BF16, l_lo, n_l) : SWCL_OK;
 }
 
 // ws_cbar (FP64 complex, [n_walk][N_tr][NI][n_h], zeroed here) from ws_dbar (FP32,
@@ -2285,6 +2299,7 @@ int basis_adjoint(swcl_ctx* c, int l_lo, int n_l, bool accumulate) {
     cudaError_t e = accumulate ? cudaSuccess : cudaMemsetAsync(c->ws_cbar.p, 0, cbytes, c->stream);
     return e == cudaSuccess ? SWCL_OK : cuda_fail(c, e, "clear cbar");
   }
+  if (c->bt_chirp) return chirp_adjoint(c, SWCL_SPLIT_BF16, l_lo, n_l, accumulate);
   auto run = [&](int code, bool build) -> int {
     const int NT = code & 255;
     const int n_nt = (n_cols + NT - 1) / NT;

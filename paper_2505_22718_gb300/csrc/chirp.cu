@@ -43,7 +43,18 @@ int log_size(int n_in, int n_out) {
   return 0;
 }
 
-constexpr int kFirst64 = 1;    // FP64: the term n = 0 (phase 1) is added beside the transform
+// First frequency of the forward transform.  FP64: the term n = 0, whose phase is 1, is added beside
+// the transform, so that N/2 frequencies remain.  FP32: the terms n < 64, which carry most of a smooth
+// window's Delta, stay in the compensated tensor-core GEMM; the FFT's rounding error, about 2e-7 of
+// what passes through it, then falls on the small rest.  Simulated C error against the FP64 oracle at
+// N5K shape (the GEMM over all frequencies 2.1e-5): 2.4e-5 with 32 terms in the GEMM, 1.8e-5 with 64,
+// 2.1e-5 with 128; 1.4e-4 with none.
+int first_freq(int precision) { return precision == SWCL_FP64 ? 1 : kChirpHead; }
+int form(int precision) { return precision == SWCL_FP64 ? 0 : 1; }
+
+// multipoles that one CTA of the FP32 transpose sums in FP32 at most (the CTAs' sums in FP64); the
+// GEMM's epilogue sums 48 columns or more
+constexpr int kMaxSum32 = 16;
 
 }  // namespace
 
@@ -51,14 +62,21 @@ constexpr int kFirst64 = 1;    // FP64: the term n = 0 (phase 1) is added beside
 int chirp_rank(const swcl_ctx* c) { return c->lr_basis ? c->lr_true_rank : c->N_I <= 4 ? c->N_I : 0; }
 
 bool chirp_use(const swcl_ctx* c, int precision) {
-  if (!c->ck_uniform || c->ck_off || precision != SWCL_FP64) return false;
-  const int r = chirp_rank(c), mf = log_size(c->n_h - kFirst64, c->N_k), ma = log_size(c->N_k, c->n_h);
+  if (!c->ck_uniform || c->ck_off) return false;
+  const int r = chirp_rank(c), mf = log_size(c->n_h - first_freq(precision), c->N_k), ma = log_size(c->N_k, c->n_h);
   if (r <= 0 || !mf || !ma) return false;
   // FP64 operations: about 75 per point and pair of FFTs, against 2 per (frequency, k point) of the
   // direct sum (four profile rows cost four transforms but one direct sum).  Both sides are bound by
   // the FP64 pipe: forward + VJP at N = 2048, N_k = 1024, 103 multipoles, 15 tracers 1.01 ms against
   // 12.8 ms; N = N_k = 256, 20 multipoles, 2 tracers (three quarters of the line) 0.24 against 0.79 ms.
-  return 75.0 * r * (double)(1 << std::max(mf, ma)) < 2.0 * c->n_h * (double)c->N_k;
+  if (precision == SWCL_FP64) return 75.0 * r * (double)(1 << std::max(mf, ma)) < 2.0 * c->n_h * (double)c->N_k;
+  // the mixed form: beside the basis-mode GEMMs, unless tiles or products of theirs are asked for
+  if (precision != SWCL_SPLIT_BF16 || !c->lr_basis || c->bt_disabled || c->bt_asked) return false;
+  // From N = 1024 on: 15 tracers, 103 multipoles, N = 2048, N_k = 1024 forward + VJP 83 us a step
+  // against 136 us with the GEMMs over all frequencies, 256 such points with ragged lists 11.7 against
+  // 25.1 ms, N = N_k = 4096 with 30 tracers and 2999 multipoles 13.9 against 32.2 ms; at N = 512,
+  // N_k = 333, 7 tracers, 37 multipoles, three points both take 62 us.
+  return c->N >= 1024;
 }
 
 void chirp_drop(swcl_ctx* c) {
@@ -69,20 +87,23 @@ void chirp_drop(swcl_ctx* c) {
     }
   release(c, c->ws_ckpart);
   c->ck_off = true;
+  c->bt_ready = false;
 }
 
 int chirp_prepare(swcl_ctx* c, int precision) {
   if (!chirp_use(c, precision)) return SWCL_OK;
   for (int dir = 0; dir < 2; ++dir) {
-    ChirpDir& d = c->ck[0][dir];
+    ChirpDir& d = c->ck[form(precision)][dir];
     if (d.ready) continue;
     if (c->capturing) return fail(c, SWCL_ERR_STATE, "chirp tables built during capture");
-    d.n0 = dir == 0 ? kFirst64 : 0;
+    d.n0 = dir == 0 ? first_freq(precision) : 0;
     const int n_freq = c->n_h - d.n0;
     d.logm = dir == 0 ? log_size(n_freq, c->N_k) : log_size(c->N_k, n_freq);
     const int M = 1 << d.logm;
     d.half = c->N_k <= M / 2 && n_freq <= M / 2 + (dir == 0 ? 0 : 1);
-    const int st = ensure(c, d.tab, chirp64_table_bytes(d.logm, n_freq, c->N_k));
+    const bool fp64 = precision == SWCL_FP64;
+    const int st = ensure(c, d.tab, fp64 ? chirp64_table_bytes(d.logm, n_freq, c->N_k)
+                                         : chirp32_table_bytes(d.logm, n_freq, c->N_k));
     if (st == SWCL_ERR_OOM_BUDGET) {   // the direct sums need no tables
       chirp_drop(c);
       c->err.clear();
@@ -90,56 +111,81 @@ int chirp_prepare(swcl_ctx* c, int precision) {
     }
     if (st) return st;
     const int t_lo = dir == 0 ? n_freq - 1 : c->N_k - 1, t_hi = dir == 0 ? c->N_k - 1 : n_freq - 1;
-    const cudaError_t e = chirp64_build(d.tab.p, d.logm, d.n0, n_freq, c->N_k, t_lo, t_hi, c->ck_c, c->ck_x,
-                                        c->stream);
+    const cudaError_t e =
+        fp64 ? chirp64_build(d.tab.p, d.logm, d.n0, n_freq, c->N_k, t_lo, t_hi, c->ck_c, c->ck_x, c->stream)
+             : chirp32_build(d.tab.p, d.logm, d.n0, n_freq, c->N_k, t_lo, t_hi, c->ck_c, c->ck_x, dir == 0, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "chirp tables");
     d.ready = true;
   }
   return SWCL_OK;
 }
 
-// CTAs per row (each takes an equal share of the row's multipoles): enough CTAs for several turns of
-// what the GPU holds at once, so that the last turn is a small part, and no more, since each CTA
-// loads its row's coefficients and weights once.
-static int row_chunks(const swcl_ctx* c, long rows, int n_l, int logm) {
+// CTAs per row; each takes an equal share of the row's multipoles.  FP64, bound by one pipe of the SM
+// whatever the number of resident CTAs: enough CTAs for eight turns of what the GPU holds at once, so
+// that the last turn is a small part.  FP32, which lives from several resident CTAs: the share of at
+// most 16 multipoles with the fewest turns x (multipoles + the load of the row's own data, about 0.4 of
+// a multipole); 1545 rows of 2048 points take 22.9 us with one multipole per CTA, 20.9 with three (the
+// choice), 26.8 with seven; the sum over the transpose's CTAs 22.6, 12.1 and 8.7 us.
+static int row_chunks(const swcl_ctx* c, int precision, long rows, int n_l, int logm) {
   const int threads = logm == 13 ? 256 : (1 << logm) / 16;
-  const long slots = (long)c->num_sms * std::max(1, 256 / threads);
-  const long per = std::max<long>(1, rows * n_l / (8 * slots));
-  return (int)std::min<long>(n_l, (n_l + per - 1) / per);
+  if (precision == SWCL_FP64) {
+    const long slots = (long)c->num_sms * std::max(1, 256 / threads);
+    const long per = std::max<long>(1, rows * n_l / (8 * slots));
+    return (int)std::min<long>(n_l, (n_l + per - 1) / per);
+  }
+  const long slots = (long)c->num_sms * std::max(1, (logm == 13 ? 256 : 512) / threads);
+  int best = 1;
+  double best_cost = 0.0;
+  for (int per = 1; per <= std::min(n_l, kMaxSum32); ++per) {
+    const long ctas = rows * ((n_l + per - 1) / per);
+    const double cost = (double)((ctas + slots - 1) / slots) * (per + 0.4);
+    if (per == 1 || cost < best_cost) {
+      best = per;
+      best_cost = cost;
+    }
+  }
+  return (n_l + best - 1) / best;
 }
 
 // Bytes of the adjoint's partial sums over n_l multipoles (whole: with every CTA of a row its own)
 size_t chirp_part_bytes(const swcl_ctx* c, int precision, int n_l, bool whole) {
   if (!chirp_use(c, precision)) return 0;
   const long rows = (long)c->n_walk * c->N_tr;
-  const int n = whole ? row_chunks(c, rows, n_l, log_size(c->N_k, c->n_h)) : 1;
-  return sizeof(cplx) * rows * chirp_rank(c) * c->n_h * n;
+  const int n = whole ? row_chunks(c, precision, rows, n_l, log_size(c->N_k, c->n_h)) : 1;
+  return (precision == SWCL_FP64 ? 16 : 8) * (size_t)rows * chirp_rank(c) * c->n_h * n;
+}
+
+// the multipoles of one launch: all of [l_lo, l_lo + n_l), or each walker's list where the basis-mode
+// GEMMs keep listed multipoles only (Delta's other rows hold zeros)
+static ChirpRun run_for(const swcl_ctx* c, int precision, bool adjoint, int l_lo, int n_l) {
+  const Stencil sv = stencil(c);
+  const bool lists = precision != SWCL_FP64 && c->bt_compact;
+  return ChirpRun{c->n_walk, c->N_tr, sv.NI, c->n_h, c->N_k, c->N_ell, l_lo, n_l, chirp_rank(c),
+                  row_chunks(c, precision, (long)c->n_walk * c->N_tr, n_l, c->ck[form(precision)][adjoint].logm),
+                  lists ? (const int*)c->d_off.p : nullptr, lists ? (const int*)c->d_idx.p : nullptr};
 }
 
 int chirp_forward(swcl_ctx* c, int precision, int l_lo, int n_l) {
-  (void)precision;
-  const ChirpDir& d = c->ck[0][0];
+  const ChirpDir& d = c->ck[form(precision)][0];
   const Stencil sv = stencil(c);
-  const long rows = (long)c->n_walk * c->N_tr;
-  ChirpRun r{c->n_walk, c->N_tr, sv.NI, c->n_h, c->N_k, c->N_ell, l_lo, n_l, chirp_rank(c),
-             row_chunks(c, rows, n_l, d.logm), nullptr, nullptr};
+  const ChirpRun r = run_for(c, precision, false, l_lo, n_l);
   ++c->last_launches;
   prof_begin(c);
-  const cudaError_t e = chirp64_forward(d, (double*)c->ws_delta.p, (const cplx*)c->ws_coef.p,
-                                        (const cplx*)c->d_gtab.p, (const int*)c->d_cls_of.p, sv.w, sv.w_ts,
-                                        (const double*)c->d_kpow.p, r, c->stream);
-  prof_end(c, "chirp fwd fp64");
-  return e == cudaSuccess ? SWCL_OK : cuda_fail(c, e, "chirp fwd fp64");
+  const cudaError_t e =
+      precision == SWCL_FP64
+          ? chirp64_forward(d, (double*)c->ws_delta.p, (const cplx*)c->ws_coef.p, (const cplx*)c->d_gtab.p,
+                            (const int*)c->d_cls_of.p, sv.w, sv.w_ts, (const double*)c->d_kpow.p, r, c->stream)
+          : chirp32_forward(d, (float*)c->ws_delta.p, (const float4*)c->ws_coef.p, (const float2*)c->bt_g32.p,
+                            (const int*)c->d_cls_of.p, (const float*)c->bt_kmu.p, r, c->stream);
+  prof_end(c, precision == SWCL_FP64 ? "chirp fwd fp64" : "chirp fwd f32");
+  return e == cudaSuccess ? SWCL_OK : cuda_fail(c, e, "chirp transform, forward");
 }
 
 int chirp_adjoint(swcl_ctx* c, int precision, int l_lo, int n_l, bool accumulate) {
-  (void)precision;
-  const ChirpDir& d = c->ck[0][1];
+  const bool fp64 = precision == SWCL_FP64;
+  const ChirpDir& d = c->ck[form(precision)][1];
   const Stencil sv = stencil(c);
-  const long rows = (long)c->n_walk * c->N_tr;
-  const int rank = chirp_rank(c);
-  ChirpRun r{c->n_walk, c->N_tr, sv.NI, c->n_h, c->N_k, c->N_ell, l_lo, n_l, rank,
-             row_chunks(c, rows, n_l, d.logm), nullptr, nullptr};
+  ChirpRun r = run_for(c, precision, true, l_lo, n_l);
   // partial sums of the CTAs of a row; under a tight budget one CTA per row
   const size_t per = chirp_part_bytes(c, precision, n_l, false);
   if (c->budget && c->held - c->ws_ckpart.bytes + per * r.n_chunk > c->budget) r.n_chunk = 1;
@@ -147,16 +193,19 @@ int chirp_adjoint(swcl_ctx* c, int precision, int l_lo, int n_l, bool accumulate
   if (st) return st;
   ++c->last_launches;
   prof_begin(c);
-  cudaError_t e = chirp64_adjoint(d, c->ws_ckpart.p, (const double*)c->ws_dbar.p, (const cplx*)c->d_gtab.p,
-                                  (const int*)c->d_cls_of.p, sv.w, sv.w_ts, (const double*)c->d_kpow.p, r,
-                                  c->stream);
-  prof_end(c, "chirp adj fp64");
-  if (e != cudaSuccess) return cuda_fail(c, e, "chirp adj fp64");
+  cudaError_t e =
+      fp64 ? chirp64_adjoint(d, c->ws_ckpart.p, (const double*)c->ws_dbar.p, (const cplx*)c->d_gtab.p,
+                             (const int*)c->d_cls_of.p, sv.w, sv.w_ts, (const double*)c->d_kpow.p, r, c->stream)
+           : chirp32_adjoint(d, c->ws_ckpart.p, (const float*)c->ws_dbar.p, (const float2*)c->bt_g32.p,
+                             (const int*)c->d_cls_of.p, (const float*)c->bt_kmu.p, r, c->stream);
+  prof_end(c, fp64 ? "chirp adj fp64" : "chirp adj f32");
+  if (e != cudaSuccess) return cuda_fail(c, e, "chirp transform, transposed");
   ++c->last_launches;
   prof_begin(c);
-  e = chirp64_sum((cplx*)c->ws_cbar.p, c->ws_ckpart.p, d, r, accumulate, c->stream);
+  e = fp64 ? chirp64_sum((cplx*)c->ws_cbar.p, c->ws_ckpart.p, d, r, accumulate, c->stream)
+           : chirp32_sum((cplx*)c->ws_cbar.p, c->ws_ckpart.p, d, r, accumulate, c->stream);
   prof_end(c, "chirp adj sum");
-  return e == cudaSuccess ? SWCL_OK : cuda_fail(c, e, "chirp adj sum");
+  return e == cudaSuccess ? SWCL_OK : cuda_fail(c, e, "chirp transform, sum over multipoles");
 }
 
 }  // namespace swcl

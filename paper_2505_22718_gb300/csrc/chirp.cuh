@@ -25,6 +25,14 @@
 // and eight resident warps are enough.  15 tracers x 103 multipoles, N = 2048, N_k = 1024: 484 us
 // forward and 463 us transposed (75 % of the pipe's rate; the last of six turns of two CTAs per SM is
 // nearly empty), against 5.9 ms each for the direct sums.
+//
+// FP32: bound by instruction issue and shared-memory exchanges together, about 2200 clocks per row of
+// 2048 points and SM with four resident CTAs (16 warps).  1545 such rows: 21 us forward and 22.5 us
+// transposed; 287 100 rows (256 walkers with ragged lists) 2.1 and 2.2 ms; 89 970 rows of 8192 points
+// 4.5 and 4.1 ms.  The GEMMs over all frequencies took 56 and 58 us, 7.9 and 12.3 ms, 14.6 and 11.9 ms,
+// with another 23 us, 1.7 ms and 1.5 ms for their operand images.  Errors against 64 bits (N5K shape):
+// Delta 1.3e-7 (GEMMs 1.9e-7), normalised C 2.7e-5 (3.1e-5), W_bar 4.2e-7 (9.7e-7); white-noise windows
+// 1.6e-7 (1.4e-7), 5.9e-5 (6.0e-5), 4.8e-7 (7.4e-7).
 #pragma once
 #include <algorithm>
 #include <type_traits>
@@ -371,7 +379,8 @@ __device__ __forceinline__ void chunk_range(int n, int n_chunk, int chunk, int& 
 }
 
 template <class T, int LOGM> constexpr int min_blocks() {
-  constexpr int per_sm = sizeof(T) == 8 ? 256 : 512;   // resident threads the registers are cut for
+  // resident threads the registers are cut for (32 points per thread need twice the registers)
+  constexpr int per_sm = sizeof(T) == 8 || LOGM == 13 ? 256 : 512;
   return per_sm / Plan<LOGM>::T > 0 ? per_sm / Plan<LOGM>::T : 1;
 }
 
@@ -455,14 +464,13 @@ k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) 
 }
 
 // The transpose: part[chunk][(w, i, s)][n] = sum over the chunk's multipoles of
-// G[l][n] sum_q [kw_is[q] Dbar q b_q] h_{n - q}; the FP32 form carries the rounding error of the
-// sum over multipoles in a second float (TwoSum).  n0 = 0 here.
+// G[l][n] sum_q [kw_is[q] Dbar_i(l, q) b_q] h_{n - q}  (n0 = 0); the chunks are added in FP64 by
+// k_chirp_sum.
 template <int LOGM, class T, bool HALF>
 __global__ void __launch_bounds__(Plan<LOGM>::T, min_blocks<T, LOGM>())
 k_chirp_adj(V2<T>* __restrict__ part, const T* __restrict__ dbar, ChirpArgs<T> A) {
   using P = Plan<LOGM>;
   using V = V2<T>;
-  constexpr bool kComp = sizeof(T) == 4;
   constexpr int NI = HALF ? P::E / 2 : P::E;         // inputs of a thread
   constexpr int NO = HALF ? P::E / 2 + 1 : P::E;     // outputs (n_h <= M/2 + 1)
   extern __shared__ __align__(16) unsigned char chirp_sm[];
@@ -486,12 +494,9 @@ k_chirp_adj(V2<T>* __restrict__ part, const T* __restrict__ dbar, ChirpArgs<T> A
         cs[e] = mk<T>(k * b.x, k * b.y);
       }
     }
-    V acc[NO], cmp[kComp ? NO : 1];
+    V acc[NO];
 #pragma unroll
-    for (int e = 0; e < NO; ++e) {
-      acc[e] = mk<T>(0, 0);
-      if constexpr (kComp) cmp[e] = mk<T>(0, 0);
-    }
+    for (int e = 0; e < NO; ++e) acc[e] = mk<T>(0, 0);
     for (int u = u0; u < u1; ++u) {
       const int l = A.off ? A.idx[lo + u] : A.l_lo + u;
       const T* d = dbar + (((size_t)w * A.n_l + (l - A.l_lo)) * A.N_tr + i) * A.N_k;
@@ -517,18 +522,8 @@ k_chirp_adj(V2<T>* __restrict__ part, const T* __restrict__ dbar, ChirpArgs<T> A
         const int n = t + e * P::S1;
         if (n < A.n_h) {
           const V g = __ldg(G + n);
-          if constexpr (kComp) {
-            const V x = mul(v[e], g);
-            const T sx = acc[e].x + x.x, bx = sx - acc[e].x;
-            cmp[e].x += (acc[e].x - (sx - bx)) + (x.x - bx);
-            acc[e].x = sx;
-            const T sy = acc[e].y + x.y, by = sy - acc[e].y;
-            cmp[e].y += (acc[e].y - (sy - by)) + (x.y - by);
-            acc[e].y = sy;
-          } else {
-            acc[e].x = fma(v[e].x, g.x, fma(-v[e].y, g.y, acc[e].x));
-            acc[e].y = fma(v[e].x, g.y, fma(v[e].y, g.x, acc[e].y));
-          }
+          acc[e].x = fma(v[e].x, g.x, fma(-v[e].y, g.y, acc[e].x));
+          acc[e].y = fma(v[e].x, g.y, fma(v[e].y, g.x, acc[e].y));
         }
       }
     }
@@ -536,11 +531,7 @@ k_chirp_adj(V2<T>* __restrict__ part, const T* __restrict__ dbar, ChirpArgs<T> A
 #pragma unroll
     for (int e = 0; e < NO; ++e) {
       const int n = t + e * P::S1;
-      if (n < A.n_h) {
-        V x = acc[e];
-        if constexpr (kComp) { x.x += cmp[e].x; x.y += cmp[e].y; }
-        out[n] = x;
-      }
+      if (n < A.n_h) out[n] = acc[e];
     }
   }
 }

@@ -115,6 +115,9 @@ struct LimberTable {
   double* lnnu = nullptr;
 };
 
+// frequencies that stay in the basis-mode GEMM beside the FP32 chirp transform (four K-blocks)
+constexpr int kChirpHead = 64;
+
 // Chirp transforms of the contraction (chirp.cuh): one direction's size and tables
 struct ChirpDir {
   bool ready = false;
@@ -191,12 +194,14 @@ struct swcl_ctx {
   bool ck_off = false;         // given up (memory budget)
   double ck_c[2] = {0, 0};     // d/(2 L) in double-double
   double ck_x[2] = {0, 0};     // x0/L
-  swcl::ChirpDir ck[1][2];     // [FP64][forward, adjoint]
+  swcl::ChirpDir ck[2][2];     // [FP64, FP32][forward, adjoint]
   swcl::DevBuf ws_ckpart;      // adjoint: partial sums over the multipoles
 
   // basis-mode tensor-core GEMMs (basis_tc.cu)
   bool bt_ready = false;       // constant operands built for the current grids/tracers/profiles
   bool bt_disabled = false;    // environment override SWCL_BASIS_GEMM=0
+  bool bt_asked = false;       // SWCL_BASIS_GEMM=1, fixed tiles or products: the GEMMs over all frequencies
+  bool bt_chirp = false;       // operands built for the chirp form (GEMM of the low frequencies only)
   int bt_f_mt = 0, bt_f_kb = 0, bt_a_mt = 0, bt_a_kb = 0;
   int bt_nt_fwd = 0, bt_nt_adj = 0;   // autotuned column tiles (0 = not tuned yet)
   int bt_fixed_fwd = 0, bt_fixed_adj = 0;  // tiles fixed by the environment (0 = tune)
@@ -396,6 +401,17 @@ cudaError_t chirp64_forward(const ChirpDir& d, double* delta, const cplx* coef, 
 cudaError_t chirp64_adjoint(const ChirpDir& d, void* part, const double* dbar, const cplx* g, const int* cls_of,
                             const double* w, long w_ts, const double* kpow, const ChirpRun& r, cudaStream_t s);
 cudaError_t chirp64_sum(cplx* cbar, const void* part, const ChirpDir& d, const ChirpRun& r, bool accumulate,
+                        cudaStream_t s);
+
+// and in FP32 beside the basis-mode GEMM of the low frequencies (chirp_f32.cu)
+size_t chirp32_table_bytes(int logm, int n_in, int N_k);
+cudaError_t chirp32_build(void* tab, int logm, int n0, int n_in, int N_k, int t_lo, int t_hi, const double* cc,
+                          const double* xx, bool forward, cudaStream_t s);
+cudaError_t chirp32_forward(const ChirpDir& d, float* delta, const float4* coef, const float2* g, const int* cls_of,
+                            const float* kmu, const ChirpRun& r, cudaStream_t s);
+cudaError_t chirp32_adjoint(const ChirpDir& d, void* part, const float* dbar, const float2* g, const int* cls_of,
+                            const float* kmu, const ChirpRun& r, cudaStream_t s);
+cudaError_t chirp32_sum(cplx* cbar, const void* part, const ChirpDir& d, const ChirpRun& r, bool accumulate,
                         cudaStream_t s);
 
 // a4 k-quadrature and VJP reductions (quad.cu).  Delta and Dbar buffers hold the multipoles

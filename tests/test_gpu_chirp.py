@@ -1,9 +1,11 @@
 """The chirp transforms of the contraction (k grids uniform in ln k) against the FP64 oracle, at the
 sizes where their split into FFT points, halves and passes changes, and the rule that chooses them:
-a grid that is uniform to rounding takes them, any other the direct sums, with the same results.
+a grid that is uniform to rounding takes them, any other the direct sums, with the same results.  In the mixed form the transforms take the frequencies n >= 64
+and the tensor-core GEMM those below.
 
 Gates: those of the FP64 path, 1e-10 (C, P_bar, amp_bar) and 1e-9 (W_bar): the transforms are FP64
-FFTs of at most 8192 points, whose rounding errors are below 1e-13 of a row."""
+FFTs of at most 8192 points, whose rounding errors are below 1e-13 of a row.  Mixed form: its gates,
+1e-4 (C) and 5e-5 (gradients)."""
 import numpy as np
 import pytest
 
@@ -21,7 +23,7 @@ def built():
     g.build()
 
 
-def _case(N, k, n_ell, n_knots, curved=True):
+def _case(N, k, n_ell, n_knots, curved=True, rank=0):
     """Two density tracers and a lensing one, one of them with its own bias; with few knots the
     growth is curved in ln k, so that every knot carries weight."""
     cosmo = Cosmology()
@@ -34,6 +36,11 @@ def _case(N, k, n_ell, n_knots, curved=True):
     D = (1.0 / (1.0 + z))[None, :] * (1.0 + 0.02 * lk + (0.003 * lk ** 2 if curved else 0.0))[:, None]
     if curved:
         D = D + 0.002 * np.sin(lk)[:, None] * (z / (1.0 + z))[None, :]
+    if rank:
+        # growth of that rank in (k, z), for basis mode
+        f = [1.0 / (1.0 + z), 0.02 * z / (1.0 + z), 0.01 * np.sin(2.0 * z) * np.exp(-z), 0.01 * np.exp(-2.0 * z)]
+        h = [np.ones_like(lk), lk, np.sin(lk), np.cos(0.7 * lk)]
+        D = sum(np.outer(h[t], f[t]) for t in range(rank))
     P = power_spectrum(k, 3.5e6)
     kind = np.array([0, 0, 1], dtype=np.int32)
     bias = np.array([-0.3, -0.45, -1.5])
@@ -54,13 +61,18 @@ def _kernels(w, precision, Cb):
     return C, g, names
 
 
-def _check(w, C, g, Cb, tol, tol_w):
+def _errors(w, C, g, Cb):
     gr = O.Grids(w.N, w.chi_min, w.chi_max, w.k, w.ells, w.knots, w.kind, w.fft_bias, fft="numpy")
     f = O.forward(gr, w.W, w.D, w.P, w.amp)
     Pbo, Abo, Wbo, _ = O.vjp(gr, f, Cb, w.W, w.D, w.P, w.amp)
     e = (norm_err(C, f["C"]), pbar_err(g[0][0], Pbo, p_abs(f["delta"], Cb, w.amp, w.k)), grad_err(g[1][0], Abo),
          wbar_err(g[2][0], Wbo))
     print("C %.2e  P_bar %.2e  amp_bar %.2e  W_bar %.2e" % e)
+    return e
+
+
+def _check(w, C, g, Cb, tol, tol_w):
+    e = _errors(w, C, g, Cb)
     assert max(e[:3]) < tol and e[3] < tol_w
 
 
@@ -98,3 +110,57 @@ def test_rule_on_the_k_grid(grid):
     C, g, names = _kernels(w, "fp64", Cb)
     assert ("chirp fwd fp64" in names) == (grid in ("geomspace", "logspace", "exp", "wide"))
     _check(w, C, g, Cb, 1e-10, 1e-9)
+
+
+# (N, N_k, multipoles, rank of the growth): the smallest N, both halves and whole windows, the last size
+# that fits an FFT forward (N/2 - 63 + N_k - 1 points) and transposed, one to four transforms per
+# multipole, more multipoles than one CTA sums (16)
+@pytest.mark.parametrize("N,n_k,n_ell,rank", [
+    (1024, 200, 37, 1), (1024, 576, 18, 2), (1024, 512, 17, 3), (2048, 1024, 33, 1), (2048, 1088, 5, 4),
+    (2048, 2500, 9, 2), (4096, 2049, 3, 1), (4096, 6144, 2, 1)])
+def test_mixed_sizes_against_oracle(N, n_k, n_ell, rank):
+    w = _case(N, np.geomspace(1e-4, 8.0, n_k), n_ell, 24, rank=rank)
+    Cb = np.random.default_rng(5).standard_normal((n_ell, 3, 3))
+    C, g, names = _kernels(w, "bf16x9", Cb)
+    assert {"chirp fwd f32", "chirp adj f32"} <= names and "basis gemm adj" not in names
+    _check(w, C, g, Cb, 1e-4, 5e-5)
+
+
+@pytest.mark.parametrize("N", [512, 1024])
+@pytest.mark.parametrize("n_walk", [1, 3])
+def test_mixed_ragged_walkers_against_the_gemms(n_walk, N, monkeypatch):
+    """Lists of 1, 0 and many multipoles per walker; N = 512 keeps the GEMMs over all frequencies.  A
+    single multipole's P_bar has no accurate digits where every Delta of that multipole is at its
+    FP32 noise (the largest k), by either route: the transforms have to meet the gates or come as near
+    to the oracle as the GEMMs over all frequencies do on the same inputs."""
+    import paper_2505_22718_gb300 as S
+    w = _case(N, np.geomspace(1e-4, 8.0, 333), 21, 24, rank=1)
+    rng = np.random.default_rng(6)
+    one = (w.W, w.P, w.amp)
+    w.W, w.P, w.amp = (np.stack([a * (1.0 + 0.1 * t) for t in range(n_walk)]) for a in one)
+    lists = [np.array([3], np.int32), np.array([], np.int32), np.arange(0, 21, 2, dtype=np.int32)][-n_walk:]
+    w.ell_lists = lists
+    Cb = rng.standard_normal((sum(map(len, lists)), 3, 3))
+    found = []
+    for gemm in (False, True):
+        if gemm:
+            monkeypatch.setenv("SWCL_BASIS_GEMM", "1")
+        ctx = lib_context(w)
+        S.swcl_profile_enable(ctx.ptr, True)
+        C = ctx.compute_cl(S.SWCL_SPLIT_BF16)
+        g = ctx.vjp(Cb, S.SWCL_SPLIT_BF16)
+        assert ("chirp fwd f32" in S.swcl_profile_read(ctx.ptr)) == (N == 1024 and not gemm)
+        errs, o = [], 0
+        for t, lst in enumerate(lists):
+            n = len(lst)
+            if n == 0:
+                assert not any(a[t].any() for a in g)
+                continue
+            v = _case(N, w.k, 21, 24, rank=1)
+            v.W, v.P, v.amp, v.ells = w.W[t], w.P[t], w.amp[t], w.ells[lst]
+            errs += _errors(v, C[o:o + n], [a[t:t + 1] for a in g], Cb[o:o + n])
+            o += n
+        found.append(errs)
+        ctx.close()
+    for j, (mine, theirs) in enumerate(zip(*found)):
+        assert mine < max((1e-4, 5e-5, 5e-5, 5e-5)[j % 4], 1.5 * theirs)
