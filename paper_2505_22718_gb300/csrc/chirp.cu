@@ -127,13 +127,12 @@ int chirp_prepare(swcl_ctx* c, int precision) {
 // a multipole); 1545 rows of 2048 points take 22.9 us with one multipole per CTA, 20.9 with three (the
 // choice), 26.8 with seven; the sum over the transpose's CTAs 22.6, 12.1 and 8.7 us.
 static int row_chunks(const swcl_ctx* c, int precision, long rows, int n_l, int logm) {
-  const int threads = logm == 13 ? 256 : (1 << logm) / 16;
   if (precision == SWCL_FP64) {
-    const long slots = (long)c->num_sms * std::max(1, 256 / threads);
+    const long slots = (long)c->num_sms * chirp64_ctas_per_sm(logm);
     const long per = std::max<long>(1, rows * n_l / (8 * slots));
     return (int)std::min<long>(n_l, (n_l + per - 1) / per);
   }
-  const long slots = (long)c->num_sms * std::max(1, (logm == 13 ? 256 : 512) / threads);
+  const long slots = (long)c->num_sms * chirp32_ctas_per_sm(logm);
   int best = 1;
   double best_cost = 0.0;
   for (int per = 1; per <= std::min(n_l, kMaxSum32); ++per) {

@@ -11,12 +11,12 @@
 //   sum_q d_q e^{-i eta_n ln k_q} = a_n sum_q [d_q b_q] h_{n - q}                  (n0 = 0),
 // multiplied by G[l][n] and summed over the multipoles before the factor a_n.
 //
-// One CTA of M/16 threads (16 points each; 32 for M = 8192) runs one row at a time: a forward FFT
-// of passes 16 x 16 x M/256 with the frequencies left in digit-reversed order, the product with the
+// One CTA of M/E threads (E = 16 or 32 points each) runs one row at a time: a forward FFT of passes
+// E x E x M/E^2 with the frequencies left in digit-reversed order, the product with the
 // filter's spectrum (stored in that order), and the inverse passes in reverse.  Each pass works in
 // registers; passes exchange through shared memory in place (a thread writes back the places it has
 // read), so the second and third pass, which stay within 16 neighbouring threads, need a warp
-// barrier only and a row needs two CTA barriers.  The window of the frequencies and of the k points
+// barrier only (or shuffles) and a row needs two CTA barriers.  The window of the frequencies and of the k points
 // is at most M/2 in the HALF form: half of the first pass's inputs are then zero and half of the
 // last pass's outputs unused.
 //
@@ -26,13 +26,14 @@
 // forward and 463 us transposed (75 % of the pipe's rate; the last of six turns of two CTAs per SM is
 // nearly empty), against 5.9 ms each for the direct sums.
 //
-// FP32: bound by instruction issue and shared-memory exchanges together, about 2200 clocks per row of
-// 2048 points and SM with four resident CTAs (16 warps).  1545 such rows: 21 us forward and 22.5 us
-// transposed; 287 100 rows (256 walkers with ragged lists) 2.1 and 2.2 ms; 89 970 rows of 8192 points
-// 4.5 and 4.1 ms.  The GEMMs over all frequencies took 56 and 58 us, 7.9 and 12.3 ms, 14.6 and 11.9 ms,
-// with another 23 us, 1.7 ms and 1.5 ms for their operand images.  Errors against 64 bits (N5K shape):
-// Delta 1.3e-7 (GEMMs 1.9e-7), normalised C 2.7e-5 (3.1e-5), W_bar 4.2e-7 (9.7e-7); white-noise windows
-// 1.6e-7 (1.4e-7), 5.9e-5 (6.0e-5), 4.8e-7 (7.4e-7).
+// FP32: bound by shared-memory and table accesses (1750 wavefronts of the load/store pipe per row of
+// 2048 points) and, close behind, by instruction issue: about 2070 clocks per row and SM with four
+// resident CTAs (16 warps).  1545 such rows 19 us forward and 20 us transposed; 287 100 rows (256 walkers
+// with ragged lists) 1.95 and 1.88 ms; 89 970 rows of 8192 points 3.84 and 3.34 ms.  The GEMMs over all
+// frequencies took 56 and 58 us, 7.9 and 12.3 ms, 14.6 and 11.9 ms, with another 23 us, 1.7 ms and
+// 1.5 ms for their operand images.  Errors against 64 bits (N5K shape): Delta 1.3e-7 (GEMMs 1.9e-7),
+// normalised C 2.7e-5 (3.1e-5), W_bar 4.2e-7 (9.7e-7); white-noise windows 1.6e-7 (1.4e-7), 5.9e-5
+// (6.0e-5), 4.8e-7 (7.4e-7).
 #pragma once
 #include <algorithm>
 #include <type_traits>
@@ -50,6 +51,28 @@ template <class T> using V2 = typename Vec2<T>::type;
 template <class T> __device__ __forceinline__ V2<T> mk(T x, T y) { V2<T> v; v.x = x; v.y = y; return v; }
 template <class V> __device__ __forceinline__ V add(V a, V b) { a.x += b.x; a.y += b.y; return a; }
 template <class V> __device__ __forceinline__ V sub(V a, V b) { a.x -= b.x; a.y -= b.y; return a; }
+// FP32: both components in one instruction (the same two roundings); 2.12 -> 1.96 ms forward and 2.22 ->
+// 1.89 ms transposed for 287 100 rows of 2048 points, together with the constant offsets below
+__device__ __forceinline__ unsigned long long pk(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 upk(unsigned long long a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+  return r;
+}
+template <> __device__ __forceinline__ float2 add<float2>(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pk(a)), "l"(pk(b)));
+  return upk(r);
+}
+template <> __device__ __forceinline__ float2 sub<float2>(float2 a, float2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pk(a)), "l"(pk(b)));
+  return upk(r);
+}
 // a b, and a conj(b)
 template <class V> __device__ __forceinline__ V mul(V a, V b) {
   V r;
@@ -68,6 +91,19 @@ template <int S, class V> __device__ __forceinline__ V rot(V a) {
   V r;
   if constexpr (S > 0) { r.x = -a.y; r.y = a.x; } else { r.x = a.y; r.y = -a.x; }
   return r;
+}
+
+// A table value that every row reads again (L1).  volatile keeps the load in the loop over rows: hoisted
+// out of it, the tables would take more registers than the data.
+__device__ __forceinline__ float2 ld_tab(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 ld_tab(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
 }
 
 // ---- DFTs in registers, X_k = sum_n v_n e^{2 pi i S n k / R}, natural order in and out ----
@@ -238,108 +274,102 @@ template <int R, int S, bool HALF = false, class V> __device__ __forceinline__ v
 
 // ---- the plan of one size ----
 
-template <int LOGM> struct Plan {
+// M = E x E x M/E^2 points, E per thread: passes of radix E at strides S1 and S2, then of radix R3 at
+// stride 1.  E = 16, and 32 at M = 8192.  In FP32 E = 32 at M = 2048, with the last pass by shuffles, has
+// a third fewer shared-memory and table accesses, but with 168 registers fewer warps to hide them:
+// 2.3 ms against 2.0 ms for 287 100 rows.
+template <int LOGM, class T> struct Plan {
   static constexpr int M = 1 << LOGM;
-  static constexpr int R1 = LOGM == 13 ? 32 : 16;   // points per thread = radix of the first pass
-  static constexpr int S1 = M / R1;                 // its stride = threads per CTA
-  static constexpr int S2 = S1 / 16;                // stride of the second pass (radix 16)
-  static constexpr int R3 = S2;                     // radix of the third pass (stride 1)
-  static constexpr int T = S1, E = R1;
-  static constexpr int C2 = E / 16;                 // second-pass columns per thread
-  static constexpr int KP = 16 / S2;                // third-pass columns per thread and column of the second
-  static constexpr int kSmem = M + M / 16;          // elements, padded by one in sixteen
-  static_assert(S2 >= 2 && S2 <= 16, "the exchange of passes 2 and 3 stays within a warp");
+  static constexpr int E = LOGM == 13 ? 32 : 16;
+  static constexpr int S1 = M / E, S2 = S1 / E, R3 = S2;
+  static constexpr int kT = S1;                        // threads per CTA
+  static constexpr int KP = E / S2;                    // third-pass columns per thread
+  static constexpr int kSmem = M + M / E;              // elements, padded by one in E
+  static_assert(S2 >= 1 && S2 <= 16, "the exchange of passes 2 and 3 stays within a warp");
 };
-__device__ __forceinline__ int pad(int i) { return i + (i >> 4); }
+// Element i sits at i + i/E.  The three access patterns split into a thread's base and a constant:
+// k S1 + t, g S1 + n3 + j S2 and g S1 + (n3 KP + e) S2 + j (t < S1; n3 < S2, S2 divides E).
+template <class P> __device__ __forceinline__ int base1(int t) { return t + t / P::E; }
+template <class P> __device__ __forceinline__ constexpr int off1(int k) { return k * (P::S1 + P::S1 / P::E); }
+template <class P> __device__ __forceinline__ int base2(int g, int n3) { return g * (P::S1 + P::S1 / P::E) + n3; }
+template <class P> __device__ __forceinline__ constexpr int off2(int j) { return j * P::S2 + j * P::S2 / P::E; }
+template <class P> __device__ __forceinline__ int base3(int g, int n3) {
+  return g * (P::S1 + P::S1 / P::E) + n3 * (P::E + 1);
+}
+template <class P> __device__ __forceinline__ constexpr int off3(int e, int j) { return e * P::S2 + j; }
 
-template <int LOGM> __device__ __forceinline__ void cta_sync() {
-  if constexpr (Plan<LOGM>::T <= 32) __syncwarp();
+template <class P> __device__ __forceinline__ void cta_sync() {
+  if constexpr (P::kT <= 32) __syncwarp();
   else __syncthreads();
 }
 
-// Tables of one size in global memory: tw1[(k1 - 1) S1 + t] = e^{-2 pi i t k1 / M}, k1 = 1..R1-1;
-// tw2[(k2 - 1) S2 + j] = e^{-2 pi i j k2 / S1}, k2 = 1..15.
+// Tables of one size in global memory: tw1[(k1 - 1) S1 + t] = e^{-2 pi i t k1 / M}, k1 = 1..E-1;
+// tw2[(k2 - 1) S2 + j] = e^{-2 pi i j k2 / S1}, k2 = 1..E-1.
 
 // v[j] = x[t + j S1] -> the spectrum in this thread's registers (digit-reversed order)
-template <int LOGM, bool HALF, class V>
+template <class P, bool HALF, class V>
 __device__ __forceinline__ void fft_fwd(V* v, V* sm, const V* __restrict__ tw1, const V* __restrict__ tw2) {
-  using P = Plan<LOGM>;
   const int t = threadIdx.x;
-  dft<P::R1, -1, HALF>(v);
-  sm[pad(t)] = v[0];
+  dft<P::E, -1, HALF>(v);
+  V* s1 = sm + base1<P>(t);
+  s1[0] = v[0];
 #pragma unroll
-  for (int k = 1; k < P::R1; ++k) sm[pad(k * P::S1 + t)] = mul(v[k], __ldg(tw1 + (k - 1) * P::S1 + t));
-  cta_sync<LOGM>();
+  for (int k = 1; k < P::E; ++k) s1[off1<P>(k)] = mul(v[k], ld_tab(tw1 + (k - 1) * P::S1 + t));
+  cta_sync<P>();
   const int g = t / P::S2, n3 = t % P::S2;
+  V *s2 = sm + base2<P>(g, n3), *s3 = sm + base3<P>(g, n3);
 #pragma unroll
-  for (int c = 0; c < P::C2; ++c) {
-    V* u = v + 16 * c;
-    const int b = (g + 16 * c) * P::S1 + n3;
+  for (int j = 0; j < P::E; ++j) v[j] = s2[off2<P>(j)];
+  dft<P::E, -1>(v);
+  s2[0] = v[0];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) u[j] = sm[pad(b + j * P::S2)];
-    dft<16, -1>(u);
-    sm[pad(b)] = u[0];
-#pragma unroll
-    for (int k = 1; k < 16; ++k) sm[pad(b + k * P::S2)] = mul(u[k], __ldg(tw2 + (k - 1) * P::S2 + n3));
-  }
+  for (int k = 1; k < P::E; ++k) s2[off2<P>(k)] = mul(v[k], ld_tab(tw2 + (k - 1) * P::S2 + n3));
   __syncwarp();
 #pragma unroll
-  for (int c = 0; c < P::C2; ++c)
+  for (int e = 0; e < P::KP; ++e) {
+    V* u = v + e * P::R3;
 #pragma unroll
-    for (int e = 0; e < P::KP; ++e) {
-      V* u = v + (c * P::KP + e) * P::R3;
-      const int b = (g + 16 * c) * P::S1 + (n3 * P::KP + e) * P::S2;
-#pragma unroll
-      for (int j = 0; j < P::R3; ++j) u[j] = sm[pad(b + j)];
-      dft<P::R3, -1>(u);
-    }
+    for (int j = 0; j < P::R3; ++j) u[j] = s3[off3<P>(e, j)];
+    dft<P::R3, -1>(u);
+  }
 }
 
 // the spectrum as fft_fwd leaves it -> v[j] = x[t + j S1] (unscaled inverse); the caller's next
 // fft_fwd may follow without a barrier (its first writes go to the places this thread read last)
-template <int LOGM, class V>
+template <class P, class V>
 __device__ __forceinline__ void fft_inv(V* v, V* sm, const V* __restrict__ tw1, const V* __restrict__ tw2) {
-  using P = Plan<LOGM>;
   const int t = threadIdx.x;
   const int g = t / P::S2, n3 = t % P::S2;
+  V *s1 = sm + base1<P>(t), *s2 = sm + base2<P>(g, n3), *s3 = sm + base3<P>(g, n3);
 #pragma unroll
-  for (int c = 0; c < P::C2; ++c)
+  for (int e = 0; e < P::KP; ++e) {
+    V* u = v + e * P::R3;
+    dft<P::R3, 1>(u);
 #pragma unroll
-    for (int e = 0; e < P::KP; ++e) {
-      V* u = v + (c * P::KP + e) * P::R3;
-      const int b = (g + 16 * c) * P::S1 + (n3 * P::KP + e) * P::S2;
-      dft<P::R3, 1>(u);
-#pragma unroll
-      for (int j = 0; j < P::R3; ++j) sm[pad(b + j)] = u[j];
-    }
-  __syncwarp();
-#pragma unroll
-  for (int c = 0; c < P::C2; ++c) {
-    V* u = v + 16 * c;
-    const int b = (g + 16 * c) * P::S1 + n3;
-    u[0] = sm[pad(b)];
-#pragma unroll
-    for (int k = 1; k < 16; ++k) u[k] = mulc(sm[pad(b + k * P::S2)], __ldg(tw2 + (k - 1) * P::S2 + n3));
-    dft<16, 1>(u);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) sm[pad(b + j * P::S2)] = u[j];
+    for (int j = 0; j < P::R3; ++j) s3[off3<P>(e, j)] = u[j];
   }
-  cta_sync<LOGM>();
-  v[0] = sm[pad(t)];
+  __syncwarp();
+  v[0] = s2[0];
 #pragma unroll
-  for (int k = 1; k < P::R1; ++k) v[k] = mulc(sm[pad(k * P::S1 + t)], __ldg(tw1 + (k - 1) * P::S1 + t));
-  dft<P::R1, 1>(v);
+  for (int k = 1; k < P::E; ++k) v[k] = mulc(s2[off2<P>(k)], ld_tab(tw2 + (k - 1) * P::S2 + n3));
+  dft<P::E, 1>(v);
+#pragma unroll
+  for (int j = 0; j < P::E; ++j) s2[off2<P>(j)] = v[j];
+  cta_sync<P>();
+  v[0] = s1[0];
+#pragma unroll
+  for (int k = 1; k < P::E; ++k) v[k] = mulc(s1[off1<P>(k)], ld_tab(tw1 + (k - 1) * P::S1 + t));
+  dft<P::E, 1>(v);
 }
 
 // x -> x * h (cyclic), filt[e T + t] = spectrum of h over M in the order of fft_fwd's registers
-template <int LOGM, bool HALF, class V>
+template <class P, bool HALF, class V>
 __device__ __forceinline__ void convolve(V* v, V* sm, const V* __restrict__ tw1,
                                          const V* __restrict__ tw2, const V* __restrict__ filt) {
-  using P = Plan<LOGM>;
-  fft_fwd<LOGM, HALF>(v, sm, tw1, tw2);
+  fft_fwd<P, HALF>(v, sm, tw1, tw2);
 #pragma unroll
-  for (int e = 0; e < P::E; ++e) v[e] = mul(v[e], __ldg(filt + e * P::T + threadIdx.x));
-  fft_inv<LOGM>(v, sm, tw1, tw2);
+  for (int e = 0; e < P::E; ++e) v[e] = mul(v[e], ld_tab(filt + e * P::kT + threadIdx.x));
+  fft_inv<P>(v, sm, tw1, tw2);
 }
 
 // ---- kernels ----
@@ -378,19 +408,24 @@ __device__ __forceinline__ void chunk_range(int n, int n_chunk, int chunk, int& 
   u1 = (int)((long)n * (chunk + 1) / n_chunk);
 }
 
+// resident threads the registers are cut for: 255 registers in FP64 (one pipe of the SM is the bound)
+// and with 32 points per thread, 128 in FP32 with 16 (at 2048 points and many rows 2.0 ms; 2.1 ms with
+// 102 registers, 2.3 ms with 168)
+template <class T, int LOGM> constexpr int resident_threads() {
+  return sizeof(T) == 8 || Plan<LOGM, T>::E == 32 ? 256 : 512;
+}
 template <class T, int LOGM> constexpr int min_blocks() {
-  // resident threads the registers are cut for (32 points per thread need twice the registers)
-  constexpr int per_sm = sizeof(T) == 8 || LOGM == 13 ? 256 : 512;
-  return per_sm / Plan<LOGM>::T > 0 ? per_sm / Plan<LOGM>::T : 1;
+  constexpr int n = resident_threads<T, LOGM>() / Plan<LOGM, T>::kT;
+  return n > 32 ? 32 : n > 0 ? n : 1;
 }
 
 // Delta[w][l - l_lo][i][q] (+)= sum_s kw_is[q] Re sum_{n >= n0} F_wisn G[l][n] e^{-i eta_n ln k_q}
 // FP64 (n0 = 1): the term n = 0, whose phase is 1, is added and Delta is written; FP32 (n0 > 0):
 // the terms below n0 are in Delta already.  CT: cplx (FP64) or float4 (double-float pairs, FP32).
 template <int LOGM, class T, class CT, bool HALF>
-__global__ void __launch_bounds__(Plan<LOGM>::T, min_blocks<T, LOGM>())
+__global__ void __launch_bounds__(Plan<LOGM, T>::kT, min_blocks<T, LOGM>())
 k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) {
-  using P = Plan<LOGM>;
+  using P = Plan<LOGM, T>;
   using V = V2<T>;
   constexpr bool kDc = sizeof(T) == 8;
   constexpr int NI = HALF ? P::E / 2 : P::E;     // inputs and outputs of a thread
@@ -439,7 +474,7 @@ k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) 
         const V f0 = coef_at(F), g0 = __ldg(G - 1);
         dc = fma(f0.x, g0.x, -f0.y * g0.y);
       }
-      convolve<LOGM, HALF>(v, sm, A.tw1, A.tw2, A.filt);
+      convolve<P, HALF>(v, sm, A.tw1, A.tw2, A.filt);
       T* out = delta + (((size_t)w * A.n_l + (l - A.l_lo)) * A.N_tr + i) * A.N_k;
 #pragma unroll
       for (int e = 0; e < NI; ++e) {
@@ -467,9 +502,9 @@ k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) 
 // G[l][n] sum_q [kw_is[q] Dbar_i(l, q) b_q] h_{n - q}  (n0 = 0); the chunks are added in FP64 by
 // k_chirp_sum.
 template <int LOGM, class T, bool HALF>
-__global__ void __launch_bounds__(Plan<LOGM>::T, min_blocks<T, LOGM>())
+__global__ void __launch_bounds__(Plan<LOGM, T>::kT, min_blocks<T, LOGM>())
 k_chirp_adj(V2<T>* __restrict__ part, const T* __restrict__ dbar, ChirpArgs<T> A) {
-  using P = Plan<LOGM>;
+  using P = Plan<LOGM, T>;
   using V = V2<T>;
   constexpr int NI = HALF ? P::E / 2 : P::E;         // inputs of a thread
   constexpr int NO = HALF ? P::E / 2 + 1 : P::E;     // outputs (n_h <= M/2 + 1)
@@ -515,7 +550,7 @@ k_chirp_adj(V2<T>* __restrict__ part, const T* __restrict__ dbar, ChirpArgs<T> A
       }
 #pragma unroll
       for (int e = NI; e < P::E; ++e) v[e] = mk<T>(0, 0);
-      convolve<LOGM, HALF>(v, sm, A.tw1, A.tw2, A.filt);
+      convolve<P, HALF>(v, sm, A.tw1, A.tw2, A.filt);
       const V* G = G0 + (size_t)l * A.n_h;
 #pragma unroll
       for (int e = 0; e < NO; ++e) {
@@ -599,13 +634,13 @@ template <class T> __device__ __forceinline__ V2<T> cast2(double2 v) { return mk
 template <int LOGM, class T, class TA>
 __global__ void k_chirp_tables(V2<T>* __restrict__ tw1, V2<T>* __restrict__ tw2, V2<TA>* __restrict__ a,
                                V2<T>* __restrict__ b, int n0, int n_in, int N_k, double2 cc, double2 xx) {
-  using P = Plan<LOGM>;
+  using P = Plan<LOGM, T>;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < (P::R1 - 1) * P::S1) {
+  if (e < (P::E - 1) * P::S1) {
     const long k1 = e / P::S1 + 1, t = e % P::S1;
     tw1[e] = cast2<T>(unit(-(double)((k1 * t) & (P::M - 1)) / P::M));
   }
-  if (e < 15 * P::S2) {
+  if (e < (P::E - 1) * P::S2) {
     const int k2 = e / P::S2 + 1, j = e % P::S2;
     tw2[e] = cast2<T>(unit(-(double)((k2 * j) & (P::S1 - 1)) / P::S1));
   }
@@ -621,10 +656,10 @@ __global__ void k_chirp_tables(V2<T>* __restrict__ tw1, V2<T>* __restrict__ tw2,
 
 // spectrum of h_t/M, t = -t_lo .. t_hi (t_lo + t_hi < M, the rest zero), in FP64, one CTA
 template <int LOGM, class T>
-__global__ void __launch_bounds__(Plan<LOGM>::T)
+__global__ void __launch_bounds__(Plan<LOGM, T>::kT)
 k_chirp_filter(V2<T>* __restrict__ filt, int t_lo, int t_hi, double2 cc, const double2* __restrict__ tw1,
                const double2* __restrict__ tw2) {
-  using P = Plan<LOGM>;
+  using P = Plan<LOGM, T>;   // T's order of the spectrum
   extern __shared__ __align__(16) unsigned char chirp_sm[];
   double2 v[P::E];
 #pragma unroll
@@ -638,14 +673,25 @@ k_chirp_filter(V2<T>* __restrict__ filt, int t_lo, int t_hi, double2 cc, const d
       v[e].y *= 1.0 / P::M;
     }
   }
-  fft_fwd<LOGM, false>(v, reinterpret_cast<double2*>(chirp_sm), tw1, tw2);
+  fft_fwd<P, false>(v, reinterpret_cast<double2*>(chirp_sm), tw1, tw2);
 #pragma unroll
-  for (int e = 0; e < P::E; ++e) filt[e * P::T + threadIdx.x] = cast2<T>(v[e]);
+  for (int e = 0; e < P::E; ++e) filt[e * P::kT + threadIdx.x] = cast2<T>(v[e]);
+}
+
+// tw1 and tw2 of T's plan in FP64, for the filter
+template <int LOGM, class T>
+__global__ void k_chirp_twiddles64(double2* __restrict__ tw1, double2* __restrict__ tw2) {
+  using P = Plan<LOGM, T>;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < (P::E - 1) * P::S1) tw1[e] = unit(-(double)(((long)(e / P::S1 + 1) * (e % P::S1)) & (P::M - 1)) / P::M);
+  if (e < (P::E - 1) * P::S2) tw2[e] = unit(-(double)((e / P::S2 + 1) * (e % P::S2) & (P::S1 - 1)) / P::S1);
 }
 
 // ---- host side of one precision (instantiated in chirp_f64.cu and chirp_f32.cu) ----
 
-template <class T> size_t smem_bytes(int logm) { return sizeof(V2<T>) * (((size_t)1 << logm) + ((size_t)1 << logm) / 16); }
+template <int LOGM, class T> constexpr size_t smem_bytes(size_t elem = sizeof(V2<T>)) {
+  return elem * Plan<LOGM, T>::kSmem;
+}
 
 template <class F> cudaError_t with_smem(F kern, size_t smem) {
   return smem > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
@@ -657,14 +703,14 @@ struct TabLayout {
   size_t tw1d, tw2d, tw1, tw2, filt, b, a, bytes;
 };
 template <class T> TabLayout tab_layout(int logm, int n_in, int N_k, size_t a_elem) {
-  const size_t M = (size_t)1 << logm, R1 = logm == 13 ? 32 : 16, S1 = M / R1, S2 = S1 / 16;
+  const size_t M = (size_t)1 << logm;   // tw1 and tw2 hold fewer than M values each
   TabLayout L;
   size_t o = 0;
   auto put = [&](size_t bytes) { const size_t at = o; o += (bytes + 255) & ~size_t(255); return at; };
-  L.tw1d = put(16 * (R1 - 1) * S1);
-  L.tw2d = put(16 * 15 * S2);
-  L.tw1 = sizeof(T) == 8 ? L.tw1d : put(8 * (R1 - 1) * S1);
-  L.tw2 = sizeof(T) == 8 ? L.tw2d : put(8 * 15 * S2);
+  L.tw1d = put(16 * M);
+  L.tw2d = put(16 * M / 16);
+  L.tw1 = sizeof(T) == 8 ? L.tw1d : put(8 * M);
+  L.tw2 = sizeof(T) == 8 ? L.tw2d : put(8 * M / 16);
   L.filt = put(sizeof(V2<T>) * M);
   L.b = put(sizeof(V2<T>) * N_k);
   L.a = put(a_elem * n_in);
@@ -675,18 +721,17 @@ template <class T> TabLayout tab_layout(int logm, int n_in, int N_k, size_t a_el
 template <int LOGM, class T, class TA>
 cudaError_t build_tables(uint8_t* p, const TabLayout& L, int n0, int n_in, int N_k, int t_lo, int t_hi,
                          double2 cc, double2 xx, cudaStream_t s) {
-  using P = Plan<LOGM>;
-  const int n = std::max({(P::R1 - 1) * P::S1, 15 * P::S2, n_in, N_k});
+  using P = Plan<LOGM, T>;
+  const int n = std::max({P::M, n_in, N_k});
   const unsigned grid = (unsigned)((n + 255) / 256);
   double2 *tw1d = (double2*)(p + L.tw1d), *tw2d = (double2*)(p + L.tw2d);
   k_chirp_tables<LOGM, T, TA><<<grid, 256, 0, s>>>((V2<T>*)(p + L.tw1), (V2<T>*)(p + L.tw2), (V2<TA>*)(p + L.a),
                                                    (V2<T>*)(p + L.b), n0, n_in, N_k, cc, xx);
-  if (sizeof(T) == 4)
-    k_chirp_tables<LOGM, double, double><<<grid, 256, 0, s>>>(tw1d, tw2d, nullptr, nullptr, 0, 0, 0, cc, xx);
-  const size_t smem = smem_bytes<double>(LOGM);
+  if (sizeof(T) == 4) k_chirp_twiddles64<LOGM, T><<<grid, 256, 0, s>>>(tw1d, tw2d);
+  const size_t smem = smem_bytes<LOGM, T>(sizeof(double2));
   cudaError_t e = with_smem(k_chirp_filter<LOGM, T>, smem);
   if (e != cudaSuccess) return e;
-  k_chirp_filter<LOGM, T><<<1, P::T, smem, s>>>((V2<T>*)(p + L.filt), t_lo, t_hi, cc, tw1d, tw2d);
+  k_chirp_filter<LOGM, T><<<1, P::kT, smem, s>>>((V2<T>*)(p + L.filt), t_lo, t_hi, cc, tw1d, tw2d);
   return cudaGetLastError();
 }
 
@@ -707,10 +752,10 @@ cudaError_t launch_fwd(int logm, bool half, T* delta, const CT* coef, const Chir
   return by_size<T>(logm, [&](auto lm) {
     constexpr int LM = decltype(lm)::value;
     auto kern = half ? k_chirp_fwd<LM, T, CT, true> : k_chirp_fwd<LM, T, CT, false>;
-    const size_t smem = smem_bytes<T>(LM);
+    constexpr size_t smem = smem_bytes<LM, T>();
     cudaError_t e = with_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)((long)n_rows * A.n_chunk), Plan<LM>::T, smem, s>>>(delta, coef, A);
+    kern<<<(unsigned)((long)n_rows * A.n_chunk), Plan<LM, T>::kT, smem, s>>>(delta, coef, A);
     return cudaGetLastError();
   });
 }
@@ -720,10 +765,10 @@ cudaError_t launch_adj(int logm, bool half, V2<T>* part, const T* dbar, const Ch
   return by_size<T>(logm, [&](auto lm) {
     constexpr int LM = decltype(lm)::value;
     auto kern = half ? k_chirp_adj<LM, T, true> : k_chirp_adj<LM, T, false>;
-    const size_t smem = smem_bytes<T>(LM);
+    constexpr size_t smem = smem_bytes<LM, T>();
     cudaError_t e = with_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)((long)n_rows * A.n_chunk), Plan<LM>::T, smem, s>>>(part, dbar, A);
+    kern<<<(unsigned)((long)n_rows * A.n_chunk), Plan<LM, T>::kT, smem, s>>>(part, dbar, A);
     return cudaGetLastError();
   });
 }

@@ -34,6 +34,15 @@ ChirpArgs<float> args(const ChirpDir& d, const ChirpRun& r, const float2* g, con
 
 }  // namespace
 
+int chirp32_ctas_per_sm(int logm) {
+  int n = 1;
+  by_size<float>(logm, [&](auto lm) {
+    n = min_blocks<float, decltype(lm)::value>();
+    return cudaSuccess;
+  });
+  return n;
+}
+
 size_t chirp32_table_bytes(int logm, int n_in, int N_k) {
   return tab_layout<float>(logm, n_in, N_k, kA).bytes;
 }

@@ -31,6 +31,15 @@ ChirpArgs<double> args(const ChirpDir& d, const ChirpRun& r, const cplx* g, cons
 
 }  // namespace
 
+int chirp64_ctas_per_sm(int logm) {
+  int n = 1;
+  by_size<double>(logm, [&](auto lm) {
+    n = min_blocks<double, decltype(lm)::value>();
+    return cudaSuccess;
+  });
+  return n;
+}
+
 size_t chirp64_table_bytes(int logm, int n_in, int N_k) {
   return tab_layout<double>(logm, n_in, N_k, sizeof(double2)).bytes;
 }

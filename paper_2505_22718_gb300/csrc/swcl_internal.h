@@ -393,6 +393,8 @@ void chirp_drop(swcl_ctx* c);
 size_t chirp_part_bytes(const swcl_ctx* c, int precision, int n_l, bool whole);
 int chirp_forward(swcl_ctx* c, int precision, int l_lo, int n_l);
 int chirp_adjoint(swcl_ctx* c, int precision, int l_lo, int n_l, bool accumulate);
+int chirp64_ctas_per_sm(int logm);
+int chirp32_ctas_per_sm(int logm);
 size_t chirp64_table_bytes(int logm, int n_in, int N_k);
 cudaError_t chirp64_build(void* tab, int logm, int n0, int n_in, int N_k, int t_lo, int t_hi, const double* cc,
                           const double* xx, cudaStream_t s);
