@@ -183,6 +183,16 @@ __device__ __forceinline__ void mma<Bf16x9>(uint32_t d_tmem, uint64_t adesc, uin
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
+// One lane of a fully active warp, the same one at every call.  The MMA warp runs its loop with all
+// lanes and issues through this lane only: the loop's barriers and descriptors are then uniform values
+// to the compiler.  Measured with a wait and a commit every 12 products of 128 x N x 16: 54 clocks per
+// product at N = 64 and 60.5 at N = 96, against 73 for both when one lane alone runs the loop.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(r));
+  return r != 0;
+}
+
 // arrive on `bar` once every tcgen05 operation issued so far by this thread has completed
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
