@@ -1776,6 +1776,244 @@ __global__ void __maxnreg__(32) k_dimg(uint8_t* __restrict__ img, const float* _
                         off64(row, ch * 16), v);
 }
 
+// ------------------------------------------------------ low frequencies (chirp form) ----
+
+// Delta from the frequencies n < kChirpHead alone, before the chirp transforms add the rest: the same
+// compensated products as the GEMM over all frequencies (two K-blocks per accumulator slot, leading
+// product and corrections apart, the two sums added with round-to-nearest), with K = 128 in all.  With
+// so little K the work is in the operands and the result, so nothing of it passes through memory but
+// Delta itself: a CTA forms H = F G for its 64 columns in shared memory once (the arithmetic of k_himg)
+// and walks its q tiles, streaming their rows of the phase image (96 KB each, from L2) through a ring of
+// six K-blocks; the accumulators are double-buffered in TMEM (4 slots x 64 columns, twice: all 512), so
+// the epilogue warps scale and store tile t while tile t + 1 multiplies.
+// Bound by the MMA issue (54 clocks per 128 x 64 x 16 product, 48 of them per tile) and, with few
+// columns, by the forming of H.  1545 columns x 1024 k 16 us, 287 100 columns 0.76 ms, 89 970 columns x
+// 4096 k 0.81 ms; the GEMM kernels with their H image took 24 us, 3.6 ms and 1.9 ms for the same K.
+// Warps: 0 copies, 1 MMA and TMEM, 2-9 form H, then drain (two warps per 32-lane quarter, 32 columns
+// each) and store.  Columns: each half of a tile holds 32/r whole groups of r profile rows.
+constexpr int kHeadNT = 64;
+constexpr int kHeadKb = 2 * kChirpHead / kK;               // 4 K-blocks
+constexpr int kHeadStages = 6;
+constexpr uint32_t kHeadA = kPlanes * kPlaneM;             // one K-block of the phase image
+constexpr uint32_t kHeadB = kPlanes * kHeadNT * kRow;      // one K-block of H
+constexpr int kHeadThreads = 320;
+
+struct HeadShape {
+  int N_k, N_tr, N_ell, n_h, l_lo, n_l, r, NI, n_groups, n_mt, q_per, q_split;
+};
+
+__global__ void __launch_bounds__(kHeadThreads, 1)
+k_head(float* __restrict__ delta, const uint8_t* __restrict__ aimg, const float4* __restrict__ F,
+       const float4* __restrict__ gdf, const int* __restrict__ cls_of, const float* __restrict__ kmu,
+       const int2* __restrict__ cmap, HeadShape sh, int* __restrict__ status) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ long long rowoff[kHeadNT];    // Delta row of the column's group (-1: no column)
+  __shared__ int kmoff[kHeadNT];           // kmu row of the column
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* bsm = base + kHeadStages * kHeadA;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(bsm + kHeadKb * kHeadB);
+  uint64_t* afull = bars;                          // a K-block of the phase image has landed
+  uint64_t* aempty = bars + kHeadStages;           // its products have been formed
+  uint64_t* accfull = bars + 2 * kHeadStages;      // [2] a q tile's sums are complete
+  uint64_t* accempty = accfull + 2;                // [2] and read
+  uint64_t* done = accempty + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int ct = blockIdx.x / sh.q_split, mt0 = (blockIdx.x % sh.q_split) * sh.q_per;
+  const int n_it = min(sh.q_per, sh.n_mt - mt0);
+  if (tid == 0) {
+    for (int s = 0; s < kHeadStages; ++s) {
+      mbar_init(smem_u32(&afull[s]), 1);
+      mbar_init(smem_u32(&aempty[s]), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&accfull[b]), 1);
+      mbar_init(smem_u32(&accempty[b]), 8);
+    }
+    mbar_init(smem_u32(done), 1);
+    *abort_flag = 0;
+    fence_barrier_init();
+  }
+  if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 512);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int n_a = n_it * kHeadKb;                  // K-blocks of the phase image this CTA streams
+  const uint8_t* asrc = aimg + (size_t)mt0 * kHeadKb * kHeadA;
+  int issued = 0;
+  auto copy = [&](int g) {
+    const int s = g % kHeadStages;
+    mbar_arrive_tx(smem_u32(&afull[s]), kHeadA);
+    bulk_g2s(smem_u32(base + s * kHeadA), asrc + (size_t)g * kHeadA, kHeadA, smem_u32(&afull[s]));
+  };
+  if (tid == 0)
+    for (; issued < min(n_a, kHeadStages); ++issued) copy(issued);
+
+  if (warp >= 2) {
+    // column c of the tile: half c / 32, group (c % 32) / r of the half, profile row (c % 32) % r
+    const int row = (tid - 64) >> 2, ch = tid & 3;
+    const int gh = 32 / sh.r, in = row & 31, gi = in / sh.r, s = in - gi * sh.r;
+    const int g = (2 * ct + (row >> 5)) * gh + gi;
+    const bool live = gi < gh && g < sh.n_groups;
+    int wi = 0, l = 0;
+    if (live) {
+      if (cmap) {
+        const int2 cm = cmap[g];
+        wi = cm.x;
+        l = cm.y;
+      } else {
+        l = g % sh.n_l;
+        wi = g / sh.n_l;
+      }
+    }
+    const int i = wi % sh.N_tr, w = wi / sh.N_tr;
+    if (ch == 0) {
+      rowoff[row] = live ? (((long long)w * sh.n_l + l) * sh.N_tr + i) * sh.N_k : -1;
+      kmoff[row] = (i * 4 + s) * sh.N_k;
+    }
+    const float4* Fr = F + ((size_t)wi * sh.NI + s) * sh.n_h;
+    const float4* Gr = gdf + ((size_t)(live ? cls_of[i] : 0) * sh.N_ell + sh.l_lo + l) * sh.n_h;
+    // one K-block (four frequencies per thread) at a time, the next one's values in flight; not
+    // unrolled: every CTA runs this once, so its instructions come from a cold cache
+    float4 fv[4], gv[4];
+    auto fetch = [&](int kb) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int n = kb * (kK / 2) + ch * 4 + u;
+        const bool in = live && n < sh.n_h;
+        fv[u] = in ? Fr[n] : make_float4(0.f, 0.f, 0.f, 0.f);
+        gv[u] = in ? __ldg(Gr + n) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    };
+    fetch(0);
+#pragma unroll 1
+    for (int kb = 0; kb < kHeadKb; ++kb) {
+      float4 f[4], g4[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) { f[u] = fv[u]; g4[u] = gv[u]; }
+      if (kb + 1 < kHeadKb) fetch(kb + 1);
+      __nv_bfloat16 v[8][kPlanes];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float rh, rl, ih, il;
+        df_dot2(f[u].x, f[u].z, g4[u].x, g4[u].z, f[u].y, f[u].w, g4[u].y, g4[u].w, -1.0f, rh, rl);
+        df_dot2(f[u].x, f[u].z, g4[u].y, g4[u].w, f[u].y, f[u].w, g4[u].x, g4[u].z, 1.0f, ih, il);
+        split_df(rh, rl, v[2 * u]);
+        split_df(-ih, -il, v[2 * u + 1]);
+      }
+      store_planes<kPlanes>(bsm + kb * kHeadB, kHeadNT * kRow, off64(row, ch * 16), v);
+    }
+    fence_proxy_async();
+  }
+  __syncthreads();
+
+  if (warp == 0) {
+    if (lane == 0) {
+      for (; issued < n_a; ++issued) {
+        const int s = issued % kHeadStages;
+        if (!mbar_wait(smem_u32(&aempty[s]), (issued / kHeadStages - 1) & 1, abort_flag)) break;
+        copy(issued);
+      }
+      if (*abort_flag)   // copies still in flight land before the CTA exits
+        for (int g = max(0, issued - kHeadStages); g < issued; ++g)
+          mbar_wait_drain(smem_u32(&afull[g % kHeadStages]), (g / kHeadStages) & 1);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // every lane runs the loop, one issues (elect_one)
+    const uint32_t idesc = idesc_bf16(kM, kHeadNT);
+    bool ok = true;
+    for (int it = 0; it < n_it && ok; ++it) {
+      const int b = it & 1;
+      if (it >= 2)
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&accempty[b]), ((it >> 1) - 1) & 1, abort_flag));
+#pragma unroll 1
+      for (int kb = 0; kb < kHeadKb && ok; ++kb) {
+        const int g = it * kHeadKb + kb, s = g % kHeadStages;
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&afull[s]), (g / kHeadStages) & 1, abort_flag));
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t da = desc64(smem_u32(base + s * kHeadA)), db = desc64(smem_u32(bsm + kb * kHeadB));
+        const uint32_t d_main = tmem + (uint32_t)(b * 256 + (kb >> 1) * 128), d_corr = d_main + 64;
+#pragma unroll
+        for (int j = 0; j < kK / 16; ++j) {
+#pragma unroll
+          for (int t = 0; t < A3B3::kProducts; ++t) {
+            const uint64_t ad = da + (uint64_t)((A3B3::pa(t) * kPlaneM + j * 256) >> 4);
+            const uint64_t bd = db + (uint64_t)((A3B3::pb(t) * kHeadNT * kRow + j * 256) >> 4);
+            const bool first = (kb & 1) == 0 && j == 0 && t <= 1;
+            mma_bf16(t == 0 ? d_main : d_corr, ad, bd, idesc, first ? 0u : 1u);
+          }
+        }
+        if (elect_one()) mma_commit(smem_u32(&aempty[s]));
+      }
+      if (ok && elect_one()) mma_commit(smem_u32(&accfull[b]));
+      __syncwarp();
+    }
+    // every issued MMA has completed before TMEM is released
+    if (elect_one()) mma_commit(smem_u32(done));
+    mbar_wait_drain(smem_u32(done), 0);
+    __syncwarp();
+  } else {
+    const int quarter = warp & 3, c0 = ((warp - 2) >> 2) * 32;
+    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + c0;
+    for (int it = 0; it < n_it; ++it) {
+      const int b = it & 1;
+      const bool got = mbar_wait(smem_u32(&accfull[b]), (it >> 1) & 1, abort_flag);
+      if (!__all_sync(0xffffffffu, got)) break;
+      tc_fence_after();
+      const int q = (mt0 + it) * kM + quarter * 32 + lane;
+      float v = 0.0f;
+      int s = 0;
+#pragma unroll 1
+      for (int c = 0; c < 32; c += 16) {
+        __syncwarp();
+        uint32_t m0[16], r0[16], m1[16], r1[16];
+        const uint32_t a = lane_base + b * 256 + c;
+        tmem_ld16_async(a, m0);
+        tmem_ld16_async(a + 64, r0);
+        tmem_ld16_async(a + 128, m1);
+        tmem_ld16_async(a + 192, r1);
+        tmem_wait_ld();
+        reg_fence(m0);
+        reg_fence(r0);
+        reg_fence(m1);
+        reg_fence(r1);
+        if (c == 16) {
+          // the buffer is read: the MMA warp may refill it
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&accempty[b]));
+        }
+        const bool in = q < sh.N_k;
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          const float z = (__uint_as_float(m0[t]) + __uint_as_float(r0[t])) +
+                          (__uint_as_float(m1[t]) + __uint_as_float(r1[t]));
+          const long long o = rowoff[c0 + c + t];
+          if (in && o >= 0) v = fmaf(__ldg(kmu + kmoff[c0 + c + t] + q), z, v);
+          if (++s == sh.r) {
+            if (in && o >= 0) delta[o + q] = v;
+            v = 0.0f;
+            s = 0;
+          }
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && *abort_flag) atomicExch(status, 1);
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
 unsigned grid_for(long total) {
   return (unsigned)std::max<long>(1, std::min<long>((total + 255) / 256, 152L * 32));
 }
@@ -2057,12 +2295,12 @@ size_t basis_fixed_bytes(const swcl_ctx* c) {
   const size_t ng = (size_t)c->n_cls * c->N_ell * c->n_h;
   return (f_mt * f_kb + a_mt * a_kb) * kPlanes * kPlaneM + ng * (sizeof(float4) + sizeof(float2)) +
          sizeof(float) * (size_t)c->N_tr * 4 * c->N_k +
-         (size_t)kMaxNTWide * (f_kb + a_kb) * kPlanes * kRow;   // column padding of the last tile
+         (chirp ? 0 : (size_t)kMaxNTWide * (f_kb + a_kb) * kPlanes * kRow);   // column padding of the last tile
 }
 
 size_t basis_bytes_per_ell(const swcl_ctx* c) {
-  const bool chirp = chirp_use(c, SWCL_SPLIT_BF16);
-  const size_t f_kb = fwd_kblocks(c, chirp), a_kb = chirp ? 0 : (c->N_k + kK - 1) / kK;
+  if (chirp_use(c, SWCL_SPLIT_BF16)) return 0;   // no images (k_head forms its operand itself)
+  const size_t f_kb = fwd_kblocks(c, false), a_kb = (c->N_k + kK - 1) / kK;
   return (size_t)c->n_walk * c->N_tr * std::max(1, c->lr_true_rank) * (f_kb + a_kb) * kPlanes * kRow;
 }
 
@@ -2254,6 +2492,39 @@ int autotune(swcl_ctx* c, const std::vector<int>& cands, Run run, int& best) {
 
 }  // namespace
 
+// The low frequencies of Delta (k_head), then the chirp transforms of the rest.
+static int head_and_chirp(swcl_ctx* c, const ColPlan& cp, int l_lo, int n_l) {
+  const Stencil sv = stencil(c);
+  HeadShape sh;
+  sh.N_k = c->N_k;
+  sh.N_tr = c->N_tr;
+  sh.N_ell = c->N_ell;
+  sh.n_h = c->n_h;
+  sh.l_lo = l_lo;
+  sh.n_l = n_l;
+  sh.r = basis_rank(c);
+  sh.NI = sv.NI;
+  sh.n_groups = cp.n_cols / sh.r;
+  sh.n_mt = c->bt_f_mt;
+  const int per = 2 * (32 / sh.r), n_ct = (sh.n_groups + per - 1) / per;
+  // q tiles per CTA: all of them where the column tiles fill the GPU, else as many as leave one turn of
+  // CTAs (each CTA forms its columns' H)
+  sh.q_per = std::min(sh.n_mt, (int)(((long)n_ct * sh.n_mt + c->num_sms - 1) / c->num_sms));
+  sh.q_split = (sh.n_mt + sh.q_per - 1) / sh.q_per;
+  const size_t smem = kHeadStages * kHeadA + kHeadKb * kHeadB + 8 * (2 * kHeadStages + 5) + 16 + 1024;
+  cudaError_t e = cudaFuncSetAttribute(k_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return cuda_fail(c, e, "basis head attribute");
+  const int st = counted(c, "basis head", [&]() -> int {
+    k_head<<<(unsigned)((long)n_ct * sh.q_split), kHeadThreads, smem, c->stream>>>(
+        (float*)c->ws_delta.p, (const uint8_t*)c->bt_eimg_f.p, (const float4*)c->ws_coef.p,
+        (const float4*)c->bt_gdf.p, (const int*)c->d_cls_of.p, (const float*)c->bt_kmu.p, cp.cmap_f, sh,
+        (int*)c->ws_status.p);
+    const cudaError_t le = cudaGetLastError();
+    return le == cudaSuccess ? SWCL_OK : cuda_fail(c, le, "basis head");
+  });
+  return st ? st : chirp_forward(c, SWCL_SPLIT_BF16, l_lo, n_l);
+}
+
 // Delta (FP32, [n_walk][n_l][N_tr][N_k]) for multipoles [l_lo, l_lo + n_l) from the basis
 // coefficients in ws_coef (double-float).
 int basis_forward(swcl_ctx* c, int l_lo, int n_l) {
@@ -2264,6 +2535,7 @@ int basis_forward(swcl_ctx* c, int l_lo, int n_l) {
   if ((st = column_plan(c, l_lo, n_l, cp))) return st;
   const int n_cols = cp.n_cols;
   if (n_cols == 0) return SWCL_OK;   // no walker lists a multipole of this chunk
+  if (c->bt_chirp) return head_and_chirp(c, cp, l_lo, n_l);
   auto run = [&](int code, bool build) -> int {
     const int NT = code & 255;
     const int n_nt = (n_cols + NT - 1) / NT;
@@ -2289,8 +2561,7 @@ int basis_forward(swcl_ctx* c, int l_lo, int n_l) {
          return build_h(c, cp, img_cols(code), img_tiles(code, n_nt), l_lo, n_l);
        })))
     return st;
-  if ((st = counted(c, "basis gemm fwd", [&] { return run(code, false); }))) return st;
-  return c->bt_chirp ? chirp_forward(c, SWCL_SPLIT_BF16, l_lo, n_l) : SWCL_OK;
+  return counted(c, "basis gemm fwd", [&] { return run(code, false); });
 }
 
 // ws_cbar (FP64 complex, [n_walk][N_tr][NI][n_h], zeroed here) from ws_dbar (FP32,
