@@ -26,12 +26,18 @@ constexpr int MAXR = 9;   // pairs per thread: ceil(64 * 65 / 2 / 256)
 
 // dU[t][l_lo + ll][i][j] for tangent t; delta [1 + n_w][n_l][N_tr][N_k] holds the base walker
 // first, then one walker per tangent when has_w.  Grid (n_l, n_dir).
+//
+// Bound by the FP64 pipe.  With Z_i = wk2 (P' Delta_i / 2 + P Delta'_i) the sum is
+// Z_i Delta_j + Delta_i Z_j: two operations per row and two per pair and k point, instead of five per
+// pair with the three products formed apart.  103 multipoles, 8 tangents, 15 tracers, 1024 k:
+// 1157 us before, 556 us now.
 template <typename T>
 __global__ void __launch_bounds__(JT)
 k_quad_jvp(double* __restrict__ dU, const T* __restrict__ delta, const double* __restrict__ P,
            const double* __restrict__ Pdot, const double* __restrict__ wk2, int has_w, int N_tr,
            int N_k, int N_ell, int l_lo, int n_l) {
-  __shared__ double D0[64 * KJS], Dt[64 * KJS], us[KJ], uds[KJ];
+  extern __shared__ double jsm[];
+  double *D0 = jsm, *Z = jsm + (size_t)N_tr * KJS;   // Delta_i and Z_i of the staged k points
   const int ll = blockIdx.x, t = blockIdx.y;
   const int npair = N_tr * (N_tr + 1) / 2;
   const T* d0 = delta + (size_t)ll * N_tr * N_k;
@@ -41,7 +47,7 @@ k_quad_jvp(double* __restrict__ dU, const T* __restrict__ delta, const double* _
   double acc[MAXR];
 #pragma unroll
   for (int r = 0; r < MAXR; ++r) {
-    int p = threadIdx.x + r * JT, i = 0;
+    int p = threadIdx.x + r * blockDim.x, i = 0;
     acc[r] = 0.0;
     if (p < npair) {
       while (p >= N_tr - i) { p -= N_tr - i; ++i; }
@@ -50,27 +56,27 @@ k_quad_jvp(double* __restrict__ dU, const T* __restrict__ delta, const double* _
     pj[r] = i + p;
   }
   for (int q0 = 0; q0 < N_k; q0 += KJ) {
-    for (int e = threadIdx.x; e < N_tr * KJ; e += JT) {
+    for (int e = threadIdx.x; e < N_tr * KJ; e += blockDim.x) {
       const int i = e / KJ, qq = e - i * KJ, q = q0 + qq;
-      D0[i * KJS + qq] = q < N_k ? (double)d0[(size_t)i * N_k + q] : 0.0;
-      Dt[i * KJS + qq] = (has_w && q < N_k) ? (double)dt[(size_t)i * N_k + q] : 0.0;
-    }
-    for (int e = threadIdx.x; e < KJ; e += JT) {
-      const int q = q0 + e;
-      us[e] = q < N_k ? wk2[q] * P[q] : 0.0;
-      uds[e] = q < N_k ? wk2[q] * pd[q] : 0.0;
+      double d = 0.0, z = 0.0;
+      if (q < N_k) {
+        const double w = wk2[q];
+        d = (double)d0[(size_t)i * N_k + q];
+        z = 0.5 * w * pd[q] * d;
+        if (has_w) z = fma(w * P[q], (double)dt[(size_t)i * N_k + q], z);
+      }
+      D0[i * KJS + qq] = d;
+      Z[i * KJS + qq] = z;
     }
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < MAXR; ++r) {
-      if (threadIdx.x + r * JT < npair) {
-        const double* ai = D0 + pi[r] * KJS;
-        const double* aj = D0 + pj[r] * KJS;
-        const double* bi = Dt + pi[r] * KJS;
-        const double* bj = Dt + pj[r] * KJS;
+      if (threadIdx.x + r * blockDim.x < npair) {
+        const double *di = D0 + pi[r] * KJS, *dj = D0 + pj[r] * KJS;
+        const double *zi = Z + pi[r] * KJS, *zj = Z + pj[r] * KJS;
         double s = acc[r];
-        for (int qq = 0; qq < KJ; ++qq)
-          s = fma(uds[qq], ai[qq] * aj[qq], fma(us[qq], fma(bi[qq], aj[qq], ai[qq] * bj[qq]), s));
+#pragma unroll 8
+        for (int qq = 0; qq < KJ; ++qq) s = fma(zi[qq], dj[qq], fma(di[qq], zj[qq], s));
         acc[r] = s;
       }
     }
@@ -79,7 +85,7 @@ k_quad_jvp(double* __restrict__ dU, const T* __restrict__ delta, const double* _
   double* out = dU + ((size_t)t * N_ell + l_lo + ll) * N_tr * N_tr;
 #pragma unroll
   for (int r = 0; r < MAXR; ++r) {
-    if (threadIdx.x + r * JT < npair) {
+    if (threadIdx.x + r * blockDim.x < npair) {
       out[pi[r] * N_tr + pj[r]] = acc[r];
       out[pj[r] * N_tr + pi[r]] = acc[r];
     }
@@ -108,8 +114,10 @@ __global__ void k_jvp_combine(double* __restrict__ Cdot, const double* __restric
   }
 }
 
-// One CTA per multipole: Ct = A_i A_j U + diag(noise) in shared memory, its Cholesky factor in
-// place (right-looking; a pivot <= 0 marks the multipole in *status and zeroes its output), then
+// One CTA per multipole and perturbation (grid (N_ell, n_x); a CTA per multipole that took the
+// perturbations in turn was one chain of 15 n_x dependent columns: 268 us with the Gram sums at 103
+// multipoles, 8 perturbations, 15 tracers, now 80 us).  Ct = A_i A_j U + diag(noise) in shared memory, its
+// Cholesky factor in place (right-looking; a pivot <= 0 marks the multipole in *status and zeroes its output), then
 // for every X_a: T = L^-1 X_a (thread j solves column j), Y^T = L^-1 T^T (thread j solves row j
 // of T, giving row j of Y), Z_a = sqrt(nu_l / 2) Y.
 __global__ void k_fisher_whiten(double* __restrict__ Z, const double* __restrict__ X,
@@ -147,12 +155,14 @@ __global__ void k_fisher_whiten(double* __restrict__ Z, const double* __restrict
     __syncthreads();
   }
   const double s = sqrt(0.5 * modes[l]);
-  for (int a = 0; a < n_x; ++a) {
+  {
+    const int a = blockIdx.y;
     const double* x = X + ((size_t)a * N_ell + l) * n2;
     double* z = Z + ((size_t)a * N_ell + l) * n2;
     if (bad) {
       for (int e = threadIdx.x; e < n2; e += blockDim.x) z[e] = 0.0;
-      continue;
+      if (threadIdx.x == 0) atomicOr(status, 1);
+      return;
     }
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
       for (int i = 0; i < n; ++i) {
@@ -171,12 +181,10 @@ __global__ void k_fisher_whiten(double* __restrict__ Z, const double* __restrict
     }
     __syncthreads();
     for (int e = threadIdx.x; e < n2; e += blockDim.x) z[e] = s * Ys[e];
-    __syncthreads();
   }
-  if (threadIdx.x == 0 && bad) atomicOr(status, 1);
 }
 
-constexpr int GT = 256;
+constexpr int GT = 1024;
 
 // F[a][b] = F[b][a] = sum_l sum_ij Z_a[l][i][j] Z_b[l][j][i]; one CTA per pair a <= b
 __global__ void __launch_bounds__(GT)
@@ -188,12 +196,17 @@ k_fisher_gram(double* __restrict__ F, const double* __restrict__ Z, int n_x, int
   const long n2 = (long)N_tr * N_tr, per = (long)N_ell * n2;
   const double* za = Z + (size_t)a * per;
   const double* zb = Z + (size_t)b * per;
+  // thread -> entry (i, j) and a share of the multipoles (GT / n2 shares; one, over several entries,
+  // when the matrices have more than GT entries)
+  const int shares = max(1, GT / (int)n2);
+  const int share = threadIdx.x / (int)min((long)GT, n2);
   double s = 0.0;
-  for (long e = threadIdx.x; e < per; e += GT) {
-    const long l = e / n2;
-    const int ij = (int)(e - l * n2);
-    const int i = ij / N_tr, j = ij - i * N_tr;
-    s = fma(za[e], zb[l * n2 + (long)j * N_tr + i], s);
+  if (share < shares) {
+    for (int ij = shares > 1 ? threadIdx.x - share * (int)n2 : threadIdx.x; ij < n2; ij += GT) {
+      const int i = ij / N_tr, j = ij - i * N_tr, ji = j * N_tr + i;
+#pragma unroll 4
+      for (int l = share; l < N_ell; l += shares) s = fma(za[l * n2 + ij], zb[l * n2 + ji], s);
+    }
   }
   red[threadIdx.x] = s;
   __syncthreads();
@@ -214,7 +227,10 @@ cudaError_t launch_quad_jvp(double* dU, const T* delta, const double* P, const d
                             const double* wk2, bool has_w, int n_dir, int N_tr, int N_k,
                             int N_ell, int l_lo, int n_l, cudaStream_t s) {
   if (N_tr > 64) return cudaErrorInvalidValue;
-  k_quad_jvp<T><<<dim3(n_l, n_dir), JT, 0, s>>>(dU, delta, P, Pdot, wk2, has_w ? 1 : 0, N_tr, N_k,
+  // threads for the pairs (up to nine per thread)
+  const int nt = std::min(JT, std::max(64, (N_tr * (N_tr + 1) / 2 + 31) & ~31));
+  const size_t smem = 2 * sizeof(double) * N_tr * KJS;
+  k_quad_jvp<T><<<dim3(n_l, n_dir), nt, smem, s>>>(dU, delta, P, Pdot, wk2, has_w ? 1 : 0, N_tr, N_k,
                                                N_ell, l_lo, n_l);
   return cudaGetLastError();
 }
@@ -242,7 +258,7 @@ cudaError_t launch_fisher(double* F, double* Z, const double* X, const double* U
   cudaError_t e = cudaFuncSetAttribute(k_fisher_whiten, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  k_fisher_whiten<<<N_ell, 64, smem, s>>>(Z, X, U, amp, noise, modes, status, n_x, N_tr, N_ell);
+  k_fisher_whiten<<<dim3(N_ell, n_x), 64, smem, s>>>(Z, X, U, amp, noise, modes, status, n_x, N_tr, N_ell);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_fisher_gram<<<n_x * (n_x + 1) / 2, GT, 0, s>>>(F, Z, n_x, N_tr, N_ell);
   return cudaGetLastError();
