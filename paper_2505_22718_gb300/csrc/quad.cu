@@ -13,6 +13,8 @@
 // a second float), FP64 above them, in one pass when a multipole's k range fits one CTA.
 #include <algorithm>
 
+#include "f32x2.cuh"
+#include "tc_common.cuh"
 #include "swcl_internal.h"
 
 namespace swcl {
@@ -527,13 +529,130 @@ k_delta_bar(T* __restrict__ dbar, double* __restrict__ pbar_part, const T* __res
     if (q0 + u < N_k) pbar_part[((size_t)l0 * n_walk + w) * N_k + q0 + u] = (double)ps[u] + (double)pc[u];
 }
 
-__global__ void k_pbar_reduce(double* __restrict__ Pbar, const double* __restrict__ part,
-                              const double* __restrict__ wk2, int n_chunk, int n_walk, int N_k,
-                              int* __restrict__ status) {
-  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long)n_walk * N_k) return;
+// FP32 form for up to 32 tracers: two neighbouring k points per thread in packed arithmetic, Delta_j of
+// both in registers (NJ rows, those past N_tr zero), S_ij A_j from shared memory as doubled values
+// {x, x} by broadcast 16-byte loads.  Per point the sums are those of k_delta_bar in the same order.
+// What bounds it: with many multipoles and walkers the traffic of Delta, Dbar and the P_bar partials;
+// k_delta_bar, which re-read Delta_j from shared memory for every group of rows, was bound by issue.
+// 256 points of 15 tracers, ragged lists: 827 us with k_delta_bar, 530 us here; 30 tracers, 2999 multipoles,
+// 4096 k 1267 and 1129 us; one point, 103 multipoles 12.2 and 10.1 us.
+template <int NJ>
+__global__ void __launch_bounds__(128)
+k_delta_bar2(float* __restrict__ dbar, double* __restrict__ pbar_part, const float* __restrict__ delta,
+             const double* __restrict__ Cf, const double* __restrict__ amp,
+             const double* __restrict__ P, const double* __restrict__ wk2, int N_tr, int N_k,
+             int N_ell, int n_walk, int l_lo, int n_l, const int* __restrict__ listed) {
+  pdl_trigger();   // the next kernel of the step may be scheduled
+  pdl_wait();      // Delta and the cotangent come from the kernels before
+  __shared__ __align__(16) float2 St[NJ * NJ];   // St[j][i] = S_ij A_j, twice
+  __shared__ float As[NJ];
+  const int w = blockIdx.z, l0 = l_lo + blockIdx.y;
+  const int q0 = (blockIdx.x * 128 + threadIdx.x) * 2;
+  const bool in0 = q0 < N_k, in1 = q0 + 1 < N_k;
+  double* pb = pbar_part + ((size_t)l0 * n_walk + w) * N_k + q0;
+  if (listed && listed[w * n_l + (l0 - l_lo)] < 0) {
+    // a multipole the walker does not list: S = 0, so Dbar = 0 and the P_bar partial is 0; its
+    // Delta rows are not read and its Dbar rows are not used
+    if (in0) pb[0] = 0.0;
+    if (in1) pb[1] = 0.0;
+    return;
+  }
+  const size_t row0 = ((size_t)w * n_l + l0 - l_lo) * N_tr * N_k + q0;
+  const bool pair = in1 && (N_k & 1) == 0;   // 8-byte aligned
+  float2 d[NJ];
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) {
+    d[j] = make_float2(0.f, 0.f);
+    if (j < N_tr) {
+      const float* p = delta + row0 + (size_t)j * N_k;
+      if (pair) {
+        d[j] = *reinterpret_cast<const float2*>(p);
+      } else {
+        if (in0) d[j].x = p[0];
+        if (in1) d[j].y = p[1];
+      }
+    }
+  }
+  const double* A = amp + (size_t)w * N_tr;
+  const double* Cl = Cf + ((size_t)w * N_ell + l0) * N_tr * N_tr;
+  for (int e = threadIdx.x; e < NJ * NJ; e += 128) {
+    const int j = e / NJ, i = e % NJ;
+    const float v = i < N_tr && j < N_tr ? (float)(Cl[i * N_tr + j] * A[j]) : 0.0f;
+    St[e] = make_float2(v, v);
+  }
+  if (threadIdx.x < NJ) As[threadIdx.x] = threadIdx.x < N_tr ? (float)A[threadIdx.x] : 0.0f;
+  float2 two_u;
+  two_u.x = in0 ? (float)(2.0 * wk2[q0] * P[(size_t)w * N_k + q0]) : 0.0f;
+  two_u.y = in1 ? (float)(2.0 * wk2[q0 + 1] * P[(size_t)w * N_k + q0 + 1]) : 0.0f;
+  __syncthreads();
+  if (!in0) return;
+  float2 ps = make_float2(0.f, 0.f), pc = ps;
+#pragma unroll
+  for (int i0 = 0; i0 < NJ; i0 += 4) {
+    if (i0 >= N_tr) break;
+    float2 t[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) t[g] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const float4 s01 = *reinterpret_cast<const float4*>(St + j * NJ + i0);
+      const float4 s23 = *reinterpret_cast<const float4*>(St + j * NJ + i0 + 2);
+      t[0] = f2_fma(make_float2(s01.x, s01.y), d[j], t[0]);
+      t[1] = f2_fma(make_float2(s01.z, s01.w), d[j], t[1]);
+      t[2] = f2_fma(make_float2(s23.x, s23.y), d[j], t[2]);
+      t[3] = f2_fma(make_float2(s23.z, s23.w), d[j], t[3]);
+    }
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int ii = i0 + g;
+      if (ii < N_tr) {
+        const float2 ai = make_float2(As[ii], As[ii]);
+        // TwoSum of A_i Delta_i T_i
+        const float2 x = f2_mul(f2_mul(ai, d[ii]), t[g]);
+        const float2 sn = f2_add(ps, x), bp = f2_sub(sn, ps);
+        pc = f2_add(pc, f2_add(f2_sub(ps, f2_sub(sn, bp)), f2_sub(x, bp)));
+        ps = sn;
+        const float2 o = f2_mul(f2_mul(two_u, ai), t[g]);
+        float* out = dbar + row0 + (size_t)ii * N_k;
+        if (pair) {
+          *reinterpret_cast<float2*>(out) = o;
+        } else {
+          out[0] = o.x;
+          if (in1) out[1] = o.y;
+        }
+      }
+    }
+  }
+  if (pair) {
+    *reinterpret_cast<double2*>(pb) = make_double2((double)ps.x + (double)pc.x, (double)ps.y + (double)pc.y);
+  } else {
+    pb[0] = (double)ps.x + (double)pc.x;
+    if (in1) pb[1] = (double)ps.y + (double)pc.y;
+  }
+}
+
+// P_bar = wk2 x the sum over the chunks (multipoles).  One thread per k point and walker took the chunks
+// one after the other: 16 CTAs and 2999 dependent loads at the large shape, 520 us.  Here eight threads
+// share a point (chunks g, g + 8, ..., then the eight sums in order): 66 us; one
+// point, 103 multipoles 16.8 and 8.0 us.
+constexpr int PQ = 32, PG = 8;
+__global__ void __launch_bounds__(PQ * PG)
+k_pbar_reduce(double* __restrict__ Pbar, const double* __restrict__ part,
+              const double* __restrict__ wk2, int n_chunk, int n_walk, int N_k,
+              int* __restrict__ status) {
+  __shared__ double red[PG][PQ];
+  const int tl = threadIdx.x % PQ, g = threadIdx.x / PQ;
+  const long t = (long)blockIdx.x * PQ + tl, n = (long)n_walk * N_k;
   double s = 0.0;
-  for (int c = 0; c < n_chunk; ++c) s += part[(size_t)c * n_walk * N_k + t];
+  if (t < n) {
+#pragma unroll 8
+    for (int c = g; c < n_chunk; c += PG) s += part[(size_t)c * n + t];
+  }
+  red[g][tl] = s;
+  __syncthreads();
+  if (g || t >= n) return;
+#pragma unroll
+  for (int u = 1; u < PG; ++u) s += red[u][tl];
   const double v = wk2[t % N_k] * s;
   flag_nonfinite(status, v);
   Pbar[t] = v;
@@ -642,6 +761,15 @@ cudaError_t launch_delta_bar(T* dbar, const T* delta, const double* Cf, const do
                              const double* P, const double* wk2, int n_walk, int N_tr, int N_k,
                              int N_ell, int l_lo, int n_l, double* scratch, cudaStream_t s,
                              const int* listed, bool pdl) {
+  if constexpr (sizeof(T) == 4) {
+    // up to 32 tracers, whose rows fit the registers
+    if (N_tr <= 32) {
+      auto kern = N_tr <= 4 ? k_delta_bar2<4> : N_tr <= 8 ? k_delta_bar2<8> : N_tr <= 16 ? k_delta_bar2<16>
+                                                                                         : k_delta_bar2<32>;
+      return launch_k(pdl, kern, dim3((N_k + 255) / 256, n_l, n_walk), dim3(128), 0, s, dbar, scratch, delta, Cf,
+                      amp, P, wk2, N_tr, N_k, N_ell, n_walk, l_lo, n_l, listed);
+    }
+  }
   constexpr int DQ = DT * DbarQ<T>::QT;
   const size_t smem = (size_t)(N_tr * delta_bar_pitch(N_tr) + N_tr * DQ + N_tr) * sizeof(T);
   if (smem > 48 * 1024) {
@@ -658,7 +786,7 @@ cudaError_t launch_pbar_reduce(double* P_bar, const double* scratch, const doubl
                                int n_walk, int N_k, int N_ell, cudaStream_t s, int* status) {
   const int n_chunk = (N_ell + LC - 1) / LC;
   const long n = (long)n_walk * N_k;
-  k_pbar_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(P_bar, scratch, wk2, n_chunk, n_walk, N_k,
+  k_pbar_reduce<<<(unsigned)((n + PQ - 1) / PQ), PQ * PG, 0, s>>>(P_bar, scratch, wk2, n_chunk, n_walk, N_k,
                                                            status);
   return cudaGetLastError();
 }
