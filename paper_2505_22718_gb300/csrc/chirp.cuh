@@ -454,6 +454,27 @@ k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) 
         if constexpr (kDc) km[e] = k;
       }
     }
+    // A row of zeros, as the tangents of all tracers that a perturbation does not touch are, transforms
+    // to zeros.  (A NaN compares unequal.)  Forward mode along 8 tangents, two of which move one window
+    // each, 15 tracers, 103 multipoles, N = 2048, N_k = 1024: 3935 -> 871 us, and the same 480 us as
+    // before where no row is zero.  In FP32 the test costs 3 to 9 % where no row is zero.
+    if constexpr (kDc) {
+      bool live = false;
+      for (int m = t - 1; m < n_in; m += P::kT) {
+        const V x = coef_at(F + A.n0 + m);
+        live = live || x.x != T(0) || x.y != T(0);
+      }
+      if (!__syncthreads_or(live)) {
+        if (s == 0) {
+          for (int u = u0; u < u1; ++u) {
+            const int l = A.off ? A.idx[lo + u] : A.l_lo + u;
+            T* out = delta + (((size_t)w * A.n_l + (l - A.l_lo)) * A.N_tr + i) * A.N_k;
+            for (int q = t; q < A.N_k; q += P::kT) out[q] = T(0);
+          }
+        }
+        continue;
+      }
+    }
     for (int u = u0; u < u1; ++u) {
       const int l = A.off ? A.idx[lo + u] : A.l_lo + u;
       const V* G = G0 + (size_t)l * A.n_h + A.n0;
