@@ -38,6 +38,7 @@ k_quad_jvp(double* __restrict__ dU, const T* __restrict__ delta, const double* _
            int N_k, int N_ell, int l_lo, int n_l) {
   extern __shared__ double jsm[];
   double *D0 = jsm, *Z = jsm + (size_t)N_tr * KJS;   // Delta_i and Z_i of the staged k points
+  double *za = Z + (size_t)N_tr * KJS, *zb = za + KJ;   // wk2 P' / 2 and wk2 P: Z_i = za Delta_i + zb Delta'_i
   const int ll = blockIdx.x, t = blockIdx.y;
   const int npair = N_tr * (N_tr + 1) / 2;
   const T* d0 = delta + (size_t)ll * N_tr * N_k;
@@ -56,14 +57,19 @@ k_quad_jvp(double* __restrict__ dU, const T* __restrict__ delta, const double* _
     pj[r] = i + p;
   }
   for (int q0 = 0; q0 < N_k; q0 += KJ) {
+    if (threadIdx.x < KJ) {
+      const int q = q0 + threadIdx.x;
+      za[threadIdx.x] = q < N_k ? 0.5 * wk2[q] * pd[q] : 0.0;
+      zb[threadIdx.x] = q < N_k && has_w ? wk2[q] * P[q] : 0.0;
+    }
+    __syncthreads();
     for (int e = threadIdx.x; e < N_tr * KJ; e += blockDim.x) {
       const int i = e / KJ, qq = e - i * KJ, q = q0 + qq;
       double d = 0.0, z = 0.0;
       if (q < N_k) {
-        const double w = wk2[q];
         d = (double)d0[(size_t)i * N_k + q];
-        z = 0.5 * w * pd[q] * d;
-        if (has_w) z = fma(w * P[q], (double)dt[(size_t)i * N_k + q], z);
+        z = za[qq] * d;
+        if (has_w) z = fma(zb[qq], (double)dt[(size_t)i * N_k + q], z);
       }
       D0[i * KJS + qq] = d;
       Z[i * KJS + qq] = z;
@@ -229,7 +235,7 @@ cudaError_t launch_quad_jvp(double* dU, const T* delta, const double* P, const d
   if (N_tr > 64) return cudaErrorInvalidValue;
   // threads for the pairs (up to nine per thread)
   const int nt = std::min(JT, std::max(64, (N_tr * (N_tr + 1) / 2 + 31) & ~31));
-  const size_t smem = 2 * sizeof(double) * N_tr * KJS;
+  const size_t smem = 2 * sizeof(double) * (N_tr * KJS + KJ);
   k_quad_jvp<T><<<dim3(n_l, n_dir), nt, smem, s>>>(dU, delta, P, Pdot, wk2, has_w ? 1 : 0, N_tr, N_k,
                                                N_ell, l_lo, n_l);
   return cudaGetLastError();
