@@ -73,6 +73,17 @@ template <> __device__ __forceinline__ float2 sub<float2>(float2 a, float2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pk(a)), "l"(pk(b)));
   return upk(r);
 }
+// a + c b and a - c b with a real constant c
+template <class V, class T> __device__ __forceinline__ V axpy(T c, V b, V a) {
+  a.x = fma(c, b.x, a.x);
+  a.y = fma(c, b.y, a.y);
+  return a;
+}
+template <> __device__ __forceinline__ float2 axpy<float2, float>(float c, float2 b, float2 a) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pk(make_float2(c, c))), "l"(pk(b)), "l"(pk(a)));
+  return upk(r);
+}
 // a b, and a conj(b)
 template <class V> __device__ __forceinline__ V mul(V a, V b) {
   V r;
@@ -136,36 +147,50 @@ __host__ __device__ constexpr double cos32(int j) {
 }
 __host__ __device__ constexpr double sin32(int j) { return cos32(j + 24); }   // cos(x - pi/2)
 
-// v e^{2 pi i S j / 32}, J a compile-time constant
-template <int S, int J, class V> __device__ __forceinline__ V tw32(V v) {
-  constexpr int j = J & 31;
-  if constexpr (j == 0) {
-    return v;
-  } else if constexpr (j == 8) {
-    return rot<S>(v);
-  } else if constexpr (j == 16) {
-    V r;
-    r.x = -v.x;
-    r.y = -v.y;
-    return r;
-  } else {
-    using T = decltype(v.x);
-    constexpr T c = (T)cos32(j), s = (T)(S * sin32(j));
-    V r;
-    if constexpr (j == 4) {
-      const T h = c;
-      if constexpr (S > 0) { r.x = (v.x - v.y) * h; r.y = (v.x + v.y) * h; }
-      else { r.x = (v.x + v.y) * h; r.y = (v.y - v.x) * h; }
-    } else if constexpr (j == 12) {
-      const T h = -c;
-      if constexpr (S > 0) { r.x = -(v.x + v.y) * h; r.y = (v.x - v.y) * h; }
-      else { r.x = (v.y - v.x) * h; r.y = -(v.x + v.y) * h; }
-    } else {
-      r.x = fma(v.x, c, -v.y * s);
-      r.y = fma(v.x, s, v.y * c);
-    }
-    return r;
+// e^{2 pi i S J / 32} = tw_scale(J) i^(S k) (1 + i S t), k the nearest quarter turn and t the tangent of the
+// rest, |t| <= 1: tw_tan is the product without the scale, one FMA per component, and the scale goes
+// into the FMAs of the additions that follow.  A 4-point DFT with three constant factors so takes 22
+// operations instead of 28: 16-point passes 144 and not 160, 8-point ones 52 and not 56.
+__host__ __device__ constexpr int tw_quarter(int J) { return ((J & 31) + 4) >> 3; }
+__host__ __device__ constexpr int tw_rest(int J) { return (J & 31) - 8 * tw_quarter(J); }   // -4 .. 3
+__host__ __device__ constexpr double tw_scale(int J) { return cos32(tw_rest(J)); }
+
+template <int S, int J, class V> __device__ __forceinline__ V tw_tan(V v) {
+  using T = decltype(v.x);
+  constexpr int r = tw_rest(J), k = tw_quarter(J) & 3;
+  V u = v;
+  if constexpr (r == -4) {
+    u.x = S > 0 ? v.x + v.y : v.x - v.y;
+    u.y = S > 0 ? v.y - v.x : v.y + v.x;
+  } else if constexpr (r != 0) {
+    constexpr T t = (T)(S * sin32(r) / cos32(r));
+    u.x = fma(-t, v.y, v.x);
+    u.y = fma(t, v.x, v.y);
   }
+  if constexpr (k == 1) return rot<S>(u);
+  if constexpr (k == 3) return rot<-S>(u);
+  if constexpr (k == 2) {
+    u.x = -u.x;
+    u.y = -u.y;
+  }
+  return u;
+}
+// a + c b with c = 1 as an addition
+template <int NUM, int DEN, class V> __device__ __forceinline__ V add_scaled(V a, V b, bool minus) {
+  using T = decltype(a.x);
+  constexpr double c = tw_scale(NUM) / tw_scale(DEN);
+  if constexpr (c == 1.0) return minus ? sub(a, b) : add(a, b);
+  else return axpy((T)(minus ? -c : c), b, a);
+}
+// the 4-point DFT of a, b w^JB, c w^JC, d w^JD (w = e^{2 pi i S / 32})
+template <int S, int JB, int JC, int JD, class V> __device__ __forceinline__ void dft4_tw(V& a, V& b, V& c, V& d) {
+  const V bp = tw_tan<S, JB>(b), cp = tw_tan<S, JC>(c), dp = tw_tan<S, JD>(d);
+  const V s0 = add_scaled<JC, 0>(a, cp, false), d0 = add_scaled<JC, 0>(a, cp, true);
+  const V s1 = add_scaled<JD, JB>(bp, dp, false), d1 = rot<S>(add_scaled<JD, JB>(bp, dp, true));
+  a = add_scaled<JB, 0>(s0, s1, false);
+  b = add_scaled<JB, 0>(d0, d1, false);
+  c = add_scaled<JB, 0>(s0, s1, true);
+  d = add_scaled<JB, 0>(d0, d1, true);
 }
 
 template <int S, class V> __device__ __forceinline__ void dft2(V* v) {
@@ -180,11 +205,8 @@ template <int S, class V> __device__ __forceinline__ void dft8(V* v) {
     u[j] = add(v[j], v[j + 4]);
     w[j] = sub(v[j], v[j + 4]);
   }
-  w[1] = tw32<S, 4>(w[1]);
-  w[2] = tw32<S, 8>(w[2]);
-  w[3] = tw32<S, 12>(w[3]);
   dft4<S>(u[0], u[1], u[2], u[3]);
-  dft4<S>(w[0], w[1], w[2], w[3]);
+  dft4_tw<S, 4, 8, 12>(w[0], w[1], w[2], w[3]);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     v[2 * j] = u[j];
@@ -194,9 +216,9 @@ template <int S, class V> __device__ __forceinline__ void dft8(V* v) {
 // the same with v[4..7] = 0
 template <int S, class V> __device__ __forceinline__ void dft8_half(V* v) {
   V u[4] = {v[0], v[1], v[2], v[3]};
-  V w[4] = {v[0], tw32<S, 4>(v[1]), tw32<S, 8>(v[2]), tw32<S, 12>(v[3])};
+  V w[4] = {v[0], v[1], v[2], v[3]};
   dft4<S>(u[0], u[1], u[2], u[3]);
-  dft4<S>(w[0], w[1], w[2], w[3]);
+  dft4_tw<S, 4, 8, 12>(w[0], w[1], w[2], w[3]);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     v[2 * j] = u[j];
@@ -211,17 +233,10 @@ template <int S, bool HALF, class V> __device__ __forceinline__ void dft16(V* v)
     else dft4<S>(v[j], v[j + 4], v[j + 8], v[j + 12]);
   }
   // now v[4 k1 + n2]; times w16^{n2 k1}
-  v[5] = tw32<S, 2>(v[5]);
-  v[6] = tw32<S, 4>(v[6]);
-  v[7] = tw32<S, 6>(v[7]);
-  v[9] = tw32<S, 4>(v[9]);
-  v[10] = tw32<S, 8>(v[10]);
-  v[11] = tw32<S, 12>(v[11]);
-  v[13] = tw32<S, 6>(v[13]);
-  v[14] = tw32<S, 12>(v[14]);
-  v[15] = tw32<S, 18>(v[15]);
-#pragma unroll
-  for (int k1 = 0; k1 < 4; ++k1) dft4<S>(v[4 * k1], v[4 * k1 + 1], v[4 * k1 + 2], v[4 * k1 + 3]);
+  dft4<S>(v[0], v[1], v[2], v[3]);
+  dft4_tw<S, 2, 4, 6>(v[4], v[5], v[6], v[7]);
+  dft4_tw<S, 4, 8, 12>(v[8], v[9], v[10], v[11]);
+  dft4_tw<S, 6, 12, 18>(v[12], v[13], v[14], v[15]);
   // v[4 k1 + k2] -> X[k1 + 4 k2]
 #pragma unroll
   for (int a = 0; a < 4; ++a)
@@ -232,10 +247,9 @@ template <int S, bool HALF, class V> __device__ __forceinline__ void dft16(V* v)
       v[4 * b + a] = t;
     }
 }
-template <int S, int K1, class V> __device__ __forceinline__ void tw_row32(V* r) {   // w32^{n2 k1}
-  r[1] = tw32<S, K1>(r[1]);
-  r[2] = tw32<S, 2 * K1>(r[2]);
-  r[3] = tw32<S, 3 * K1>(r[3]);
+template <int S, int K1, class V> __device__ __forceinline__ void dft_row32(V* r) {   // times w32^{n2 k1}
+  if constexpr (K1 == 0) dft4<S>(r[0], r[1], r[2], r[3]);
+  else dft4_tw<S, K1, 2 * K1, 3 * K1>(r[0], r[1], r[2], r[3]);
 }
 // n = 4 n1 + n2, n1 < 8, k = k1 + 8 k2
 template <int S, bool HALF, class V> __device__ __forceinline__ void dft32(V* v) {
@@ -249,19 +263,18 @@ template <int S, bool HALF, class V> __device__ __forceinline__ void dft32(V* v)
 #pragma unroll
     for (int a = 0; a < 8; ++a) y[a][j] = c[a];
   }
-  tw_row32<S, 1>(y[1]);
-  tw_row32<S, 2>(y[2]);
-  tw_row32<S, 3>(y[3]);
-  tw_row32<S, 4>(y[4]);
-  tw_row32<S, 5>(y[5]);
-  tw_row32<S, 6>(y[6]);
-  tw_row32<S, 7>(y[7]);
+  dft_row32<S, 0>(y[0]);
+  dft_row32<S, 1>(y[1]);
+  dft_row32<S, 2>(y[2]);
+  dft_row32<S, 3>(y[3]);
+  dft_row32<S, 4>(y[4]);
+  dft_row32<S, 5>(y[5]);
+  dft_row32<S, 6>(y[6]);
+  dft_row32<S, 7>(y[7]);
 #pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    dft4<S>(y[a][0], y[a][1], y[a][2], y[a][3]);
+  for (int a = 0; a < 8; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) v[a + 8 * b] = y[a][b];
-  }
 }
 // R points; HALF: v[R/2 .. R-1] = 0 on input
 template <int R, int S, bool HALF = false, class V> __device__ __forceinline__ void dft(V* v) {
