@@ -779,7 +779,6 @@ static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need, bool whole_par
                  + 2 * sizeof(double) * nw * N_ell * ntr2               // U, symmetrised cotangent
                  + sizeof(double) * out_count(c) * ntr2                 // output staging
                  + sizeof(double) * nrow * c->N
-                 + swcl::fftlog_adj_scratch_bytes(c->n_walk, c->N_tr, sv.NI, c->N)
                  + swcl::delta_bar_scratch_bytes(c->n_walk, c->N_k, N_ell)
                  + sizeof(double) * (nw * c->N_k + nrow);
   if (basis) fixed += swcl::basis_fixed_bytes(c);
@@ -1043,7 +1042,7 @@ int swcl_vjp(swcl_ctx* c, int precision, const double* C_bar, double* P_bar, dou
   SWCL_TRY(swcl::ensure(c, c->ws_outP, sizeof(double) * nw * (size_t)N_k));
   SWCL_TRY(swcl::ensure(c, c->ws_outA, sizeof(double) * nrow));
   const size_t wbytes = sizeof(double) * nrow * N;
-  SWCL_TRY(swcl::ensure(c, c->ws_outW, wbytes + swcl::fftlog_adj_scratch_bytes(nw, N_tr, N_I, N)));
+  SWCL_TRY(swcl::ensure(c, c->ws_outW, wbytes));
   if (c->overlap) {
     // unpacked on the auxiliary stream during the forward pass (swcl_compute_batched)
     SWCL_TRY_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_unpack, 0), "join unpack");
@@ -1121,12 +1120,11 @@ int swcl_vjp(swcl_ctx* c, int precision, const double* C_bar, double* P_bar, dou
   double* Wb = nullptr;
   if (W_bar) {
     Wb = swcl::is_device_ptr(W_bar) ? W_bar : (double*)c->ws_outW.p;
-    double* scratch = (double*)((char*)c->ws_outW.p + wbytes);
     if (n_fft > 0) {
-      SWCL_LAUNCH(c, swcl::launch_fftlog_adj(Wb, (const cplx*)c->ws_cbar.p,
+      SWCL_LAUNCH(c, swcl::launch_fftlog_adj(Wb, (cplx*)c->ws_cbar.p,
                                              (const double*)c->d_chipow.p, sv.D, sv.B,
                                              (const cplx*)c->d_psi.p, (const cplx*)c->d_twiddle.p,
-                                             nw, N_tr, N_I, N, scratch, c->stream,
+                                             nw, N_tr, N_I, N, c->stream,
                                              (int*)c->ws_status.p, c->pdl && !c->prof), "fftlog adj");
       if (!swcl::fftlog_adj_single_launch(nw, N_tr, N_I, N)) ++c->last_launches;  // chunk reduction
     } else {

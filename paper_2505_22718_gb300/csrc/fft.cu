@@ -9,6 +9,8 @@
 // e^{-2 pi i t/N}, t < N, so the only FP64 arithmetic is the butterflies themselves.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "swcl_internal.h"
 
 namespace cg = cooperative_groups;
@@ -134,32 +136,45 @@ k_fftlog_fwd(CT* __restrict__ coef, const double* __restrict__ W,
   }
   __syncthreads();
   cplx* Z = stockham(a, b, n2, rows, tw, N);
-  // unpack: X_n = E_n + e^{-2 pi i n/N} O_n, E = (Z_n + conj Z_{n2-n})/2, O = (Z_n - conj Z_{n2-n})/(2i)
-  for (int g = threadIdx.x; g < rows * n_h; g += blockDim.x) {
-    int r = g / n_h, n = g - r * n_h;
-    long row = row0 + r;
-    int i = (int)((row / N_I) % N_tr);
+  // unpack: X_n = E_n + e^{-2 pi i n/N} O_n, E = (Z_n + conj Z_{n2-n})/2, O = (Z_n - conj Z_{n2-n})/(2i),
+  // and X_{n2-n} = conj(E_n - e^{-2 pi i n/N} O_n) from the same products (the FP64 pipe is the bound: 2250
+  // rows of 2048 points 267 us with every n for itself, 247 us so)
+  const int np = n2 / 2 + 1;
+  for (int g = threadIdx.x; g < rows * np; g += blockDim.x) {
+    const int r = g / np, n = g - r * np, m = n2 - n;
+    const long row = row0 + r;
+    const int i = (int)((row / N_I) % N_tr);
     const cplx* z = Z + r * n2;
-    cplx zn = z[n == n2 ? 0 : n];
-    cplx zc = cconj(z[n == 0 ? 0 : n2 - n]);
-    cplx e = {0.5 * (zn.x + zc.x), 0.5 * (zn.y + zc.y)};
-    cplx dlt = {0.5 * (zn.x - zc.x), 0.5 * (zn.y - zc.y)};
-    cplx o = {dlt.y, -dlt.x};  // dlt / i
-    cplx x = cadd(e, cmul(tw[n], o));
-    store_coef(coef + row * n_h + n, cmul(psi[(size_t)i * n_h + n], x));
+    const cplx zn = z[n], zc = cconj(z[n == 0 ? 0 : m]);
+    const cplx e = {0.5 * (zn.x + zc.x), 0.5 * (zn.y + zc.y)};
+    const cplx dlt = {0.5 * (zn.x - zc.x), 0.5 * (zn.y - zc.y)};
+    const cplx t = cmul(tw[n], cplx{dlt.y, -dlt.x});  // O = dlt / i
+    CT* out = coef + row * n_h;
+    const cplx* ps = psi + (size_t)i * n_h;
+    store_coef(out + n, cmul(ps[n], cadd(e, t)));
+    if (m != n) store_coef(out + m, cmul(ps[m], cconj(csub(e, t))));
   }
 }
 
 // Adjoint.  For row (w, i, a): Y_n = conj(psi_n) cbar_n, H_0 = Re Y_0, H_{N/2} = Re Y_{N/2},
 // H_n = Y_n / 2 otherwise; gbar_m = sum_{n<N} H_n e^{+2 pi i n m/N} (Hermitian H), computed as
 // x_{2j} + i x_{2j+1} = sum_n (E_n + i O_n) e^{+2 pi i n j/(N/2)} with
-// E_n = H_n + conj H_{n2-n}, O_n = (H_n - conj H_{n2-n}) e^{+2 pi i n/N}; the inverse transform is
-// conj(FFT(conj(.))).  Each CTA sums gbar * chipow * D_a * B_ia over a chunk of knots of one
-// (walker, tracer) into scratch[chunk][w*N_tr+i][m].
+// E_n = H_n + conj H_{n2-n}, O_n = (H_n - conj H_{n2-n}) e^{+2 pi i n/N}, E_{n2-n} = conj E_n and
+// O_{n2-n} = conj O_n; the inverse transform is conj(FFT(conj(.))).  Each CTA sums gbar * chipow * D_a *
+// B_ia over a chunk of kc knots of one (walker, tracer).  One chunk writes W_bar; with several, the sum of a chunk goes to the place of the
+// chunk's first row of cbar, which nothing else reads and which is longer by two values, and
+// k_sum_chunks adds them in order.
 constexpr int kKnotChunk = 16;
 
+// Knots per CTA: as many as leave eight CTAs per SM, since the transforms of one CTA are a serial chain
+// of passes and barriers.  15 rows of 150 knots, N = 2048: 561 us with 16 knots in each of 150 CTAs, 532 us
+// with 5 in 450, and with one in 2250 236 us and 20 us for the sum over them.
+inline int knots_per_cta(long rows, int N_I) {
+  return (int)std::max<long>(1, std::min<long>({rows * N_I / (8 * 152), N_I, kKnotChunk}));
+}
+
 __global__ void __launch_bounds__(kThreads)
-k_fftlog_adj(double* __restrict__ scratch, const cplx* __restrict__ cbar,
+k_fftlog_adj(double* __restrict__ W_bar, cplx* cbar, int kc, int* __restrict__ status,
              const double* __restrict__ chipow, const double* __restrict__ D,
              const double* __restrict__ B, const cplx* __restrict__ psi,
              const cplx* __restrict__ tw, int n_walk, int N_tr, int N_I, int N) {
@@ -169,58 +184,67 @@ k_fftlog_adj(double* __restrict__ scratch, const cplx* __restrict__ cbar,
   const int n2 = N / 2, n_h = N / 2 + 1;
   cplx* a = smem;
   cplx* b = smem + n2;
-  double* acc = reinterpret_cast<double*>(smem + 2 * n2);
+  double* acc = reinterpret_cast<double*>(smem + 2 * n2);   // sums over the knots (kc > 1)
   const int wi = blockIdx.y;          // walker * N_tr + tracer
   const int i = wi % N_tr;
-  const int chunk = blockIdx.x;
-  const int a0 = chunk * kKnotChunk;
-  const int a1 = min(N_I, a0 + kKnotChunk);
-  for (int m = threadIdx.x; m < N; m += blockDim.x) acc[m] = 0.0;
+  const int a0 = blockIdx.x * kc;
+  const int a1 = min(N_I, a0 + kc);
+  const bool whole = gridDim.x == 1;
+  double* out = whole ? W_bar + (size_t)wi * N
+                      : reinterpret_cast<double*>(cbar + ((size_t)wi * N_I + a0) * n_h);
   const cplx* ps = psi + (size_t)i * n_h;
   for (int ka = a0; ka < a1; ++ka) {
     const cplx* cb = cbar + ((size_t)wi * N_I + ka) * n_h;
-    for (int n = threadIdx.x; n < n2; n += blockDim.x) {
-      // H_n and conj H_{n2-n}
-      cplx y = cmulc(cb[n], ps[n]);           // cbar * conj(psi) ... conj(psi) cbar
-      cplx h = (n == 0) ? cplx{y.x, 0.0} : cplx{0.5 * y.x, 0.5 * y.y};
-      int m = n2 - n;
-      cplx ym = cmulc(cb[m], ps[m]);
-      cplx hm = (m == n2) ? cplx{ym.x, 0.0} : cplx{0.5 * ym.x, 0.5 * ym.y};
-      cplx hmc = cconj(hm);
-      cplx e = cadd(h, hmc);
-      cplx d = csub(h, hmc);
-      cplx o = cmulc(d, tw[n]);                // * e^{+2 pi i n/N}
-      // Z = E + i O, store conj(Z) for the forward transform
-      cplx z = {e.x - o.y, e.y + o.x};
-      a[n] = cconj(z);
+    for (int n = threadIdx.x; n <= n2 / 2; n += blockDim.x) {
+      const int m = n2 - n;
+      const cplx y = cmulc(cb[n], ps[n]), ym = cmulc(cb[m], ps[m]);   // conj(psi) cbar
+      const cplx h = n == 0 ? cplx{y.x, 0.0} : cplx{0.5 * y.x, 0.5 * y.y};
+      const cplx hmc = n == 0 ? cplx{ym.x, 0.0} : cplx{0.5 * ym.x, -0.5 * ym.y};
+      const cplx e = cadd(h, hmc);
+      const cplx o = cmulc(csub(h, hmc), tw[n]);   // * e^{+2 pi i n/N}
+      // conj(E + i O) at n, for the forward transform; conj(conj E + i conj O) at n2 - n
+      a[n] = {e.x - o.y, -(e.y + o.x)};
+      if (n > 0 && m != n) a[m] = {e.x + o.y, e.y - o.x};
     }
     __syncthreads();
-    cplx* Z = stockham(a, b, n2, 1, tw, N);
+    const cplx* Z = stockham(a, b, n2, 1, tw, N);
     const double* cp = chipow + (size_t)i * N;
     const double* d = D + (size_t)ka * N;
     const double* bb = B ? B + ((size_t)i * N_I + ka) * N : nullptr;
     for (int j = threadIdx.x; j < n2; j += blockDim.x) {
-      cplx v = cconj(Z[j]);
-      int m = 2 * j;
+      const cplx v = cconj(Z[j]);
+      const int m = 2 * j;
       double f0 = cp[m] * d[m], f1 = cp[m + 1] * d[m + 1];
       if (bb) { f0 *= bb[m]; f1 *= bb[m + 1]; }
-      acc[m] = fma(v.x, f0, acc[m]);
-      acc[m + 1] = fma(v.y, f1, acc[m + 1]);
+      const double x0 = ka > a0 ? fma(v.x, f0, acc[m]) : v.x * f0;
+      const double x1 = ka > a0 ? fma(v.y, f1, acc[m + 1]) : v.y * f1;
+      if (ka + 1 < a1) {
+        acc[m] = x0;
+        acc[m + 1] = x1;
+      } else {
+        if (whole) {
+          flag_nonfinite(status, x0);
+          flag_nonfinite(status, x1);
+        }
+        out[m] = x0;
+        out[m + 1] = x1;
+      }
     }
     __syncthreads();
   }
-  double* out = scratch + ((size_t)chunk * n_walk * N_tr + wi) * N;
-  for (int m = threadIdx.x; m < N; m += blockDim.x) out[m] = acc[m];
 }
 
-__global__ void k_sum_chunks(double* __restrict__ W_bar, const double* __restrict__ scratch,
-                             long per_chunk, int nchunk, int* __restrict__ status) {
+__global__ void k_sum_chunks(double* __restrict__ W_bar, const cplx* __restrict__ cbar, long total, int N,
+                             int N_I, int kc, int* __restrict__ status) {
   pdl_trigger();   // the next kernel of the step may be scheduled
   pdl_wait();      // every earlier kernel of the step has completed
-  long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= per_chunk) return;
+  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= total) return;
+  const long wi = t / N, n_h = N / 2 + 1;
+  const double* p = reinterpret_cast<const double*>(cbar + wi * N_I * n_h) + (t - wi * N);
   double s = 0.0;
-  for (int c = 0; c < nchunk; ++c) s += scratch[(size_t)c * per_chunk + t];
+#pragma unroll 4
+  for (int a = 0; a < N_I; a += kc) s += p[2 * n_h * a];
   flag_nonfinite(status, s);
   W_bar[t] = s;
 }
@@ -364,9 +388,9 @@ k_fftlog_fwd_cl(CT* __restrict__ coef, const double* __restrict__ W,
 
 // Adjoint in the cluster form for rows (w, i) with all their knots (N_I <= kKnotChunk): the
 // inverse transform of each knot's Hermitian-packed input by the same four-step DFT, the
-// products with chipow D_a B_ia summed over the knots in registers, one chunk of scratch.
+// products with chipow D_a B_ia summed over the knots in registers, straight to W_bar.
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
-k_fftlog_adj_cl(double* __restrict__ scratch, const cplx* __restrict__ cbar,
+k_fftlog_adj_cl(double* __restrict__ W_bar, const cplx* __restrict__ cbar,
                 const double* __restrict__ chipow, const double* __restrict__ D,
                 const double* __restrict__ B, const cplx* __restrict__ psi,
                 const cplx* __restrict__ tw, int N_tr, int N_I, int N, int* __restrict__ status) {
@@ -443,7 +467,7 @@ k_fftlog_adj_cl(double* __restrict__ scratch, const cplx* __restrict__ cbar,
     }
     cl.sync();   // Y and Xo are reused by the next knot; the other CTAs have finished reading
   }
-  double* out = scratch + (size_t)wi * N;
+  double* out = W_bar + (size_t)wi * N;
 #pragma unroll
   for (int u = 0; u < kOut; ++u) {
     const int o = threadIdx.x + u * kClThreads;
@@ -503,40 +527,38 @@ cudaError_t launch_fftlog_fwd_df(float4* coef, const double* W, const double* ch
   return fftlog_fwd(coef, W, chipow, D, B, psi, twiddle, n_walk, N_tr, N_I, N, s);
 }
 
+static bool adj_cluster(int n_walk, int N_tr, int N_I, int N) {
+  return N_I <= kKnotChunk && use_cluster((long)n_walk * N_tr, N);
+}
+
 bool fftlog_adj_single_launch(int n_walk, int N_tr, int N_I, int N) {
-  return (N_I + kKnotChunk - 1) / kKnotChunk == 1 && use_cluster((long)n_walk * N_tr, N);
+  return adj_cluster(n_walk, N_tr, N_I, N) || knots_per_cta((long)n_walk * N_tr, N_I) >= N_I;
 }
 
-size_t fftlog_adj_scratch_bytes(int n_walk, int N_tr, int N_I, int N) {
-  int nchunk = (N_I + kKnotChunk - 1) / kKnotChunk;
-  return (size_t)nchunk * n_walk * N_tr * N * sizeof(double);
-}
-
-cudaError_t launch_fftlog_adj(double* W_bar, const cplx* cbar, const double* chipow,
-                              const double* D, const double* B, const cplx* psi,
-                              const cplx* twiddle, int n_walk, int N_tr, int N_I, int N,
-                              double* scratch, cudaStream_t s, int* status, bool pdl) {
-  int nchunk = (N_I + kKnotChunk - 1) / kKnotChunk;
-  if (nchunk == 1 && use_cluster((long)n_walk * N_tr, N)) {
-    // one chunk: the cluster kernel writes W_bar directly
+cudaError_t launch_fftlog_adj(double* W_bar, cplx* cbar, const double* chipow, const double* D,
+                              const double* B, const cplx* psi, const cplx* twiddle, int n_walk,
+                              int N_tr, int N_I, int N, cudaStream_t s, int* status, bool pdl) {
+  if (adj_cluster(n_walk, N_tr, N_I, N)) {
     const size_t csm = (size_t)8 * (N / 2 / kCl) * sizeof(cplx);
     return launch_k(pdl, k_fftlog_adj_cl, dim3((unsigned)((long)n_walk * N_tr * kCl)),
-                    dim3(kClThreads), csm, s, W_bar, cbar, chipow, D, B, psi, twiddle, N_tr, N_I,
+                    dim3(kClThreads), csm, s, W_bar, (const cplx*)cbar, chipow, D, B, psi, twiddle, N_tr, N_I,
                     N, status);
   }
-  size_t smem = (size_t)(N / 2) * 2 * sizeof(cplx) + (size_t)N * sizeof(double);
+  const int kc = knots_per_cta((long)n_walk * N_tr, N_I);
+  const size_t smem = (size_t)(N / 2) * 2 * sizeof(cplx) + (kc > 1 ? (size_t)N * sizeof(double) : 0);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_fftlog_adj, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
   }
+  const int nchunk = (N_I + kc - 1) / kc;
   dim3 g(nchunk, n_walk * N_tr);
-  k_fftlog_adj<<<g, kThreads, smem, s>>>(scratch, cbar, chipow, D, B, psi, twiddle, n_walk, N_tr,
+  k_fftlog_adj<<<g, kThreads, smem, s>>>(W_bar, cbar, kc, status, chipow, D, B, psi, twiddle, n_walk, N_tr,
                                           N_I, N);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  long per = (long)n_walk * N_tr * N;
-  k_sum_chunks<<<(unsigned)((per + 255) / 256), 256, 0, s>>>(W_bar, scratch, per, nchunk, status);
+  if (e != cudaSuccess || nchunk == 1) return e;
+  const long total = (long)n_walk * N_tr * N;
+  k_sum_chunks<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(W_bar, cbar, total, N, N_I, kc, status);
   return cudaGetLastError();
 }
 

@@ -364,12 +364,11 @@ cudaError_t launch_fftlog_fwd_df(float4* coef, const double* W, const double* ch
                                   const cplx* twiddle, int n_walk, int N_tr, int N_I, int N,
                                   cudaStream_t s);
 // adjoint: W_bar[w][i][m] = chipow_i[m] sum_a D_a[m] B_ia[m] Re sum_n conj(psi_n) cbar_n e^{+2pi i n m/N}
-cudaError_t launch_fftlog_adj(double* W_bar, const cplx* cbar, const double* chipow,
+// (cbar is overwritten)
+cudaError_t launch_fftlog_adj(double* W_bar, cplx* cbar, const double* chipow,
                               const double* D, const double* B, const cplx* psi,
                               const cplx* twiddle, int n_walk, int N_tr, int N_I, int N,
-                              double* scratch, cudaStream_t s, int* status = nullptr,
-                              bool pdl = false);
-size_t fftlog_adj_scratch_bytes(int n_walk, int N_tr, int N_I, int N);
+                              cudaStream_t s, int* status = nullptr, bool pdl = false);
 bool fftlog_adj_single_launch(int n_walk, int N_tr, int N_I, int N);   // no chunk reduction
 
 // a3 FP64 contraction (contract_fp64.cu)
