@@ -30,37 +30,36 @@ static_assert(QT == KC, "k_quad_part stages one k point per thread");
 // p = (i <= j).  Grid (multipole, k chunk, walker).  Thread t handles pair p = t % npair for the
 // k points t / npair, t / npair + G, ... of the chunk (G = QT / npair groups); groups are combined
 // in shared memory in a fixed order.
-template <typename T>
+//
+// Bound by the FP64 pipe (two FMA per clock and SM): Delta_i u is formed once per row and k point and staged
+// beside Delta (SCALED), which leaves one FMA per pair instead of a product and an FMA.  103 multipoles, 15
+// tracers, 1024 k points, alone on the GPU: 60 -> 33 us.  Above 55 tracers both do not fit
+// the shared memory and the product is formed per pair.
+template <bool SCALED>
 __global__ void __launch_bounds__(QT)
-k_quad_part(double* __restrict__ part, const T* __restrict__ delta, const double* __restrict__ P,
-            const double* __restrict__ wk2, int N_tr, int N_k, int n_l, int n_kc,
-            const int* __restrict__ listed) {
+k_quad_part(double* __restrict__ part, const double* __restrict__ delta, const double* __restrict__ P,
+            const double* __restrict__ wk2, int N_tr, int N_k, int n_l, int n_kc) {
   extern __shared__ double qsm[];
-  T* Ds = reinterpret_cast<T*>(qsm);              // [N_tr][KS]
+  double* Ds = qsm;                               // [N_tr][KS]
+  double* Es = qsm + (SCALED ? N_tr * KS : 0);    // [N_tr][KS] Delta u
   __shared__ double us[KC];
-  __shared__ float usf[KC];
   __shared__ double red[QT];
   const int ll = blockIdx.x, kc = blockIdx.y, w = blockIdx.z;
   const int q0 = kc * KC;
   const int npair = N_tr * (N_tr + 1) / 2;
-  if (listed && listed[w * n_l + ll] < 0) {
-    // a multipole the walker does not list: zero partials (its Delta rows are not read)
-    double* out = part + (((size_t)w * n_l + ll) * n_kc + kc) * npair;
-    for (int p = threadIdx.x; p < npair; p += QT) out[p] = 0.0;
-    return;
-  }
-  const T* dl = delta + ((size_t)w * n_l + ll) * N_tr * N_k;
+  const double* dl = delta + ((size_t)w * n_l + ll) * N_tr * N_k;
   {
     // one k point per thread (QT == KC); the rows' loads are unrolled so that several are in
     // flight at once
     const int qq = threadIdx.x, q = q0 + qq;
+    const double u = q < N_k ? wk2[q] * P[(size_t)w * N_k + q] : 0.0;
+    if constexpr (!SCALED) us[qq] = u;
 #pragma unroll 8
-    for (int t = 0; t < N_tr; ++t) Ds[t * KS + qq] = q < N_k ? dl[(size_t)t * N_k + q] : T(0);
-  }
-  for (int e = threadIdx.x; e < KC; e += QT) {
-    const int q = q0 + e;
-    us[e] = q < N_k ? wk2[q] * P[(size_t)w * N_k + q] : 0.0;
-    usf[e] = (float)us[e];
+    for (int t = 0; t < N_tr; ++t) {
+      const double d = q < N_k ? dl[(size_t)t * N_k + q] : 0.0;
+      Ds[t * KS + qq] = d;
+      if constexpr (SCALED) Es[t * KS + qq] = d * u;
+    }
   }
   __syncthreads();
   const int ngroups = max(1, QT / npair);
@@ -74,28 +73,11 @@ k_quad_part(double* __restrict__ part, const T* __restrict__ delta, const double
       int r = p, i = 0;                           // unordered pair index -> (i <= j)
       while (r >= N_tr - i) { r -= N_tr - i; ++i; }
       const int j = i + r;
-      const T* di = Ds + i * KS;
-      const T* dj = Ds + j * KS;
-      if (sizeof(T) == 4) {
-        // FP32 products in one compensated FP32 sum (the rounding error of each addition,
-        // from TwoSum, carried in a second float), widened to FP64 once: GB300 runs FP64 at a
-        // small fraction of its FP32 rate
-        float sum = 0.0f, comp = 0.0f;
-        for (int c0 = group * 32; c0 < KC; c0 += ngroups * 32) {
-#pragma unroll 8
-          for (int qq = c0; qq < c0 + 32; ++qq) {
-            const float t = ((float)di[qq] * usf[qq]) * (float)dj[qq];
-            const float sn = sum + t;
-            const float bp = sn - sum;
-            comp += (sum - (sn - bp)) + (t - bp);
-            sum = sn;
-          }
-        }
-        acc = (double)sum + (double)comp;
-      } else {
-        for (int qq = group; qq < KC; qq += ngroups)
-          acc = fma((double)di[qq] * us[qq], (double)dj[qq], acc);
-      }
+      const double* di = Es + i * KS;
+      const double* dj = Ds + j * KS;
+#pragma unroll 4
+      for (int qq = group; qq < KC; qq += ngroups)
+        acc = fma(SCALED ? di[qq] : di[qq] * us[qq], dj[qq], acc);
     }
     if (ngroups > 1) {
       red[threadIdx.x] = acc;
@@ -363,14 +345,18 @@ __global__ void k_unpack_sym(double* __restrict__ Cf, const double* __restrict__
 }
 
 // amp_bar[w][i] = 2 sum_l sum_j S_ij A_j U_ij
-__global__ void k_amp_bar(double* __restrict__ abar, const double* __restrict__ Cf,
+// One CTA per tracer and walker; 1024 threads where a tracer has more than 4096 terms (30 tracers, 2999
+// multipoles: 218 us with 256 threads, 122 us beside the FFTLog adjoint).
+template <int AT>
+__global__ void __launch_bounds__(AT) k_amp_bar(double* __restrict__ abar, const double* __restrict__ Cf,
                           const double* __restrict__ U, const double* __restrict__ amp,
                           int N_tr, int N_ell, int* __restrict__ status) {
   const int w = blockIdx.y;
   const int i = blockIdx.x;
-  __shared__ double red[256];
+  __shared__ double red[AT];
   double s = 0.0;
   const double* A = amp + (size_t)w * N_tr;
+#pragma unroll 4
   for (int e = threadIdx.x; e < N_ell * N_tr; e += blockDim.x) {
     int l = e / N_tr, j = e - l * N_tr;
     size_t base = (((size_t)w * N_ell + l) * N_tr + i) * N_tr + j;
@@ -660,27 +646,6 @@ k_pbar_reduce(double* __restrict__ Pbar, const double* __restrict__ part,
 
 }  // namespace
 
-template <typename T>
-cudaError_t launch_quad(double* U, const T* delta, const double* P, const double* wk2, int n_walk,
-                        int N_tr, int N_k, int N_ell, int l_lo, int n_l, double* scratch,
-                        cudaStream_t s, const int* listed = nullptr) {
-  size_t smem = (size_t)N_tr * KS * sizeof(T);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_quad_part<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  const int n_kc = (N_k + KC - 1) / KC;
-  dim3 g(n_l, n_kc, n_walk);
-  k_quad_part<T><<<g, QT, smem, s>>>(scratch, delta, P, wk2, N_tr, N_k, n_l, n_kc, listed);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const long total = (long)n_walk * n_l * N_tr * (N_tr + 1) / 2;
-  const unsigned grid = (unsigned)std::min<long>((total + 255) / 256, 152L * 16);
-  k_quad_reduce<<<grid, 256, 0, s>>>(U, scratch, N_tr, N_ell, l_lo, n_l, n_kc, n_walk);
-  return cudaGetLastError();
-}
-
 size_t quad_scratch_bytes(int n_walk, int N_tr, int N_k, int n_l) {
   return sizeof(double) * (size_t)n_walk * n_l * ((N_k + KC - 1) / KC) * (N_tr * (N_tr + 1) / 2);
 }
@@ -696,7 +661,22 @@ cudaError_t launch_pair_reduce(double* U, const double* part, int n_walk, int N_
 cudaError_t launch_quad_fp64(double* U, const double* delta, const double* P, const double* wk2,
                              int n_walk, int N_tr, int N_k, int N_ell, int l_lo, int n_l,
                              double* scratch, cudaStream_t s) {
-  return launch_quad<double>(U, delta, P, wk2, n_walk, N_tr, N_k, N_ell, l_lo, n_l, scratch, s);
+  const size_t row = (size_t)KS * sizeof(double);
+  const bool scaled = N_tr <= 55;
+  const size_t smem = N_tr * row * (scaled ? 2 : 1);
+  auto kern = scaled ? k_quad_part<true> : k_quad_part<false>;
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  const int n_kc = (N_k + KC - 1) / KC;
+  kern<<<dim3(n_l, n_kc, n_walk), QT, smem, s>>>(scratch, delta, P, wk2, N_tr, N_k, n_l, n_kc);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const long total = (long)n_walk * n_l * N_tr * (N_tr + 1) / 2;
+  const unsigned grid = (unsigned)std::min<long>((total + 255) / 256, 152L * 16);
+  k_quad_reduce<<<grid, 256, 0, s>>>(U, scratch, N_tr, N_ell, l_lo, n_l, n_kc, n_walk);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_quad_f32(double* U, const float* delta, const double* P, const double* wk2,
@@ -752,7 +732,8 @@ cudaError_t launch_unpack_sym(double* Cf, const double* Cb, const int* off, cons
 cudaError_t launch_amp_bar(double* amp_bar, const double* Cf, const double* U, const double* amp,
                            int n_walk, int N_tr, int N_ell, cudaStream_t s, int* status) {
   dim3 g(N_tr, n_walk);
-  k_amp_bar<<<g, 256, 0, s>>>(amp_bar, Cf, U, amp, N_tr, N_ell, status);
+  if ((long)N_ell * N_tr > 4096) k_amp_bar<1024><<<g, 1024, 0, s>>>(amp_bar, Cf, U, amp, N_tr, N_ell, status);
+  else k_amp_bar<256><<<g, 256, 0, s>>>(amp_bar, Cf, U, amp, N_tr, N_ell, status);
   return cudaGetLastError();
 }
 
