@@ -30,7 +30,7 @@ constexpr int MAXR = 9;   // pairs per thread: ceil(64 * 65 / 2 / 256)
 // Bound by the FP64 pipe.  With Z_i = wk2 (P' Delta_i / 2 + P Delta'_i) the sum is
 // Z_i Delta_j + Delta_i Z_j: two operations per row and two per pair and k point, instead of five per
 // pair with the three products formed apart.  103 multipoles, 8 tangents, 15 tracers, 1024 k:
-// 1157 us before, 556 us now.
+// 1157 us before, 476 us now (553 us with wk2 P'/2 and wk2 P formed again for every tracer).
 template <typename T>
 __global__ void __launch_bounds__(JT)
 k_quad_jvp(double* __restrict__ dU, const T* __restrict__ delta, const double* __restrict__ P,
