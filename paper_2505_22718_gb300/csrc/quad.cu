@@ -8,9 +8,9 @@
 // The unit-amplitude spectra U of the FP64 form are formed in two passes: partial sums of each
 // unordered pair (i <= j) over chunks of 256 k points (one CTA per multipole and chunk), then the
 // chunks added in a fixed order and written to both (i,j) and (j,i), so C is symmetric bit for
-// bit and the same from run to run.  Delta in FP32 (mixed paths) goes through k_quad_blocks
-// below: FP32 products, compensated FP32 sums (TwoSum; the rounding of each addition carried in
-// a second float), FP64 above them, in one pass when a multipole's k range fits one CTA.
+// bit and the same from run to run.  Delta in FP32 (mixed paths) goes through k_quad_blocks or
+// k_quad_stream below: FP32 products, compensated FP32 sums (TwoSum; the rounding of each addition carried in
+// a second float), FP64 above them.
 #include <algorithm>
 
 #include "f32x2.cuh"
@@ -117,20 +117,25 @@ __global__ void k_quad_reduce(double* __restrict__ U, const double* __restrict__
 
 // ---- FP32 form: register blocks of 4 x 4 tracer pairs ----
 //
-// One CTA per (multipole, k chunk, walker) copies the chunk's Delta rows into shared memory as
-// they lie in global memory ([tracer][k], rows padded to a multiple of four tracers with zeros)
-// with asynchronous 16-byte copies, all in flight at once, and u = wk2 P in FP32.  Warp b takes
+// Delta rows lie in shared memory as in global memory ([tracer][k], rows padded to a multiple of four
+// tracers with zeros), brought by asynchronous 16-byte copies, and u = wk2 P in FP32.  A warp takes
 // the block of pairs (4 ib .. 4 ib + 3) x (4 jb .. 4 jb + 3), ib <= jb; lane l takes the k points
 // l, l + 32, ... (consecutive lanes read consecutive words: no bank conflicts).  Per k point a lane
-// forms a_i = Delta_i u (four products, rounded as in the two-pass form) and sixteen FMAs a_i
-// Delta_j into block sums; every QB_GROUP points the block sums are added into compensated
-// (TwoSum) accumulators.  The 32 lanes are then combined by a butterfly that halves the pairs
-// each lane holds at every step (each combination a TwoSum), so lane pair (2p, 2p + 1) ends with
-// pair p of the block.  The order of every addition is fixed: the result is the same from run to
-// run.  With one chunk the sum, widened to FP64, is U itself (both triangles); with several, the
-// per-chunk sums go through the chunk reduction of the other form.
-constexpr int QB_MAX_WARPS = 20;
-constexpr int QB_GROUP = 4;                  // k points per lane between compensated additions
+// forms a_i = Delta_i u (four products, rounded as in the two-pass form) and sixteen products a_i Delta_j;
+// after every four points the block sums go into compensated (TwoSum) accumulators.  The 32 lanes are
+// then combined by a butterfly that halves the pairs each lane holds at every step (each combination a
+// TwoSum), so lane pair (2p, 2p + 1) ends with pair p of the block.  The order of every addition is
+// fixed: the result is the same from run to run.
+//
+// Two kernels.  k_quad_blocks: one CTA per (multipole, k chunk, walker) with all its copies in flight at
+// once; with one chunk the sum, widened to FP64, is U itself (both triangles); with several, the
+// per-chunk sums go through the chunk reduction of the FP64 form.  k_quad_stream, where many rows of more
+// than ten blocks need several chunks each: resident CTAs that stream the rows through a ring of stages,
+// so that the next rows arrive while a block is summed, combined and written, and the lanes are combined
+// once per row instead of once per chunk.  30 tracers, 2999 multipoles, 4096 k: 1842 us and 80 us for the
+// chunk reduction with one CTA per row and chunk, 1494 us so.  Packed FP32 (two points per instruction)
+// took as long and spilled; 30 warps with 64 registers instead of 20 with 96 took 2460 us.
+constexpr int QB_MAX_WARPS = 20;             // per SM, 96 registers each
 constexpr int QB_SMEM = 100 * 1024;          // staged rows per CTA at most (2 CTAs per SM)
 
 __device__ __forceinline__ void qb_two_sum(float& s, float& c, float b) {
@@ -165,6 +170,45 @@ __device__ __forceinline__ void qb_scatter_step(float* s, float* c, int lane) {
   }
 }
 
+// One group of up to 128 k points of a block: n = 64 or 128; ra, rb and ru are at this lane's first point
+__device__ __forceinline__ void qb_group(float* s, float* c, const float* ra, const float* rb, const float* ru,
+                                         int pitch, int n) {
+  float bs[16];
+#pragma unroll
+  for (int k = 0; k < 128; k += 32) {
+    if (k == 64 && n <= 64) break;
+    const float u = ru[k];
+    float ai[4], dj[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      ai[x] = ra[x * pitch + k] * u;
+      dj[x] = rb[x * pitch + k];
+    }
+#pragma unroll
+    for (int p = 0; p < 16; ++p) bs[p] = k == 0 ? ai[p >> 2] * dj[p & 3] : fmaf(ai[p >> 2], dj[p & 3], bs[p]);
+  }
+#pragma unroll
+  for (int p = 0; p < 16; ++p) qb_two_sum(s[p], c[p], bs[p]);
+}
+
+// The 32 lanes' sums of a block's sixteen pairs -> pair lane / 2
+__device__ __forceinline__ float2 qb_lanes(float* s, float* c, int lane) {
+  qb_scatter_step<8, 16>(s, c, lane);
+  qb_scatter_step<4, 8>(s, c, lane);
+  qb_scatter_step<2, 4>(s, c, lane);
+  qb_scatter_step<1, 2>(s, c, lane);
+  const float os = __shfl_xor_sync(0xffffffffu, s[0], 1), oc = __shfl_xor_sync(0xffffffffu, c[0], 1);
+  qb_combine(s[0], c[0], os, oc);
+  return make_float2(s[0], c[0]);
+}
+
+// block b -> (ib <= jb)
+__device__ __forceinline__ void qb_block(int b, int n_ib, int& ib, int& jb) {
+  ib = 0;
+  while (b >= n_ib - ib) { b -= n_ib - ib; ++ib; }
+  jb = ib + b;
+}
+
 __global__ void __launch_bounds__(QB_MAX_WARPS * 32, 1)
 k_quad_blocks(double* __restrict__ U, double* __restrict__ part, const float* __restrict__ delta,
               const double* __restrict__ P, const double* __restrict__ wk2, int N_tr, int N_k,
@@ -177,7 +221,7 @@ k_quad_blocks(double* __restrict__ U, double* __restrict__ part, const float* __
   const int npair = N_tr * (N_tr + 1) / 2;
   const int q0 = kc * kcap;
   const int nk = min(kcap, N_k - q0);
-  const int nk32 = (nk + 31) & ~31;
+  const int nk64 = (nk + 63) & ~63;
   double* Uw = U + ((size_t)w * N_ell + l_lo + ll) * N_tr * N_tr;
   double* pw = part + (((size_t)w * n_l + ll) * n_kc + kc) * npair;
   if (listed && listed[w * n_l + ll] < 0) {
@@ -195,7 +239,7 @@ k_quad_blocks(double* __restrict__ U, double* __restrict__ part, const float* __
   if (vec4) {
     // rows start on 16-byte boundaries (N_k and q0 multiples of 4): 16-byte copies, the part of
     // a group past the chunk's end (and every padding row) filled with zeros by the copy itself
-    const int ng = nk32 >> 2;
+    const int ng = nk64 >> 2;
     for (int e = threadIdx.x; e < rows * ng; e += blockDim.x) {
       const int t = e / ng, gq = e - t * ng;
       const int left = nk - 4 * gq;
@@ -206,8 +250,8 @@ k_quad_blocks(double* __restrict__ U, double* __restrict__ part, const float* __
                    "r"(bytes) : "memory");
     }
   } else {
-    for (int e = threadIdx.x; e < rows * nk32; e += blockDim.x) {
-      const int t = e / nk32, kk = e - t * nk32;
+    for (int e = threadIdx.x; e < rows * nk64; e += blockDim.x) {
+      const int t = e / nk64, kk = e - t * nk64;
       const int bytes = t < N_tr && kk < nk ? 4 : 0;
       const float* src = bytes ? dl + (size_t)t * N_k + kk : dl;
       const unsigned dst = (unsigned)__cvta_generic_to_shared(Ds + (size_t)t * kcap + kk);
@@ -216,63 +260,36 @@ k_quad_blocks(double* __restrict__ U, double* __restrict__ part, const float* __
     }
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
-  for (int kk = threadIdx.x; kk < nk32; kk += blockDim.x)
+  for (int kk = threadIdx.x; kk < nk64; kk += blockDim.x)
     us[kk] = kk < nk ? (float)(wk2[q0 + kk] * P[(size_t)w * N_k + q0 + kk]) : 0.0f;
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
   // warp wi: k part h = wi / wb of ks, blocks bw, bw + wb, ... (bw = wi % wb); part h takes the
-  // 32-point groups [h n32 / ks, (h + 1) n32 / ks) of the chunk
+  // 64-point groups [h n64 / ks, (h + 1) n64 / ks) of the chunk
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const int wb = (blockDim.x >> 5) / ks, h = wi / wb, bw = wi - h * wb;
-  const int n32 = nk32 >> 5;
-  const int k_lo = 32 * (h * n32 / ks), k_hi = 32 * ((h + 1) * n32 / ks);
+  const int n64 = nk64 >> 6;
+  const int k_lo = 64 * (h * n64 / ks), k_hi = 64 * ((h + 1) * n64 / ks);
   float2* red = reinterpret_cast<float2*>(us + kcap);         // [ks][nb][16] (sum, compensation)
   for (int b = bw; b < nb && h < ks; b += wb) {
-    int ib = 0, r = b;                                          // block b -> (ib <= jb)
-    while (r >= n_ib - ib) { r -= n_ib - ib; ++ib; }
-    const int jb = ib + r;
-    const float* ra = Ds + (size_t)(4 * ib) * kcap;
-    const float* rb = Ds + (size_t)(4 * jb) * kcap;
-    float s[16], c[16];
+    int ib, jb;
+    qb_block(b, n_ib, ib, jb);
+    const float* ra = Ds + (size_t)(4 * ib) * kcap + lane;
+    const float* rb = Ds + (size_t)(4 * jb) * kcap + lane;
+    const float* ru = us + lane;
+    float s2[16], c2[16];
 #pragma unroll
-    for (int p = 0; p < 16; ++p) s[p] = c[p] = 0.0f;
-    for (int g0 = k_lo; g0 < k_hi; g0 += 32 * QB_GROUP) {
-      float bs[16];
-#pragma unroll
-      for (int p = 0; p < 16; ++p) bs[p] = 0.0f;
-      const int g1 = min(k_hi, g0 + 32 * QB_GROUP);
-#pragma unroll 2
-      for (int kk = g0 + lane; kk < g1; kk += 32) {
-        const float u = us[kk];
-        float ai[4], dj[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          ai[x] = ra[(size_t)x * kcap + kk] * u;
-          dj[x] = rb[(size_t)x * kcap + kk];
-        }
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-          for (int y = 0; y < 4; ++y) bs[4 * x + y] = fmaf(ai[x], dj[y], bs[4 * x + y]);
-      }
-#pragma unroll
-      for (int p = 0; p < 16; ++p) qb_two_sum(s[p], c[p], bs[p]);
-    }
-    qb_scatter_step<8, 16>(s, c, lane);
-    qb_scatter_step<4, 8>(s, c, lane);
-    qb_scatter_step<2, 4>(s, c, lane);
-    qb_scatter_step<1, 2>(s, c, lane);
-    qb_combine(s[0], c[0], __shfl_xor_sync(0xffffffffu, s[0], 1),
-               __shfl_xor_sync(0xffffffffu, c[0], 1));
-    if (!(lane & 1)) red[((size_t)h * nb + b) * 16 + (lane >> 1)] = make_float2(s[0], c[0]);
+    for (int p = 0; p < 16; ++p) s2[p] = c2[p] = 0.0f;
+    for (int g0 = k_lo; g0 < k_hi; g0 += 128) qb_group(s2, c2, ra + g0, rb + g0, ru + g0, kcap, k_hi - g0);
+    const float2 t = qb_lanes(s2, c2, lane);
+    if (!(lane & 1)) red[((size_t)h * nb + b) * 16 + (lane >> 1)] = t;
   }
   __syncthreads();
   // the k parts of each pair, added in order; pair p of block b is (4 ib + p / 4, 4 jb + p % 4)
   for (int e = threadIdx.x; e < nb * 16; e += blockDim.x) {
     const int b = e >> 4, p = e & 15;
-    int ib = 0, r = b;
-    while (r >= n_ib - ib) { r -= n_ib - ib; ++ib; }
-    const int jb = ib + r;
+    int ib, jb;
+    qb_block(b, n_ib, ib, jb);
     const int i = 4 * ib + (p >> 2), j = 4 * jb + (p & 3);
     if (i >= N_tr || j >= N_tr || i > j) continue;
     float2 t = red[e];
@@ -286,6 +303,102 @@ k_quad_blocks(double* __restrict__ U, double* __restrict__ part, const float* __
       Uw[j * N_tr + i] = v;
     } else {
       pw[i * N_tr - i * (i - 1) / 2 + (j - i)] = v;
+    }
+  }
+}
+
+// Items (walker, multipole, part of the blocks), an equal share of consecutive ones per CTA.  A part's
+// blocks have a warp each; their accumulators live over all the k points of a row.
+constexpr int QS_RING = 4;                   // stages; three are in flight while one is summed
+constexpr int QS_MAX_K = 8192;               // u of all k points stays in shared memory
+__global__ void __launch_bounds__(QB_MAX_WARPS * 32, 1)
+k_quad_stream(double* __restrict__ U, const float* __restrict__ delta, const double* __restrict__ P,
+              const double* __restrict__ wk2, int N_tr, int N_k, int N_ell, int l_lo, int n_l, int n_walk,
+              int n_part, int nbp, int lg_sk, bool vec4) {
+  extern __shared__ float4 qb_smv[];
+  const int n_ib = (N_tr + 3) / 4, nb = n_ib * (n_ib + 1) / 2, rows = 4 * n_ib;
+  const int sk = 1 << lg_sk, n_st = (N_k + sk - 1) >> lg_sk, nk64 = (N_k + 63) & ~63;
+  float* ring = reinterpret_cast<float*>(qb_smv);               // [QS_RING][rows][sk]
+  float* us = ring + (size_t)QS_RING * rows * sk;               // [nk64]
+  const int lane = threadIdx.x & 31, bw = threadIdx.x >> 5;
+  const long n_item = (long)n_walk * n_l * n_part;
+  const int it0 = (int)(n_item * blockIdx.x / gridDim.x), it1 = (int)(n_item * (blockIdx.x + 1) / gridDim.x);
+  // the producer's place: stage pst of item pit
+  int pit = it0, pst = 0, slot = 0;
+  auto issue = [&](int to) {
+    if (pit < it1) {
+      const int k0 = pst << lg_sk, ns = min(sk, nk64 - k0);
+      const float* dl = delta + (size_t)(pit / n_part) * N_tr * N_k;
+      float* st = ring + (size_t)to * rows * sk;
+      if (vec4) {
+        for (int e = threadIdx.x; e < rows << (lg_sk - 2); e += blockDim.x) {
+          const int t = e >> (lg_sk - 2), kk = (e & ((sk >> 2) - 1)) << 2, left = N_k - k0 - kk;
+          if (kk >= ns) continue;
+          const int bytes = t < N_tr && left > 0 ? 16 : 0;      // N_k is a multiple of 4
+          const float* src = bytes ? dl + (size_t)t * N_k + k0 + kk : dl;
+          const unsigned dst = (unsigned)__cvta_generic_to_shared(st + (t << lg_sk) + kk);
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src),
+                       "r"(bytes) : "memory");
+        }
+      } else {
+        for (int e = threadIdx.x; e < rows << lg_sk; e += blockDim.x) {
+          const int t = e >> lg_sk, kk = e & (sk - 1);
+          if (kk >= ns) continue;
+          const int bytes = t < N_tr && k0 + kk < N_k ? 4 : 0;
+          const float* src = bytes ? dl + (size_t)t * N_k + k0 + kk : dl;
+          const unsigned dst = (unsigned)__cvta_generic_to_shared(st + (t << lg_sk) + kk);
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(dst), "l"(src),
+                       "r"(bytes) : "memory");
+        }
+      }
+      if (++pst == n_st) {
+        pst = 0;
+        ++pit;
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");   // empty past the end: the count goes on
+  };
+#pragma unroll
+  for (int x = 0; x < QS_RING - 1; ++x) issue(x);
+  int cur_w = -1;
+  for (int it = it0; it < it1; ++it) {
+    const int wl = it / n_part, part = it - wl * n_part, w = wl / n_l, ll = wl - w * n_l;
+    double* Uw = U + ((size_t)w * N_ell + l_lo + ll) * N_tr * N_tr;
+    if (w != cur_w) {
+      __syncthreads();   // the sums of the walker before have read us
+      for (int q = threadIdx.x; q < nk64; q += blockDim.x)
+        us[q] = q < N_k ? (float)(wk2[q] * P[(size_t)w * N_k + q]) : 0.0f;
+      cur_w = w;
+    }
+    const int b = part * nbp + bw;
+    const bool work = b < nb;
+    int ib, jb;
+    qb_block(work ? b : 0, n_ib, ib, jb);
+    const int oa = ((4 * ib) << lg_sk) + lane, ob = ((4 * jb) << lg_sk) + lane;
+    float s2[16], c2[16];
+#pragma unroll
+    for (int p = 0; p < 16; ++p) s2[p] = c2[p] = 0.0f;
+    for (int st = 0; st < n_st; ++st) {
+      // this stage has arrived, and every warp is done with the one before, whose place is free
+      asm volatile("cp.async.wait_group %0;\n" ::"n"(QS_RING - 2) : "memory");
+      __syncthreads();
+      issue(slot == 0 ? QS_RING - 1 : slot - 1);
+      const float* d = ring + (size_t)slot * rows * sk;
+      slot = slot + 1 == QS_RING ? 0 : slot + 1;
+      if (!work) continue;
+      const int k0 = st << lg_sk, ns = min(sk, nk64 - k0);
+      const float* ru = us + k0 + lane;
+      for (int g0 = 0; g0 < ns; g0 += 128) qb_group(s2, c2, d + oa + g0, d + ob + g0, ru + g0, sk, ns - g0);
+    }
+    if (!work) continue;
+    const float2 t = qb_lanes(s2, c2, lane);
+    if (!(lane & 1)) {
+      const int p = lane >> 1, i = 4 * ib + (p >> 2), j = 4 * jb + (p & 3);
+      if (i <= j && j < N_tr) {
+        const double v = (double)t.x + (double)t.y;
+        Uw[i * N_tr + j] = v;
+        Uw[j * N_tr + i] = v;
+      }
     }
   }
 }
@@ -684,18 +797,36 @@ cudaError_t launch_quad_f32(double* U, const float* delta, const double* P, cons
                             double* scratch, cudaStream_t s, const int* listed) {
   if (n_walk <= 0 || n_l <= 0) return cudaSuccess;
   const int n_ib = (N_tr + 3) / 4, nb = n_ib * (n_ib + 1) / 2;
+  const bool vec4 = N_k % 4 == 0 && ((uintptr_t)delta & 15) == 0;
+  const long n_row = (long)n_walk * n_l;
   // k parts per block: with few CTAs (one walker), enough warps per CTA to hide the shared-load
   // and FMA latencies; with many, one part (each further part repeats the lane combination)
-  const long n_cta0 = (long)n_walk * n_l * ((N_k + 1023) / 1024);
+  const long n_cta0 = (long)n_walk * N_ell * ((N_k + 1023) / 1024);
   const int ks = n_cta0 >= 2 * 152 ? 1 : std::max(1, std::min(4, QB_MAX_WARPS / nb));
   const int warps = ks * std::min(nb, QB_MAX_WARPS / ks);
   const size_t red_bytes = sizeof(float2) * (size_t)ks * nb * 16;
   // k points per CTA: the largest power of two up to 1024 whose rows fit QB_SMEM
   int kcap = 1024;
-  while (kcap > 32 && (size_t)kcap * (16 * n_ib + 4) + red_bytes > (size_t)QB_SMEM) kcap >>= 1;
+  while (kcap > 64 && (size_t)kcap * (16 * n_ib + 4) + red_bytes > (size_t)QB_SMEM) kcap >>= 1;
   const int n_kc = (N_k + kcap - 1) / kcap;
   const size_t smem = (size_t)kcap * (16 * n_ib + 4) + red_bytes;
-  const bool vec4 = N_k % 4 == 0 && ((uintptr_t)delta & 15) == 0;
+  // A stream of rows: from two rows per SM on (by all the multipoles, so that a launch over a part of them
+  // sums in the same order), where the other form needs several chunks per row and more blocks than half
+  // the warps.  Its equal shares want equal rows: ragged lists stay with the CTAs per row, which the
+  // hardware hands out.  More than twenty blocks go in parts (each reads the rows again, from L2); stages
+  // of up to 32 KB keep 100 KB in flight per SM.
+  if ((long)n_walk * N_ell >= 2 * 152 && !listed && n_kc > 1 && nb > QB_MAX_WARPS / 2 && N_k <= QS_MAX_K &&
+      n_row * nb < (1L << 31)) {
+    const int n_part = (nb + QB_MAX_WARPS - 1) / QB_MAX_WARPS, nbp = (nb + n_part - 1) / n_part;
+    int lg_sk = 7;
+    while (lg_sk < 10 && (size_t)(4 * n_ib) * (8 << lg_sk) <= 32 * 1024) ++lg_sk;
+    const size_t ring = sizeof(float) * ((size_t)QS_RING * (4 * n_ib) * (1 << lg_sk) + ((N_k + 63) & ~63));
+    cudaError_t e = cudaFuncSetAttribute(k_quad_stream, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
+    if (e != cudaSuccess) return e;
+    k_quad_stream<<<(unsigned)std::min<long>(n_row * n_part, 152), nbp * 32, ring, s>>>(
+        U, delta, P, wk2, N_tr, N_k, N_ell, l_lo, n_l, n_walk, n_part, nbp, lg_sk, vec4);
+    return cudaGetLastError();
+  }
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_quad_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
