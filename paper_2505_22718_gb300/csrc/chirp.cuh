@@ -20,16 +20,16 @@
 // is at most M/2 in the HALF form: half of the first pass's inputs are then zero and half of the
 // last pass's outputs unused.
 //
-// FP64: bound by the FP64 pipe (two FMA per clock and SM): about 1160 FP64 instructions per thread and
+// FP64: bound by the FP64 pipe (two FMA per clock and SM): about 1080 FP64 instructions per thread and
 // row of 2048 points, so the largest radix whose points fit the registers (fewest twiddle products)
-// and eight resident warps are enough.  15 tracers x 103 multipoles, N = 2048, N_k = 1024: 484 us
-// forward and 463 us transposed (75 % of the pipe's rate; the last of six turns of two CTAs per SM is
+// and eight resident warps are enough.  15 tracers x 103 multipoles, N = 2048, N_k = 1024: 459 us
+// forward and 440 us transposed (75 % of the pipe's rate; the last of six turns of two CTAs per SM is
 // nearly empty), against 5.9 ms each for the direct sums.
 //
 // FP32: bound by shared-memory and table accesses (1750 wavefronts of the load/store pipe per row of
 // 2048 points) and, close behind, by instruction issue: about 2070 clocks per row and SM with four
 // resident CTAs (16 warps).  1545 such rows 19 us forward and 20 us transposed; 287 100 rows (256 walkers
-// with ragged lists) 1.95 and 1.88 ms; 89 970 rows of 8192 points 3.84 and 3.34 ms.  The GEMMs over all
+// with ragged lists) 1.89 and 1.85 ms; 89 970 rows of 8192 points 3.78 and 3.28 ms.  The GEMMs over all
 // frequencies took 56 and 58 us, 7.9 and 12.3 ms, 14.6 and 11.9 ms, with another 23 us, 1.7 ms and
 // 1.5 ms for their operand images.  Errors against 64 bits (N5K shape): Delta 1.3e-7 (GEMMs 1.9e-7),
 // normalised C 2.7e-5 (3.1e-5), W_bar 4.2e-7 (9.7e-7); white-noise windows 1.6e-7 (1.4e-7), 5.9e-5
