@@ -32,14 +32,9 @@ int ensure(swcl_ctx* c, DevBuf& b, size_t bytes) {
     return fail(c, SWCL_ERR_OOM_BUDGET,
                 "memory budget exceeded: need " + std::to_string(c->held - freed + bytes) +
                     " bytes, budget " + std::to_string(c->budget));
-  if (b.p) {
-    cudaFree(b.p);
-    c->held -= b.bytes;
-    b.p = nullptr;
-    b.bytes = 0;
-  }
   if (c->capturing)
     return fail(c, SWCL_ERR_STATE, "device buffer would grow during graph capture");
+  release(c, b);
   cudaError_t e = cudaMalloc(&b.p, bytes);
   if (e != cudaSuccess) {
     b.p = nullptr;
@@ -51,10 +46,13 @@ int ensure(swcl_ctx* c, DevBuf& b, size_t bytes) {
   return SWCL_OK;
 }
 
+// A captured graph holds the addresses of the buffers its kernels use, so that freeing any of them
+// makes the captured graphs unusable (alloc_gen), whether or not another buffer takes its place.
 void release(swcl_ctx* c, DevBuf& b) {
   if (b.p) {
     cudaFree(b.p);
     c->held -= b.bytes;
+    ++c->alloc_gen;
   }
   b.p = nullptr;
   b.bytes = 0;
@@ -804,7 +802,7 @@ static int plan_chunk(swcl_ctx* c, int precision, int n_need, int& n_lc) {
   if (n_lc == 0 && swcl::chirp_use(c, precision)) {
     n_lc = plan_ell_chunk(c, precision, n_need, false);
     if (n_lc == 0) {
-      swcl::chirp_drop(c);
+      SWCL_TRY(swcl::chirp_drop(c));
       n_lc = plan_ell_chunk(c, precision, n_need, true);
     }
   }

@@ -79,7 +79,8 @@ bool chirp_use(const swcl_ctx* c, int precision) {
   return c->N >= 1024;
 }
 
-void chirp_drop(swcl_ctx* c) {
+int chirp_drop(swcl_ctx* c) {
+  if (c->capturing) return fail(c, SWCL_ERR_STATE, "chirp tables given up during capture");
   for (auto& p : c->ck)
     for (auto& d : p) {
       release(c, d.tab);
@@ -88,6 +89,7 @@ void chirp_drop(swcl_ctx* c) {
   release(c, c->ws_ckpart);
   c->ck_off = true;
   c->bt_ready = false;
+  return SWCL_OK;
 }
 
 int chirp_prepare(swcl_ctx* c, int precision) {
@@ -105,9 +107,8 @@ int chirp_prepare(swcl_ctx* c, int precision) {
     const int st = ensure(c, d.tab, fp64 ? chirp64_table_bytes(d.logm, n_freq, c->N_k)
                                          : chirp32_table_bytes(d.logm, n_freq, c->N_k));
     if (st == SWCL_ERR_OOM_BUDGET) {   // the direct sums need no tables
-      chirp_drop(c);
       c->err.clear();
-      return SWCL_OK;
+      return chirp_drop(c);
     }
     if (st) return st;
     const int t_lo = dir == 0 ? n_freq - 1 : c->N_k - 1, t_hi = dir == 0 ? c->N_k - 1 : n_freq - 1;

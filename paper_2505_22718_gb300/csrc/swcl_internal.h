@@ -271,7 +271,7 @@ struct swcl_ctx {
     const void* ptrs[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     int64_t alloc_gen = -1;
   } graph_key;
-  int64_t alloc_gen = 0;      // bumped whenever a device buffer is (re)allocated or sizes change
+  int64_t alloc_gen = 0;      // bumped whenever a device buffer is allocated or freed, or sizes change
   bool capturing = false;
   int64_t graph_launches = 0; // kernels in the captured graph
 
@@ -388,7 +388,7 @@ void chirp_fit_grid(swcl_ctx* c);
 bool chirp_use(const swcl_ctx* c, int precision);
 int chirp_rank(const swcl_ctx* c);
 int chirp_prepare(swcl_ctx* c, int precision);      // tables; gives the transforms up on a full budget
-void chirp_drop(swcl_ctx* c);
+int chirp_drop(swcl_ctx* c);                        // frees them; refused during graph capture
 size_t chirp_part_bytes(const swcl_ctx* c, int precision, int n_l, bool whole);
 int chirp_forward(swcl_ctx* c, int precision, int l_lo, int n_l);
 int chirp_adjoint(swcl_ctx* c, int precision, int l_lo, int n_l, bool accumulate);

@@ -1,0 +1,133 @@
+"""The chirp transforms in a context with a memory budget: what happens when their tables or partial
+sums do not fit.  Budgets are found by bisection on fresh contexts, so that they lie within 4 KB of
+where a call begins to fit, whatever the sizes of the buffers are."""
+import numpy as np
+import pytest
+
+from gpu_helpers import lib_context, max_rel
+from workloads.n5k_synth import CHI_MAX, CHI_MIN, Cosmology, Workload, clustering_window, ell_list, power_spectrum
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__ as g
+    g.build()
+
+
+def _case(N, n_k, n_ell, n_tr=3, n_walk=1, seed=2):
+    rng = np.random.default_rng(seed)
+    cosmo = Cosmology()
+    chi = CHI_MIN * np.exp(np.arange(N) * np.log(CHI_MAX / CHI_MIN) / N)
+    z = cosmo.z_of_chi(chi)
+    W = np.array([clustering_window(cosmo, chi, m, 0.2, z) for m in np.linspace(0.4, 1.2, n_tr)])
+    W = W * rng.uniform(0.8, 1.2, (n_walk, n_tr, 1))
+    k = np.geomspace(1e-4, 8.0, n_k)
+    knots = np.geomspace(1e-4, 8.0, 12)
+    D = (1.0 / (1.0 + z))[None, :] * (1.0 + 0.02 * np.log(knots / 0.1))[:, None]
+    P = power_spectrum(k, 3.5e6) * rng.uniform(0.9, 1.1, (n_walk, 1))
+    w = Workload("budget", N, CHI_MIN, CHI_MAX, k, ell_list(2, 900, n_ell), knots, np.zeros(n_tr, np.int32),
+                 np.full(n_tr, -0.3), W, D, None, P, rng.uniform(1.0, 2.0, (n_walk, n_tr)))
+    return w, rng
+
+
+class _Step:
+    """swcl_compute_batched (a captured graph) into its own device arrays."""
+
+    def __init__(self, w, seed=4):
+        import torch
+        n_walk, n_tr, _ = w.W.shape
+        self.Cb = torch.tensor(np.random.default_rng(seed).standard_normal((n_walk * len(w.ells), n_tr, n_tr)), device="cuda")
+        self.out = [torch.zeros_like(self.Cb)] + [torch.zeros(a.shape, dtype=torch.float64, device="cuda")
+                                                  for a in (w.P, w.amp, w.W)]
+
+    def __call__(self, ctx, precision):
+        import paper_2505_22718_gb300 as S
+        for t in self.out:
+            t.zero_()
+        import torch
+        torch.cuda.synchronize()
+        S.swcl_compute_batched(ctx.ptr, precision, self.out[0], self.Cb, *self.out[1:])
+        ctx.sync()
+        return [t.cpu().numpy() for t in self.out]
+
+
+def _over_budget(call):
+    """Whether call() was refused for the memory budget (any other error is raised)."""
+    import paper_2505_22718_gb300 as S
+    try:
+        call()
+    except S.SwiftClError as e:
+        assert "budget" in str(e)
+        return True
+    return False
+
+
+def _context(w, budget):
+    """A context, or None where its inputs and tables alone exceed the budget."""
+    got = []
+    return None if _over_budget(lambda: got.append(lib_context(w, budget=budget))) else got[0]
+
+
+def _smallest_budget(fits, hi):
+    """The smallest budget, to 4 KB, for which fits(budget) holds (it holds for hi)."""
+    assert fits(hi)
+    lo = 0
+    while hi - lo > 4096:
+        mid = (lo + hi) // 2
+        if fits(mid):
+            hi = mid
+        else:
+            lo = mid
+    return hi
+
+
+def _same(a, b, tol):
+    for x, y in zip(a, b):
+        assert max_rel(x, y) < tol
+
+
+def test_graph_after_the_tables_were_freed():
+    """A batched FP64 step captured with the chirp transforms; then a forward-mode call that fits the
+    budget only without their tables (they are freed), or does not fit at all; then the step
+    again: it must not replay the graph that holds the freed addresses.  FP64 results by either route
+    agree to 1e-10 (the gate of the FP64 path)."""
+    import paper_2505_22718_gb300 as S
+    w, rng = _case(512, 400, 40)
+    step, W_dot = _Step(w), rng.standard_normal((8,) + w.W.shape[1:]) * w.W[0]
+    free = lib_context(w)
+    want = step(free, S.SWCL_FP64)
+    J = free.jvp(W_dot=W_dot)
+    most = free.query(S.SWCL_Q_WORKSPACE_BYTES)
+    free.close()
+
+    def run(budget, check):
+        """None (the step does not fit), else whether the JVP fits"""
+        ctx = _context(w, budget)
+        if ctx is None:
+            return None
+        try:
+            if not check and _over_budget(lambda: step(ctx, S.SWCL_FP64)):
+                return None
+            if check:
+                for _ in range(2):
+                    _same(step(ctx, S.SWCL_FP64), want, 1e-10)
+            S.swcl_profile_enable(ctx.ptr, True)
+            got = []
+            fits = not _over_budget(lambda: got.append(ctx.jvp(W_dot=W_dot)))
+            names = set(S.swcl_profile_read(ctx.ptr))
+            S.swcl_profile_enable(ctx.ptr, False)
+            if check:
+                if fits:
+                    assert max_rel(got[0], J) < 1e-10 and "contract fp64" in names   # the tables were given up
+                for _ in range(2):
+                    _same(step(ctx, S.SWCL_FP64), want, 1e-10)
+                assert ctx.query(S.SWCL_Q_WORKSPACE_BYTES) <= budget
+            return fits
+        finally:
+            ctx.close()
+
+    b = _smallest_budget(lambda x: bool(run(x, False)), most + (64 << 20))
+    assert run(b, True) is True
+    assert run(b - 65536, True) is False
