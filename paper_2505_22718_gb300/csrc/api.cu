@@ -1088,6 +1088,11 @@ int swcl_vjp(swcl_ctx* c, int precision, const double* C_bar, double* P_bar, dou
                                                        ? (const int*)c->bt_lpos.p : nullptr,
                                                    c->pdl && !c->prof),
                   "delta_bar f32");
+    if (fork && l_lo + n_l == n_fft) {
+      // P_bar's reduction waits for the last delta_bar only
+      SWCL_TRY_CUDA(c, cudaEventRecord(c->ev_fork, c->stream), "fork");
+      SWCL_TRY_CUDA(c, cudaStreamWaitEvent(c->aux, c->ev_fork, 0), "fork");
+    }
     if (!W_bar) continue;
     if (fp64 && swcl::chirp_use(c, precision)) {
       SWCL_TRY(swcl::chirp_adjoint(c, precision, l_lo, n_l, accumulate));
@@ -1105,11 +1110,6 @@ int swcl_vjp(swcl_ctx* c, int precision, const double* C_bar, double* P_bar, dou
     } else {
       SWCL_TRY(swcl::contract_adj_tc(c, precision));   // whole multipole range (no chunks)
     }
-  }
-  if (fork) {
-    // the reduction waits for the last delta_bar chunk (main stream)
-    SWCL_TRY_CUDA(c, cudaEventRecord(c->ev_fork, c->stream), "fork");
-    SWCL_TRY_CUDA(c, cudaStreamWaitEvent(c->aux, c->ev_fork, 0), "fork");
   }
   SWCL_LAUNCH(c, swcl::launch_pbar_reduce(Pb, (const double*)c->ws_pbpart.p,
                                           (const double*)c->d_wk2.p, nw, N_k, n_fft, side,
