@@ -375,7 +375,7 @@ int swcl_destroy(swcl_ctx* c) {
                     &c->bt_g32, &c->bt_kmu, &c->bt_himg, &c->bt_dimg, &c->ws_qpart, &c->bt_cmap_f,
                     &c->bt_cmap_a, &c->bt_lpos, &c->bt_wbase,
                     &c->ws_jin, &c->ws_dU, &c->ws_jout, &c->ws_fz, &c->ws_fsmall, &c->ws_lq,
-                    &c->ws_ltab, &c->ws_ckpart, &c->hs_C, &c->hs_Cb, &c->hs_Pb, &c->hs_Ab, &c->hs_Wb};
+                    &c->ws_ltab, &c->ws_ckpart, &c->ck_head, &c->hs_C, &c->hs_Cb, &c->hs_Pb, &c->hs_Ab, &c->hs_Wb};
   for (DevBuf* b : bufs) swcl::release(c, *b);
   for (auto& p : c->ck)
     for (auto& d : p) swcl::release(c, d.tab);

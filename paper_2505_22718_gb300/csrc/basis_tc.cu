@@ -16,7 +16,7 @@
 //   A[2n][q] = Re E, A[2n+1][q] = -Im E;  B[j][q] = kpow mu Dbar;
 // its epilogue multiplies by conj(G) and sums over l.
 //
-// On k grids uniform in ln k (from N = 1024 on) only the frequencies n < 64 take the forward GEMM, and
+// On k grids uniform in ln k (from N = 1024 on) only the lowest 64 to 256 frequencies take the forward GEMM, and
 // the rest of the sum and its whole transpose the FP32 chirp transforms (chirp.cuh).
 //
 // Compensated products with FP32 accumulation (the 5th-generation tensor cores take bf16 operands
@@ -34,6 +34,7 @@
 // warps per 32-lane quarter, each with half of the columns) and run the epilogue.  All waits are bounded; a timeout raises
 // the context's status word (SWCL_ERR_TIMEOUT).
 #include <algorithm>
+#include <type_traits>
 #include <cuda_bf16.h>
 
 #include "swcl_internal.h"
@@ -1778,37 +1779,111 @@ __global__ void __maxnreg__(32) k_dimg(uint8_t* __restrict__ img, const float* _
 
 // ------------------------------------------------------ low frequencies (chirp form) ----
 
-// Delta from the frequencies n < kChirpHead alone, before the chirp transforms add the rest: the same
+// Delta from the lowest frequencies alone, before the chirp transforms add the rest: the same
 // compensated products as the GEMM over all frequencies (two K-blocks per accumulator slot, leading
-// product and corrections apart, the two sums added with round-to-nearest), with K = 128 in all.  With
-// so little K the work is in the operands and the result, so nothing of it passes through memory but
-// Delta itself: a CTA forms H = F G for its 64 columns in shared memory once (the arithmetic of k_himg)
-// and walks its q tiles, streaming their rows of the phase image (96 KB each, from L2) through a ring of
-// six K-blocks; the accumulators are double-buffered in TMEM (4 slots x 64 columns, twice: all 512), so
+// product and corrections apart, the two sums added with round-to-nearest), in rounds of kChirpHead = 64
+// frequencies, K = 128 each.
+//
+// How many rounds a row (walker, tracer) takes follows from its own coefficients.  The rounding errors of
+// the FP32 transform are spread evenly over the k points, in proportion to the root sum of squares of
+// what passes through it, so that they weigh most where Delta is far below its largest value (the
+// largest k).  There the GEMM's sums over all frequencies are better, unless what passes is a small part of
+// the row: the smallest of 64, 128, 192 and 256 frequencies after which at most kHeadRest of the
+// row's root sum of squares is left.  Wide windows take one round, narrow ones at high redshift up to four.
+// P_bar's error against 64 bits with the GEMMs, with one round for every row and so: 30 tracers,
+// sigma_z = 0.03, a bias that grows as k^2, k to 20: 2.6e-7, 9.5e-7, 2.4e-7.  72 shapes (N = 1024 to 4096,
+// sigma_z 0.03 to 0.1, k to 10 and 20, with and without such a bias): 1.54 times the GEMMs' in the
+// geometric mean and 5.5 at most with one round, 0.98 and 2.1 so (0.95 and 1.9 with kHeadRest = 0.1, which
+// gives windows of N5K shape a second round, 45 us instead of 40 us forward).  C 0.997, W_bar 0.46.
+//
+// With so little K the work is in the operands and the result, so nothing of it passes through memory but
+// Delta itself: a CTA forms H = F G of a round for its 64 columns in shared memory (the arithmetic of
+// k_himg) and walks its q tiles, streaming their rows of the phase image (96 KB each, from L2) through a ring
+// of six K-blocks; the accumulators are double-buffered in TMEM (4 slots x 64 columns, twice: all 512), so
 // the epilogue warps scale and store tile t while tile t + 1 multiplies.
-// Bound by the MMA issue (54 clocks per 128 x 64 x 16 product, 48 of them per tile) and, with few
-// columns, by the forming of H.  1545 columns x 1024 k 16 us, 287 100 columns 0.76 ms, 89 970 columns x
-// 4096 k 0.81 ms; the GEMM kernels with their H image took 24 us, 3.6 ms and 1.9 ms for the same K.
+// Bound by the MMA issue (54 clocks per 128 x 64 x 16 product, 48 of them per tile and round) and, with few
+// columns, by the forming of H.  1545 columns x 1024 k 16 us, 287 100 columns 0.80 ms (0.76 ms without the
+// choice of rounds), 89 970 columns x 4096 k 2.0 ms at 1 to 4 rounds a row (0.81 ms with one); the GEMM kernels
+// with their H image took 24 us, 3.6 ms and 1.9 ms for the K of one round.
 // Warps: 0 copies, 1 MMA and TMEM, 2-9 form H, then drain (two warps per 32-lane quarter, 32 columns
-// each) and store.  Columns: each half of a tile holds 32/r whole groups of r profile rows.
+// each) and store, 10-11 find the rounds of the tile's rows during the first one.  Columns: each half of a
+// tile holds 32/r whole groups of r profile rows.
 constexpr int kHeadNT = 64;
-constexpr int kHeadKb = 2 * kChirpHead / kK;               // 4 K-blocks
+constexpr int kHeadKb = 2 * kChirpHead / kK;               // 4 K-blocks a round
+constexpr int kHeadRounds = 4;                             // at most
+constexpr double kHeadRest = 0.2;
 constexpr int kHeadStages = 6;
 constexpr uint32_t kHeadA = kPlanes * kPlaneM;             // one K-block of the phase image
 constexpr uint32_t kHeadB = kPlanes * kHeadNT * kRow;      // one K-block of H
-constexpr int kHeadThreads = 320;
+constexpr int kHeadThreads = 384;
 
 struct HeadShape {
-  int N_k, N_tr, N_ell, n_h, l_lo, n_l, r, NI, n_groups, n_mt, q_per, q_split;
+  int N_k, N_tr, N_ell, n_h, l_lo, n_l, r, NI, n_groups, n_mt, f_kb, q_per, q_split;
 };
 
-__global__ void __launch_bounds__(kHeadThreads, 1)
+// Rounds of a row from its r profile rows' coefficients, by one warp: the same value whichever CTA asks.
+// FP32 squares, scaled by the largest coefficient of the first round so that none leaves the range.
+__device__ __noinline__ int head_rounds(const float4* __restrict__ F, int r, int n_h, int lane) {
+  int rounds = 1;
+  for (int s = 0; s < r; ++s) {
+    const float4* f = F + (size_t)s * n_h;
+    float e[kHeadRounds + 1];   // squares of round t's frequencies; of those after all the rounds
+    float2 v[kHeadRounds][kChirpHead / 32];
+    float top = 0.0f;
+#pragma unroll
+    for (int t = 0; t < kHeadRounds; ++t)
+#pragma unroll
+      for (int u = 0; u < kChirpHead / 32; ++u)   // n < 256 < n_h
+        v[t][u] = *reinterpret_cast<const float2*>(f + t * kChirpHead + u * 32 + lane);
+#pragma unroll
+    for (int u = 0; u < kChirpHead / 32; ++u) top = fmaxf(top, fmaxf(fabsf(v[0][u].x), fabsf(v[0][u].y)));
+#pragma unroll
+    for (int o = 16; o; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    const float scale = top > 1e-37f ? 1.0f / top : 1.0f;
+#pragma unroll
+    for (int t = 0; t < kHeadRounds; ++t) {
+      e[t] = 0.0f;
+#pragma unroll
+      for (int u = 0; u < kChirpHead / 32; ++u) {
+        const float x = scale * v[t][u].x, y = scale * v[t][u].y;
+        e[t] = fmaf(x, x, fmaf(y, y, e[t]));
+      }
+    }
+    e[kHeadRounds] = 0.0f;
+#pragma unroll 8
+    for (int n = kHeadRounds * kChirpHead + lane; n < n_h; n += 32) {
+      const float2 w = *reinterpret_cast<const float2*>(f + n);
+      const float x = scale * w.x, y = scale * w.y;
+      e[kHeadRounds] = fmaf(x, x, fmaf(y, y, e[kHeadRounds]));
+    }
+    float all = 0.0f;
+#pragma unroll
+    for (int t = 0; t <= kHeadRounds; ++t) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) e[t] += __shfl_xor_sync(0xffffffffu, e[t], o);
+      all += e[t];
+    }
+    float rest = e[kHeadRounds];
+    int need = kHeadRounds;
+#pragma unroll
+    for (int t = kHeadRounds - 1; t >= 1; --t) {
+      rest += e[t];                                   // what is left after t rounds
+      if (need == t + 1 && rest <= (float)(kHeadRest * kHeadRest) * all) need = t;
+    }
+    rounds = max(rounds, need);
+  }
+  return rounds;
+}
+
+__global__ void __maxnreg__(128)   // (with 156 registers as few spills and 2.63 instead of 1.98 ms at the large shape)
 k_head(float* __restrict__ delta, const uint8_t* __restrict__ aimg, const float4* __restrict__ F,
        const float4* __restrict__ gdf, const int* __restrict__ cls_of, const float* __restrict__ kmu,
-       const int2* __restrict__ cmap, HeadShape sh, int* __restrict__ status) {
+       const int2* __restrict__ cmap, HeadShape sh, int* __restrict__ head, int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ long long rowoff[kHeadNT];    // Delta row of the column's group (-1: no column)
+  __shared__ long long rowoff[kHeadNT];    // Delta row of the column's group (-1: no column, or complete)
   __shared__ int kmoff[kHeadNT];           // kmu row of the column
+  __shared__ int colrd[kHeadNT];           // rounds of the column's row
+  __shared__ int tile_rd;                  // most rounds of the tile
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* bsm = base + kHeadStages * kHeadA;
   uint64_t* bars = reinterpret_cast<uint64_t*>(bsm + kHeadKb * kHeadB);
@@ -1835,6 +1910,7 @@ k_head(float* __restrict__ delta, const uint8_t* __restrict__ aimg, const float4
     }
     mbar_init(smem_u32(done), 1);
     *abort_flag = 0;
+    tile_rd = 1;
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 512);
@@ -1842,169 +1918,218 @@ k_head(float* __restrict__ delta, const uint8_t* __restrict__ aimg, const float4
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int n_a = n_it * kHeadKb;                  // K-blocks of the phase image this CTA streams
-  const uint8_t* asrc = aimg + (size_t)mt0 * kHeadKb * kHeadA;
+  const int n_a = n_it * kHeadKb;                  // K-blocks of the phase image per round
+  // thread 0: copies of K-blocks issued so far, in the order in which they are multiplied; up to `limit`
   int issued = 0;
-  auto copy = [&](int g) {
-    const int s = g % kHeadStages;
-    mbar_arrive_tx(smem_u32(&afull[s]), kHeadA);
-    bulk_g2s(smem_u32(base + s * kHeadA), asrc + (size_t)g * kHeadA, kHeadA, smem_u32(&afull[s]));
+  auto feed = [&](int limit) {
+    for (; issued < limit; ++issued) {
+      const int s = issued % kHeadStages;
+      if (issued >= kHeadStages &&
+          !mbar_wait(smem_u32(&aempty[s]), (issued / kHeadStages - 1) & 1, abort_flag))
+        break;
+      const int rd = issued / n_a, g = issued - rd * n_a;
+      const size_t blk = (size_t)(mt0 + g / kHeadKb) * sh.f_kb + rd * kHeadKb + g % kHeadKb;
+      mbar_arrive_tx(smem_u32(&afull[s]), kHeadA);
+      bulk_g2s(smem_u32(base + s * kHeadA), aimg + blk * kHeadA, kHeadA, smem_u32(&afull[s]));
+    }
   };
-  if (tid == 0)
-    for (; issued < min(n_a, kHeadStages); ++issued) copy(issued);
 
-  if (warp >= 2) {
-    // column c of the tile: half c / 32, group (c % 32) / r of the half, profile row (c % 32) % r
-    const int row = (tid - 64) >> 2, ch = tid & 3;
-    const int gh = 32 / sh.r, in = row & 31, gi = in / sh.r, s = in - gi * sh.r;
-    const int g = (2 * ct + (row >> 5)) * gh + gi;
-    const bool live = gi < gh && g < sh.n_groups;
-    int wi = 0, l = 0;
-    if (live) {
-      if (cmap) {
-        const int2 cm = cmap[g];
-        wi = cm.x;
-        l = cm.y;
-      } else {
-        l = g % sh.n_l;
-        wi = g / sh.n_l;
+  int n_round = 1;
+  for (int rd = 0; rd < n_round; ++rd) {
+    if (tid == 0) feed(rd * n_a + min(n_a, kHeadStages));
+    if (warp >= 2 && warp < 10) {
+      // column c of the tile: half c / 32, group (c % 32) / r of the half, profile row (c % 32) % r
+      const int row = (tid - 64) >> 2, ch = tid & 3;
+      const int gh = 32 / sh.r, in = row & 31, gi = in / sh.r, s = in - gi * sh.r;
+      const int g = (2 * ct + (row >> 5)) * gh + gi;
+      const bool live = gi < gh && g < sh.n_groups;
+      int wi = 0, l = 0;
+      if (live) {
+        if (cmap) {
+          const int2 cm = cmap[g];
+          wi = cm.x;
+          l = cm.y;
+        } else {
+          l = g % sh.n_l;
+          wi = g / sh.n_l;
+        }
       }
-    }
-    const int i = wi % sh.N_tr, w = wi / sh.N_tr;
-    if (ch == 0) {
-      rowoff[row] = live ? (((long long)w * sh.n_l + l) * sh.N_tr + i) * sh.N_k : -1;
-      kmoff[row] = (i * 4 + s) * sh.N_k;
-    }
-    const float4* Fr = F + ((size_t)wi * sh.NI + s) * sh.n_h;
-    const float4* Gr = gdf + ((size_t)(live ? cls_of[i] : 0) * sh.N_ell + sh.l_lo + l) * sh.n_h;
-    // one K-block (four frequencies per thread) at a time, the next one's values in flight; not
-    // unrolled: every CTA runs this once, so its instructions come from a cold cache
-    float4 fv[4], gv[4];
-    auto fetch = [&](int kb) {
+      const int i = wi % sh.N_tr, w = wi / sh.N_tr;
+      if (ch == 0 && rd == 0) {
+        rowoff[row] = live ? (((long long)w * sh.n_l + l) * sh.N_tr + i) * sh.N_k : -1;
+        kmoff[row] = (i * 4 + s) * sh.N_k;
+      }
+      if (ch == 0 && rd > 0 && colrd[row] <= rd) rowoff[row] = -1;   // this row is complete
+      const float4* Fr = F + ((size_t)wi * sh.NI + s) * sh.n_h;
+      const float4* Gr = gdf + ((size_t)(live ? cls_of[i] : 0) * sh.N_ell + sh.l_lo + l) * sh.n_h;
+      const int n_end = !live ? 0 : rd == 0 ? kChirpHead : min(sh.n_h, colrd[row] * kChirpHead);
+      // one K-block (four frequencies per thread) at a time, the next one's values in flight; not
+      // unrolled: every CTA runs this once or a few times, so its instructions come from a cold cache
+      float4 fv[4], gv[4];
+      auto fetch = [&](int kb) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int n = kb * (kK / 2) + ch * 4 + u;
-        const bool in = live && n < sh.n_h;
-        fv[u] = in ? Fr[n] : make_float4(0.f, 0.f, 0.f, 0.f);
-        gv[u] = in ? __ldg(Gr + n) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    };
-    fetch(0);
+        for (int u = 0; u < 4; ++u) {
+          const int n = rd * kChirpHead + kb * (kK / 2) + ch * 4 + u;
+          fv[u] = n < n_end ? Fr[n] : make_float4(0.f, 0.f, 0.f, 0.f);
+          gv[u] = n < n_end ? __ldg(Gr + n) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      };
+      fetch(0);
 #pragma unroll 1
-    for (int kb = 0; kb < kHeadKb; ++kb) {
-      float4 f[4], g4[4];
+      for (int kb = 0; kb < kHeadKb; ++kb) {
+        float4 f[4], g4[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) { f[u] = fv[u]; g4[u] = gv[u]; }
-      if (kb + 1 < kHeadKb) fetch(kb + 1);
-      __nv_bfloat16 v[8][kPlanes];
+        for (int u = 0; u < 4; ++u) { f[u] = fv[u]; g4[u] = gv[u]; }
+        if (kb + 1 < kHeadKb) fetch(kb + 1);
+        __nv_bfloat16 v[8][kPlanes];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        float rh, rl, ih, il;
-        df_dot2(f[u].x, f[u].z, g4[u].x, g4[u].z, f[u].y, f[u].w, g4[u].y, g4[u].w, -1.0f, rh, rl);
-        df_dot2(f[u].x, f[u].z, g4[u].y, g4[u].w, f[u].y, f[u].w, g4[u].x, g4[u].z, 1.0f, ih, il);
-        split_df(rh, rl, v[2 * u]);
-        split_df(-ih, -il, v[2 * u + 1]);
+        for (int u = 0; u < 4; ++u) {
+          float rh, rl, ih, il;
+          df_dot2(f[u].x, f[u].z, g4[u].x, g4[u].z, f[u].y, f[u].w, g4[u].y, g4[u].w, -1.0f, rh, rl);
+          df_dot2(f[u].x, f[u].z, g4[u].y, g4[u].w, f[u].y, f[u].w, g4[u].x, g4[u].z, 1.0f, ih, il);
+          split_df(rh, rl, v[2 * u]);
+          split_df(-ih, -il, v[2 * u + 1]);
+        }
+        store_planes<kPlanes>(bsm + kb * kHeadB, kHeadNT * kRow, off64(row, ch * 16), v);
       }
-      store_planes<kPlanes>(bsm + kb * kHeadB, kHeadNT * kRow, off64(row, ch * 16), v);
+      fence_proxy_async();
+    } else if (warp >= 10 && rd == 0) {
+      // rounds of each row of the tile, one warp a row.  A row's columns are neighbours
+      const int gh = 32 / sh.r;
+      auto row_of = [&](int half) {   // walker N_tr + tracer of column 32 half + lane (-1: no column)
+        const int gi = lane / sh.r, g = (2 * ct + half) * gh + gi;
+        return gi >= gh || g >= sh.n_groups ? -1 : cmap ? cmap[g].x : g / sh.n_l;
+      };
+      const int w0 = row_of(0), w1 = row_of(1);
+      int p0 = __shfl_up_sync(0xffffffffu, w0, 1), p1 = __shfl_up_sync(0xffffffffu, w1, 1);
+      const int end0 = __shfl_sync(0xffffffffu, w0, gh * sh.r - 1);
+      if (lane == 0) { p0 = -1; p1 = end0; }
+      uint32_t f0 = __ballot_sync(0xffffffffu, w0 >= 0 && p0 != w0), f1 = __ballot_sync(0xffffffffu, w1 >= 0 && p1 != w1);
+      for (int k = 0; f0 | f1; ++k) {   // the first column of every row
+        int wi;
+        if (f0) { wi = __shfl_sync(0xffffffffu, w0, __ffs(f0) - 1); f0 &= f0 - 1; }
+        else { wi = __shfl_sync(0xffffffffu, w1, __ffs(f1) - 1); f1 &= f1 - 1; }
+        if ((k & 1) != warp - 10) continue;
+        const int need = head_rounds(F + (size_t)wi * sh.NI * sh.n_h, sh.r, sh.n_h, lane);
+        if (w0 == wi) colrd[lane] = need;
+        if (w1 == wi) colrd[32 + lane] = need;
+        if (lane == 0) {
+          head[wi] = need * kChirpHead;
+          atomicMax(&tile_rd, need);
+        }
+      }
     }
-    fence_proxy_async();
-  }
-  __syncthreads();
+    __syncthreads();
+    n_round = tile_rd;
 
-  if (warp == 0) {
-    if (lane == 0) {
-      for (; issued < n_a; ++issued) {
-        const int s = issued % kHeadStages;
-        if (!mbar_wait(smem_u32(&aempty[s]), (issued / kHeadStages - 1) & 1, abort_flag)) break;
-        copy(issued);
-      }
-      if (*abort_flag)   // copies still in flight land before the CTA exits
-        for (int g = max(0, issued - kHeadStages); g < issued; ++g)
-          mbar_wait_drain(smem_u32(&afull[g % kHeadStages]), (g / kHeadStages) & 1);
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    // every lane runs the loop, one issues (elect_one)
-    const uint32_t idesc = idesc_bf16(kM, kHeadNT);
-    bool ok = true;
-    for (int it = 0; it < n_it && ok; ++it) {
-      const int b = it & 1;
-      if (it >= 2)
-        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&accempty[b]), ((it >> 1) - 1) & 1, abort_flag));
+    if (warp == 0) {
+      if (lane == 0) feed((rd + 1) * n_a);
+      __syncwarp();
+    } else if (warp == 1) {
+      // every lane runs the loop, one issues (elect_one)
+      const uint32_t idesc = idesc_bf16(kM, kHeadNT);
+      bool ok = true;
+      for (int it = rd * n_it; it < (rd + 1) * n_it && ok; ++it) {
+        const int b = it & 1;
+        if (it >= 2)
+          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&accempty[b]), ((it >> 1) - 1) & 1, abort_flag));
 #pragma unroll 1
-      for (int kb = 0; kb < kHeadKb && ok; ++kb) {
-        const int g = it * kHeadKb + kb, s = g % kHeadStages;
-        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&afull[s]), (g / kHeadStages) & 1, abort_flag));
-        if (!ok) break;
-        tc_fence_after();
-        const uint64_t da = desc64(smem_u32(base + s * kHeadA)), db = desc64(smem_u32(bsm + kb * kHeadB));
-        const uint32_t d_main = tmem + (uint32_t)(b * 256 + (kb >> 1) * 128), d_corr = d_main + 64;
+        for (int kb = 0; kb < kHeadKb && ok; ++kb) {
+          const int g = it * kHeadKb + kb, s = g % kHeadStages;
+          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&afull[s]), (g / kHeadStages) & 1, abort_flag));
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t da = desc64(smem_u32(base + s * kHeadA)), db = desc64(smem_u32(bsm + kb * kHeadB));
+          const uint32_t d_main = tmem + (uint32_t)(b * 256 + (kb >> 1) * 128), d_corr = d_main + 64;
 #pragma unroll
-        for (int j = 0; j < kK / 16; ++j) {
+          for (int j = 0; j < kK / 16; ++j) {
 #pragma unroll
-          for (int t = 0; t < A3B3::kProducts; ++t) {
-            const uint64_t ad = da + (uint64_t)((A3B3::pa(t) * kPlaneM + j * 256) >> 4);
-            const uint64_t bd = db + (uint64_t)((A3B3::pb(t) * kHeadNT * kRow + j * 256) >> 4);
-            const bool first = (kb & 1) == 0 && j == 0 && t <= 1;
-            mma_bf16(t == 0 ? d_main : d_corr, ad, bd, idesc, first ? 0u : 1u);
+            for (int t = 0; t < A3B3::kProducts; ++t) {
+              const uint64_t ad = da + (uint64_t)((A3B3::pa(t) * kPlaneM + j * 256) >> 4);
+              const uint64_t bd = db + (uint64_t)((A3B3::pb(t) * kHeadNT * kRow + j * 256) >> 4);
+              const bool first = (kb & 1) == 0 && j == 0 && t <= 1;
+              mma_bf16(t == 0 ? d_main : d_corr, ad, bd, idesc, first ? 0u : 1u);
+            }
+          }
+          if (elect_one()) mma_commit(smem_u32(&aempty[s]));
+        }
+        if (ok && elect_one()) mma_commit(smem_u32(&accfull[b]));
+        __syncwarp();
+      }
+    } else if (warp < 10) {
+      const int quarter = warp & 3, c0 = ((warp - 2) >> 2) * 32;
+      const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + c0;
+      // one q tile; `more`: added to the sums of the rounds before
+      auto drain = [&](int it, auto more) {
+        const int b = it & 1;
+        const int q = (mt0 + it - rd * n_it) * kM + quarter * 32 + lane;
+        const bool in = q < sh.N_k;
+        float v = 0.0f;
+        int s = 0;
+#pragma unroll 1
+        for (int c = 0; c < 32; c += 16) {
+          __syncwarp();
+          float old[16];
+          if constexpr (decltype(more)::value) {   // all loads in flight at once
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {
+              const long long o = rowoff[c0 + c + t];
+              old[t] = in && o >= 0 ? delta[o + q] : 0.0f;
+            }
+          }
+          uint32_t m0[16], r0[16], m1[16], r1[16];
+          const uint32_t a = lane_base + b * 256 + c;
+          tmem_ld16_async(a, m0);
+          tmem_ld16_async(a + 64, r0);
+          tmem_ld16_async(a + 128, m1);
+          tmem_ld16_async(a + 192, r1);
+          tmem_wait_ld();
+          reg_fence(m0);
+          reg_fence(r0);
+          reg_fence(m1);
+          reg_fence(r1);
+          if (c == 16) {
+            // the buffer is read: the MMA warp may refill it
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&accempty[b]));
+          }
+#pragma unroll
+          for (int t = 0; t < 16; ++t) {
+            const float z = (__uint_as_float(m0[t]) + __uint_as_float(r0[t])) +
+                            (__uint_as_float(m1[t]) + __uint_as_float(r1[t]));
+            const long long o = rowoff[c0 + c + t];
+            if (in && o >= 0) v = fmaf(__ldg(kmu + kmoff[c0 + c + t] + q), z, v);
+            if (++s == sh.r) {
+              if constexpr (decltype(more)::value) v += old[t];
+              if (in && o >= 0) delta[o + q] = v;
+              v = 0.0f;
+              s = 0;
+            }
           }
         }
-        if (elect_one()) mma_commit(smem_u32(&aempty[s]));
+      };
+      for (int it = rd * n_it; it < (rd + 1) * n_it; ++it) {
+        const bool got = mbar_wait(smem_u32(&accfull[it & 1]), (it >> 1) & 1, abort_flag);
+        if (!__all_sync(0xffffffffu, got)) break;
+        tc_fence_after();
+        if (rd == 0) drain(it, std::false_type());
+        else drain(it, std::true_type());
       }
-      if (ok && elect_one()) mma_commit(smem_u32(&accfull[b]));
-      __syncwarp();
     }
+    // the round's products are complete and read: H and the ring are free
+    if (__syncthreads_or(*abort_flag)) break;
+  }
+  if (warp == 0 && lane == 0 && *abort_flag)   // copies still in flight land before the CTA exits
+    for (int g = max(0, issued - kHeadStages); g < issued; ++g)
+      mbar_wait_drain(smem_u32(&afull[g % kHeadStages]), (g / kHeadStages) & 1);
+  if (warp == 1) {
+    __syncwarp();
     // every issued MMA has completed before TMEM is released
     if (elect_one()) mma_commit(smem_u32(done));
     mbar_wait_drain(smem_u32(done), 0);
-    __syncwarp();
-  } else {
-    const int quarter = warp & 3, c0 = ((warp - 2) >> 2) * 32;
-    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + c0;
-    for (int it = 0; it < n_it; ++it) {
-      const int b = it & 1;
-      const bool got = mbar_wait(smem_u32(&accfull[b]), (it >> 1) & 1, abort_flag);
-      if (!__all_sync(0xffffffffu, got)) break;
-      tc_fence_after();
-      const int q = (mt0 + it) * kM + quarter * 32 + lane;
-      float v = 0.0f;
-      int s = 0;
-#pragma unroll 1
-      for (int c = 0; c < 32; c += 16) {
-        __syncwarp();
-        uint32_t m0[16], r0[16], m1[16], r1[16];
-        const uint32_t a = lane_base + b * 256 + c;
-        tmem_ld16_async(a, m0);
-        tmem_ld16_async(a + 64, r0);
-        tmem_ld16_async(a + 128, m1);
-        tmem_ld16_async(a + 192, r1);
-        tmem_wait_ld();
-        reg_fence(m0);
-        reg_fence(r0);
-        reg_fence(m1);
-        reg_fence(r1);
-        if (c == 16) {
-          // the buffer is read: the MMA warp may refill it
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&accempty[b]));
-        }
-        const bool in = q < sh.N_k;
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-          const float z = (__uint_as_float(m0[t]) + __uint_as_float(r0[t])) +
-                          (__uint_as_float(m1[t]) + __uint_as_float(r1[t]));
-          const long long o = rowoff[c0 + c + t];
-          if (in && o >= 0) v = fmaf(__ldg(kmu + kmoff[c0 + c + t] + q), z, v);
-          if (++s == sh.r) {
-            if (in && o >= 0) delta[o + q] = v;
-            v = 0.0f;
-            s = 0;
-          }
-        }
-      }
-    }
   }
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (tid == 0 && *abort_flag) atomicExch(status, 1);
@@ -2283,7 +2408,7 @@ bool valid_tile(int code, const std::vector<int>& cands) {
 
 // K-blocks of the forward GEMM: every frequency, or those below the chirp transform's
 static int fwd_kblocks(const swcl_ctx* c, bool chirp) {
-  return (2 * (chirp ? kChirpHead : c->n_h) + kK - 1) / kK;
+  return chirp ? kHeadRounds * kHeadKb : (2 * c->n_h + kK - 1) / kK;
 }
 
 size_t basis_fixed_bytes(const swcl_ctx* c) {
@@ -2506,6 +2631,7 @@ static int head_and_chirp(swcl_ctx* c, const ColPlan& cp, int l_lo, int n_l) {
   sh.NI = sv.NI;
   sh.n_groups = cp.n_cols / sh.r;
   sh.n_mt = c->bt_f_mt;
+  sh.f_kb = c->bt_f_kb;
   const int per = 2 * (32 / sh.r), n_ct = (sh.n_groups + per - 1) / per;
   // q tiles per CTA: all of them where the column tiles fill the GPU, else as many as leave one turn of
   // CTAs (each CTA forms its columns' H)
@@ -2514,11 +2640,13 @@ static int head_and_chirp(swcl_ctx* c, const ColPlan& cp, int l_lo, int n_l) {
   const size_t smem = kHeadStages * kHeadA + kHeadKb * kHeadB + 8 * (2 * kHeadStages + 5) + 16 + 1024;
   cudaError_t e = cudaFuncSetAttribute(k_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return cuda_fail(c, e, "basis head attribute");
-  const int st = counted(c, "basis head", [&]() -> int {
+  int st = ensure(c, c->ck_head, sizeof(int) * (size_t)c->n_walk * c->N_tr);
+  if (st) return st;
+  st = counted(c, "basis head", [&]() -> int {
     k_head<<<(unsigned)((long)n_ct * sh.q_split), kHeadThreads, smem, c->stream>>>(
         (float*)c->ws_delta.p, (const uint8_t*)c->bt_eimg_f.p, (const float4*)c->ws_coef.p,
         (const float4*)c->bt_gdf.p, (const int*)c->d_cls_of.p, (const float*)c->bt_kmu.p, cp.cmap_f, sh,
-        (int*)c->ws_status.p);
+        (int*)c->ck_head.p, (int*)c->ws_status.p);
     const cudaError_t le = cudaGetLastError();
     return le == cudaSuccess ? SWCL_OK : cuda_fail(c, le, "basis head");
   });

@@ -44,11 +44,12 @@ int log_size(int n_in, int n_out) {
 }
 
 // First frequency of the forward transform.  FP64: the term n = 0, whose phase is 1, is added beside
-// the transform, so that N/2 frequencies remain.  FP32: the terms n < 64, which carry most of a smooth
-// window's Delta, stay in the compensated tensor-core GEMM; the FFT's rounding error, about 2e-7 of
-// what passes through it, then falls on the small rest.  Simulated C error against the FP64 oracle at
-// N5K shape (the GEMM over all frequencies 2.1e-5): 2.4e-5 with 32 terms in the GEMM, 1.8e-5 with 64,
-// 2.1e-5 with 128; 1.4e-4 with none.
+// the transform, so that N/2 frequencies remain.  FP32: at least the terms n < 64, which carry most of a
+// smooth window's Delta, stay in compensated tensor-core products; the FFT's rounding error, about 2e-7 of what
+// passes through it, then falls on the small rest.  Rows with a larger rest keep more (k_head), and zeros
+// take their places in the transform.  Simulated C error against the FP64 oracle at N5K shape
+// (the GEMM over all frequencies 2.1e-5): 2.4e-5 with 32 terms in the products, 1.8e-5 with 64, 2.1e-5
+// with 128; 1.4e-4 with none.
 int first_freq(int precision) { return precision == SWCL_FP64 ? 1 : kChirpHead; }
 int form(int precision) { return precision == SWCL_FP64 ? 0 : 1; }
 
@@ -176,7 +177,7 @@ int chirp_forward(swcl_ctx* c, int precision, int l_lo, int n_l) {
           ? chirp64_forward(d, (double*)c->ws_delta.p, (const cplx*)c->ws_coef.p, (const cplx*)c->d_gtab.p,
                             (const int*)c->d_cls_of.p, sv.w, sv.w_ts, (const double*)c->d_kpow.p, r, c->stream)
           : chirp32_forward(d, (float*)c->ws_delta.p, (const float4*)c->ws_coef.p, (const float2*)c->bt_g32.p,
-                            (const int*)c->d_cls_of.p, (const float*)c->bt_kmu.p, r, c->stream);
+                            (const int*)c->d_cls_of.p, (const float*)c->bt_kmu.p, (const int*)c->ck_head.p, r, c->stream);
   prof_end(c, precision == SWCL_FP64 ? "chirp fwd fp64" : "chirp fwd f32");
   return e == cudaSuccess ? SWCL_OK : cuda_fail(c, e, "chirp transform, forward");
 }

@@ -398,6 +398,7 @@ template <class T> struct ChirpArgs {
   const T* kw;           // FP64: stencil weights [tracer stride lw_ts][N_k][4]; FP32: kpow mu [N_tr][4][N_k]
   long lw_ts;
   const double* kpow;    // FP64: [N_tr][N_k]
+  const int* head;       // FP32 forward: [walker N_tr + tracer] the frequencies below this are in Delta already
   const int* off;        // ragged lists (null: multipoles l_lo .. l_lo + n_l - 1)
   const int* idx;
   int N_tr, NI, n_h, N_k, N_ell, l_lo, n_l, r, n0, n_chunk;
@@ -434,7 +435,7 @@ template <class T, int LOGM> constexpr int min_blocks() {
 
 // Delta[w][l - l_lo][i][q] (+)= sum_s kw_is[q] Re sum_{n >= n0} F_wisn G[l][n] e^{-i eta_n ln k_q}
 // FP64 (n0 = 1): the term n = 0, whose phase is 1, is added and Delta is written; FP32 (n0 > 0):
-// the terms below n0 are in Delta already.  CT: cplx (FP64) or float4 (double-float pairs, FP32).
+// the terms below head >= n0 are in Delta already.  CT: cplx (FP64) or float4 (double-float pairs, FP32).
 template <int LOGM, class T, class CT, bool HALF>
 __global__ void __launch_bounds__(Plan<LOGM, T>::kT, min_blocks<T, LOGM>())
 k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) {
@@ -456,11 +457,13 @@ k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) 
     const CT* F = coef + ((size_t)wi * A.NI + s) * A.n_h;
     V f[HALF ? NI : 1], cs[HALF ? NI : 1];
     T km[kDc && HALF ? NI : 1];
+    const int m0 = kDc ? 0 : A.head[wi] - A.n0;   // first frequency here, from n0
     if constexpr (HALF) {
 #pragma unroll
       for (int e = 0; e < NI; ++e) {
         const int m = t + e * P::S1;
-        f[e] = m < n_in ? mul(coef_at(F + A.n0 + m), A.a[m]) : mk<T>(0, 0);
+        // (a row's tensor-core rounds end below frequency 256)
+        f[e] = m < n_in && (e * P::S1 >= 192 || m >= m0) ? mul(coef_at(F + A.n0 + m), A.a[m]) : mk<T>(0, 0);
         const T k = m < A.N_k ? k_weight(A, i, s, m) : T(0);
         const V b = m < A.N_k ? A.b[m] : mk<T>(0, 0);
         cs[e] = mk<T>(k * b.x, k * b.y);
@@ -498,7 +501,7 @@ k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) 
         if constexpr (HALF) {
           v[e] = m < n_in ? mul(f[e], __ldg(G + m)) : mk<T>(0, 0);
         } else {
-          v[e] = m < n_in ? mul(mul(coef_at(F + A.n0 + m), A.a[m]), __ldg(G + m)) : mk<T>(0, 0);
+          v[e] = m >= m0 && m < n_in ? mul(mul(coef_at(F + A.n0 + m), A.a[m]), __ldg(G + m)) : mk<T>(0, 0);
         }
       }
 #pragma unroll

@@ -25,6 +25,7 @@ ChirpArgs<float> args(const ChirpDir& d, const ChirpRun& r, const float2* g, con
   A.kw = kmu;
   A.lw_ts = 0;
   A.kpow = nullptr;
+  A.head = nullptr;
   A.off = r.off;
   A.idx = r.idx;
   A.N_tr = r.N_tr; A.NI = r.NI; A.n_h = r.n_h; A.N_k = r.N_k; A.N_ell = r.N_ell;
@@ -59,8 +60,10 @@ cudaError_t chirp32_build(void* tab, int logm, int n0, int n_in, int N_k, int t_
 }
 
 cudaError_t chirp32_forward(const ChirpDir& d, float* delta, const float4* coef, const float2* g, const int* cls_of,
-                            const float* kmu, const ChirpRun& r, cudaStream_t s) {
-  return launch_fwd<float>(d.logm, d.half, delta, coef, args(d, r, g, cls_of, kmu), r.n_walk * r.N_tr, s);
+                            const float* kmu, const int* head, const ChirpRun& r, cudaStream_t s) {
+  ChirpArgs<float> A = args(d, r, g, cls_of, kmu);
+  A.head = head;
+  return launch_fwd<float>(d.logm, d.half, delta, coef, A, r.n_walk * r.N_tr, s);
 }
 
 cudaError_t chirp32_adjoint(const ChirpDir& d, void* part, const float* dbar, const float2* g, const int* cls_of,

@@ -22,6 +22,7 @@ ChirpArgs<double> args(const ChirpDir& d, const ChirpRun& r, const cplx* g, cons
   A.kw = w;
   A.lw_ts = w_ts;
   A.kpow = kpow;
+  A.head = nullptr;
   A.off = r.off;
   A.idx = r.idx;
   A.N_tr = r.N_tr; A.NI = r.NI; A.n_h = r.n_h; A.N_k = r.N_k; A.N_ell = r.N_ell;

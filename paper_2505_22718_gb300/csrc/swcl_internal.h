@@ -115,7 +115,8 @@ struct LimberTable {
   double* lnnu = nullptr;
 };
 
-// frequencies that stay in the basis-mode GEMM beside the FP32 chirp transform (four K-blocks)
+// frequencies of one round of tensor-core products beside the FP32 chirp transform (four K-blocks); the
+// first of them is the least that a row takes
 constexpr int kChirpHead = 64;
 
 // Chirp transforms of the contraction (chirp.cuh): one direction's size and tables
@@ -196,6 +197,7 @@ struct swcl_ctx {
   double ck_x[2] = {0, 0};     // x0/L
   swcl::ChirpDir ck[2][2];     // [FP64, FP32][forward, adjoint]
   swcl::DevBuf ws_ckpart;      // adjoint: partial sums over the multipoles
+  swcl::DevBuf ck_head;        // mixed form: [n_walk][N_tr] frequencies in the tensor-core products
 
   // basis-mode tensor-core GEMMs (basis_tc.cu)
   bool bt_ready = false;       // constant operands built for the current grids/tracers/profiles
@@ -409,7 +411,7 @@ size_t chirp32_table_bytes(int logm, int n_in, int N_k);
 cudaError_t chirp32_build(void* tab, int logm, int n0, int n_in, int N_k, int t_lo, int t_hi, const double* cc,
                           const double* xx, bool forward, cudaStream_t s);
 cudaError_t chirp32_forward(const ChirpDir& d, float* delta, const float4* coef, const float2* g, const int* cls_of,
-                            const float* kmu, const ChirpRun& r, cudaStream_t s);
+                            const float* kmu, const int* head, const ChirpRun& r, cudaStream_t s);
 cudaError_t chirp32_adjoint(const ChirpDir& d, void* part, const float* dbar, const float2* g, const int* cls_of,
                             const float* kmu, const ChirpRun& r, cudaStream_t s);
 cudaError_t chirp32_sum(cplx* cbar, const void* part, const ChirpDir& d, const ChirpRun& r, bool accumulate,
