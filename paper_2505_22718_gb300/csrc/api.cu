@@ -526,6 +526,7 @@ int swcl_set_tracers(swcl_ctx* c, int N_tr, const int* kind, const double* fft_b
   c->u_valid = false;
   c->lr_dirty = true;
   c->lr_basis = false;
+  c->ck_off = false;
   c->N_tr = N_tr;
   c->n_cls = (int)cls.size();
   c->kind_h = kh;
@@ -795,15 +796,17 @@ static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need, bool whole_par
 }
 
 // The same with the tables of the chirp transforms built first.  Where the budget has no room for 8
-// multipoles beside them, their partial sums are planned at the least, then they are given up.
+// multipoles beside them, their partial sums are planned at the least; then the FP64 form gives them up,
+// until other grids or tracers are set.
 static int plan_chunk(swcl_ctx* c, int precision, int n_need, int& n_lc) {
   SWCL_TRY(swcl::chirp_prepare(c, precision));
   n_lc = plan_ell_chunk(c, precision, n_need, true);
   if (n_lc == 0 && swcl::chirp_use(c, precision)) {
     n_lc = plan_ell_chunk(c, precision, n_need, false);
-    if (n_lc == 0) {
+    if (n_lc == 0 && precision == SWCL_FP64) {
       SWCL_TRY(swcl::chirp_drop(c));
       n_lc = plan_ell_chunk(c, precision, n_need, true);
+      if (n_lc == 0) c->ck_off = false;   // of no use: a smaller call may have room for them
     }
   }
   if (n_lc == 0)
@@ -1479,6 +1482,12 @@ int swcl_jvp(swcl_ctx* c, int precision, int n_dir, const double* P_dot, const d
   c->u_valid = false;
   {
     WalkScope scope(c, nw2);
+    // what these 1 + n_dir walkers have no room for, a pass of one may have
+    struct KeepOff {
+      swcl_ctx* c;
+      bool off;
+      ~KeepOff() { c->ck_off = off; }
+    } keep{c, c->ck_off};
     int n_lc = 0;
     SWCL_TRY(plan_chunk(c, precision, n_fft, n_lc));
     c->ell_chunk = n_lc;

@@ -63,7 +63,7 @@ constexpr int kMaxSum32 = 16;
 int chirp_rank(const swcl_ctx* c) { return c->lr_basis ? c->lr_true_rank : c->N_I <= 4 ? c->N_I : 0; }
 
 bool chirp_use(const swcl_ctx* c, int precision) {
-  if (!c->ck_uniform || c->ck_off) return false;
+  if (!c->ck_uniform || (c->ck_off && precision == SWCL_FP64)) return false;
   const int r = chirp_rank(c), mf = log_size(c->n_h - first_freq(precision), c->N_k), ma = log_size(c->N_k, c->n_h);
   if (r <= 0 || !mf || !ma) return false;
   // FP64 operations: about 75 per point and pair of FFTs, against 2 per (frequency, k point) of the
@@ -80,16 +80,16 @@ bool chirp_use(const swcl_ctx* c, int precision) {
   return c->N >= 1024;
 }
 
+// FP64 only: the direct sums need no tables.  (The mixed form has nothing to gain from giving its
+// transforms up: the images of the GEMMs over all frequencies take several times as much memory.)
 int chirp_drop(swcl_ctx* c) {
   if (c->capturing) return fail(c, SWCL_ERR_STATE, "chirp tables given up during capture");
-  for (auto& p : c->ck)
-    for (auto& d : p) {
-      release(c, d.tab);
-      d.ready = false;
-    }
+  for (auto& d : c->ck[form(SWCL_FP64)]) {
+    release(c, d.tab);
+    d.ready = false;
+  }
   release(c, c->ws_ckpart);
   c->ck_off = true;
-  c->bt_ready = false;
   return SWCL_OK;
 }
 
@@ -107,7 +107,7 @@ int chirp_prepare(swcl_ctx* c, int precision) {
     const bool fp64 = precision == SWCL_FP64;
     const int st = ensure(c, d.tab, fp64 ? chirp64_table_bytes(d.logm, n_freq, c->N_k)
                                          : chirp32_table_bytes(d.logm, n_freq, c->N_k));
-    if (st == SWCL_ERR_OOM_BUDGET) {   // the direct sums need no tables
+    if (st == SWCL_ERR_OOM_BUDGET && fp64) {
       c->err.clear();
       return chirp_drop(c);
     }

@@ -192,7 +192,7 @@ struct swcl_ctx {
 
   // chirp transforms (chirp.cu): set by the grids
   bool ck_uniform = false;     // ln k_q = x0 + q d
-  bool ck_off = false;         // given up (memory budget)
+  bool ck_off = false;         // FP64 form: given up for now (memory budget)
   double ck_c[2] = {0, 0};     // d/(2 L) in double-double
   double ck_x[2] = {0, 0};     // x0/L
   swcl::ChirpDir ck[2][2];     // [FP64, FP32][forward, adjoint]
@@ -389,8 +389,8 @@ cudaError_t launch_contract_fp64_adj(cplx* cbar, const double* dbar, const cplx*
 void chirp_fit_grid(swcl_ctx* c);
 bool chirp_use(const swcl_ctx* c, int precision);
 int chirp_rank(const swcl_ctx* c);
-int chirp_prepare(swcl_ctx* c, int precision);      // tables; gives the transforms up on a full budget
-int chirp_drop(swcl_ctx* c);                        // frees them; refused during graph capture
+int chirp_prepare(swcl_ctx* c, int precision);      // tables; FP64: given up on a full budget
+int chirp_drop(swcl_ctx* c);                        // frees the FP64 tables; refused during graph capture
 size_t chirp_part_bytes(const swcl_ctx* c, int precision, int n_l, bool whole);
 int chirp_forward(swcl_ctx* c, int precision, int l_lo, int n_l);
 int chirp_adjoint(swcl_ctx* c, int precision, int l_lo, int n_l, bool accumulate);

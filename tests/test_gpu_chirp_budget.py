@@ -83,6 +83,17 @@ def _smallest_budget(fits, hi):
     return hi
 
 
+def _routes(ctx, call):
+    """Names of the kernels that call() runs (outside a graph)."""
+    import paper_2505_22718_gb300 as S
+    S.swcl_profile_enable(ctx.ptr, True)
+    S.swcl_profile_reset(ctx.ptr)
+    call()
+    names = set(S.swcl_profile_read(ctx.ptr))
+    S.swcl_profile_enable(ctx.ptr, False)
+    return names
+
+
 def _same(a, b, tol):
     for x, y in zip(a, b):
         assert max_rel(x, y) < tol
@@ -131,3 +142,71 @@ def test_graph_after_the_tables_were_freed():
     b = _smallest_budget(lambda x: bool(run(x, False)), most + (64 << 20))
     assert run(b, True) is True
     assert run(b - 65536, True) is False
+
+
+def test_tables_given_up_for_one_call_only():
+    """The same forward-mode call that leaves no room for the tables: the FP64 passes of one point that
+    follow have it, and take the transforms again."""
+    import paper_2505_22718_gb300 as S
+    w, rng = _case(512, 400, 40)
+    W_dot = rng.standard_normal((8,) + w.W.shape[1:]) * w.W[0]
+
+    def fits(budget):
+        ctx = _context(w, budget)
+        if ctx is None:
+            return False
+        try:
+            return not _over_budget(lambda: ctx.jvp(W_dot=W_dot))
+        finally:
+            ctx.close()
+
+    free = lib_context(w)
+    want = free.compute_cl(S.SWCL_FP64)
+    free.jvp(W_dot=W_dot)
+    most = free.query(S.SWCL_Q_WORKSPACE_BYTES)
+    free.close()
+    ctx = lib_context(w, budget=_smallest_budget(fits, most + (64 << 20)))
+    got = []
+    assert "contract fp64" in _routes(ctx, lambda: ctx.jvp(W_dot=W_dot))
+    assert "chirp fwd fp64" in _routes(ctx, lambda: got.append(ctx.compute_cl(S.SWCL_FP64)))
+    assert max_rel(got[0], want) < 1e-10
+    ctx.close()
+
+
+def test_mixed_step_between_calls_that_do_not_fit():
+    """A mixed step under a budget that it just fits.  Calls that find no room there (forward mode along
+    eight windows, the FP64 form beside the FP32 tables) leave its route and its results as they were: C,
+    P_bar and amp_bar bit for bit; W_bar, whose partial sums are as many as the budget has room for, to the
+    1e-5 of the other tests of budgets."""
+    import paper_2505_22718_gb300 as S
+    w, rng = _case(1024, 400, 40)
+    W_dot = rng.standard_normal((8,) + w.W.shape[1:]) * w.W[0]
+    step = _Step(w)
+    free = lib_context(w)
+    want = step(free, S.SWCL_SPLIT_BF16)
+    want64 = free.compute_cl(S.SWCL_FP64)
+    most = free.query(S.SWCL_Q_WORKSPACE_BYTES)
+    free.close()
+
+    def fits(budget):
+        ctx = _context(w, budget)
+        if ctx is None:
+            return False
+        try:
+            return not _over_budget(lambda: step(ctx, S.SWCL_SPLIT_BF16)) and ctx.query(S.SWCL_Q_RECOMPUTE) == 0
+        finally:
+            ctx.close()
+
+    def check(got):
+        assert all(np.array_equal(a, b) for a, b in zip(got[:3], want)) and max_rel(got[3], want[3]) < 1e-5
+
+    ctx = lib_context(w, budget=_smallest_budget(fits, most + (64 << 20)))
+    C = np.empty_like(want[0])
+    for _ in range(2):
+        check(step(ctx, S.SWCL_SPLIT_BF16))
+        assert _over_budget(lambda: ctx.jvp(W_dot=W_dot, precision=S.SWCL_SPLIT_BF16))
+        if not _over_budget(lambda: ctx.compute_cl(S.SWCL_FP64, C)):
+            assert max_rel(C, want64) < 1e-10
+        assert {"basis head", "chirp fwd f32"} <= _routes(ctx, lambda: ctx.compute_cl(S.SWCL_SPLIT_BF16))
+    check(step(ctx, S.SWCL_SPLIT_BF16))
+    ctx.close()
