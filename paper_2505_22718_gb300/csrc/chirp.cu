@@ -161,8 +161,8 @@ size_t chirp_part_bytes(const swcl_ctx* c, int precision, int n_l, bool whole) {
 static ChirpRun run_for(const swcl_ctx* c, int precision, bool adjoint, int l_lo, int n_l) {
   const Stencil sv = stencil(c);
   const bool lists = precision != SWCL_FP64 && c->bt_compact;
-  return ChirpRun{c->n_walk, c->N_tr, sv.NI, c->n_h, c->N_k, c->N_ell, l_lo, n_l, chirp_rank(c),
-                  row_chunks(c, precision, (long)c->n_walk * c->N_tr, n_l, c->ck[form(precision)][adjoint].logm),
+  const int n = row_chunks(c, precision, (long)c->n_walk * c->N_tr, n_l, c->ck[form(precision)][adjoint].logm);
+  return ChirpRun{c->n_walk, c->N_tr, sv.NI, c->n_h, c->N_k, c->N_ell, l_lo, n_l, chirp_rank(c), n, n, 0,
                   lists ? (const int*)c->d_off.p : nullptr, lists ? (const int*)c->d_idx.p : nullptr};
 }
 
@@ -187,26 +187,40 @@ int chirp_adjoint(swcl_ctx* c, int precision, int l_lo, int n_l, bool accumulate
   const ChirpDir& d = c->ck[form(precision)][1];
   const Stencil sv = stencil(c);
   ChirpRun r = run_for(c, precision, true, l_lo, n_l);
-  // partial sums of the CTAs of a row; under a tight budget one CTA per row
+  // Partial sums of the CTAs of a row: those of all the shares of its multipoles, or as many as the budget
+  // has room for.  FP64: then so many larger shares.  FP32, where a share is bounded (kMaxSum32): the
+  // shares in turn, group by group, each group added to the sums of those before in FP64.
   const size_t per = chirp_part_bytes(c, precision, n_l, false);
-  if (c->budget && c->held - c->ws_ckpart.bytes + per * r.n_chunk > c->budget) r.n_chunk = 1;
-  const int st = ensure(c, c->ws_ckpart, per * r.n_chunk);
+  int fit = r.n_total;
+  if (c->budget) {
+    const size_t others = c->held - c->ws_ckpart.bytes;
+    fit = (int)std::min<size_t>(fit, others < c->budget ? (c->budget - others) / per : 0);
+  }
+  if (c->capturing) fit = (int)std::min<size_t>(fit, c->ws_ckpart.bytes / per);
+  fit = std::max(fit, 1);
+  const int st = ensure(c, c->ws_ckpart, per * fit);
   if (st) return st;
-  ++c->last_launches;
-  prof_begin(c);
-  cudaError_t e =
-      fp64 ? chirp64_adjoint(d, c->ws_ckpart.p, (const double*)c->ws_dbar.p, (const cplx*)c->d_gtab.p,
-                             (const int*)c->d_cls_of.p, sv.w, sv.w_ts, (const double*)c->d_kpow.p, r, c->stream)
-           : chirp32_adjoint(d, c->ws_ckpart.p, (const float*)c->ws_dbar.p, (const float2*)c->bt_g32.p,
-                             (const int*)c->d_cls_of.p, (const float*)c->bt_kmu.p, r, c->stream);
-  prof_end(c, fp64 ? "chirp adj fp64" : "chirp adj f32");
-  if (e != cudaSuccess) return cuda_fail(c, e, "chirp transform, transposed");
-  ++c->last_launches;
-  prof_begin(c);
-  e = fp64 ? chirp64_sum((cplx*)c->ws_cbar.p, c->ws_ckpart.p, d, r, accumulate, c->stream)
-           : chirp32_sum((cplx*)c->ws_cbar.p, c->ws_ckpart.p, d, r, accumulate, c->stream);
-  prof_end(c, "chirp adj sum");
-  return e == cudaSuccess ? SWCL_OK : cuda_fail(c, e, "chirp transform, sum over multipoles");
+  if (fp64) r.n_total = fit;
+  for (r.chunk0 = 0; r.chunk0 < r.n_total; r.chunk0 += fit) {
+    r.n_chunk = std::min(fit, r.n_total - r.chunk0);
+    ++c->last_launches;
+    prof_begin(c);
+    cudaError_t e =
+        fp64 ? chirp64_adjoint(d, c->ws_ckpart.p, (const double*)c->ws_dbar.p, (const cplx*)c->d_gtab.p,
+                               (const int*)c->d_cls_of.p, sv.w, sv.w_ts, (const double*)c->d_kpow.p, r, c->stream)
+             : chirp32_adjoint(d, c->ws_ckpart.p, (const float*)c->ws_dbar.p, (const float2*)c->bt_g32.p,
+                               (const int*)c->d_cls_of.p, (const float*)c->bt_kmu.p, r, c->stream);
+    prof_end(c, fp64 ? "chirp adj fp64" : "chirp adj f32");
+    if (e != cudaSuccess) return cuda_fail(c, e, "chirp transform, transposed");
+    ++c->last_launches;
+    prof_begin(c);
+    const bool add = accumulate || r.chunk0 > 0;
+    e = fp64 ? chirp64_sum((cplx*)c->ws_cbar.p, c->ws_ckpart.p, d, r, add, c->stream)
+             : chirp32_sum((cplx*)c->ws_cbar.p, c->ws_ckpart.p, d, r, add, c->stream);
+    prof_end(c, "chirp adj sum");
+    if (e != cudaSuccess) return cuda_fail(c, e, "chirp transform, sum over multipoles");
+  }
+  return SWCL_OK;
 }
 
 }  // namespace swcl

@@ -401,7 +401,8 @@ template <class T> struct ChirpArgs {
   const int* head;       // FP32 forward: [walker N_tr + tracer] the frequencies below this are in Delta already
   const int* off;        // ragged lists (null: multipoles l_lo .. l_lo + n_l - 1)
   const int* idx;
-  int N_tr, NI, n_h, N_k, N_ell, l_lo, n_l, r, n0, n_chunk;
+  int N_tr, NI, n_h, N_k, N_ell, l_lo, n_l, r, n0;
+  int n_chunk, n_total, chunk0;   // CTAs of a row: shares chunk0 .. chunk0 + n_chunk - 1 of n_total
 };
 
 // FP64: kpow lw; FP32: the product is tabulated
@@ -450,7 +451,7 @@ k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) 
   const int i = wi % A.N_tr, w = wi / A.N_tr;
   const int lo = A.off ? A.off[w] : 0;
   int u0, u1;
-  chunk_range(A.off ? A.off[w + 1] - lo : A.n_l, A.n_chunk, chunk, u0, u1);
+  chunk_range(A.off ? A.off[w + 1] - lo : A.n_l, A.n_total, A.chunk0 + chunk, u0, u1);
   const V* G0 = A.g + (size_t)A.cls_of[i] * A.N_ell * A.n_h;
   const int n_in = A.n_h - A.n0;
   for (int s = 0; s < A.r; ++s) {
@@ -535,7 +536,7 @@ k_chirp_fwd(T* __restrict__ delta, const CT* __restrict__ coef, ChirpArgs<T> A) 
   }
 }
 
-// The transpose: part[chunk][(w, i, s)][n] = sum over the chunk's multipoles of
+// The transpose: part[chunk][(w, i, s)][n] = sum over the multipoles of share chunk0 + chunk of
 // G[l][n] sum_q [kw_is[q] Dbar_i(l, q) b_q] h_{n - q}  (n0 = 0); the chunks are added in FP64 by
 // k_chirp_sum.
 template <int LOGM, class T, bool HALF>
@@ -552,7 +553,7 @@ k_chirp_adj(V2<T>* __restrict__ part, const T* __restrict__ dbar, ChirpArgs<T> A
   const int i = wi % A.N_tr, w = wi / A.N_tr;
   const int lo = A.off ? A.off[w] : 0;
   int u0, u1;
-  chunk_range(A.off ? A.off[w + 1] - lo : A.n_l, A.n_chunk, chunk, u0, u1);
+  chunk_range(A.off ? A.off[w + 1] - lo : A.n_l, A.n_total, A.chunk0 + chunk, u0, u1);
   const V* G0 = A.g + (size_t)A.cls_of[i] * A.N_ell * A.n_h;
   const size_t rows = (size_t)(gridDim.x / A.n_chunk) * A.r;
   for (int s = 0; s < A.r; ++s) {

@@ -27,6 +27,7 @@ ChirpArgs<double> args(const ChirpDir& d, const ChirpRun& r, const cplx* g, cons
   A.idx = r.idx;
   A.N_tr = r.N_tr; A.NI = r.NI; A.n_h = r.n_h; A.N_k = r.N_k; A.N_ell = r.N_ell;
   A.l_lo = r.l_lo; A.n_l = r.n_l; A.r = r.rank; A.n0 = d.n0; A.n_chunk = r.n_chunk;
+  A.n_total = r.n_total; A.chunk0 = r.chunk0;
   return A;
 }
 

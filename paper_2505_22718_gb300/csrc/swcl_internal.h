@@ -127,9 +127,10 @@ struct ChirpDir {
   int n0 = 0;           // first frequency of the transform
   DevBuf tab;
 };
-// one launch: shapes, multipoles, transforms per row, CTAs per row, ragged lists (null: all)
+// one launch: shapes, multipoles, transforms per row, CTAs per row (n_chunk of the n_total shares of the
+// multipoles, from chunk0 on), ragged lists (null: all)
 struct ChirpRun {
-  int n_walk, N_tr, NI, n_h, N_k, N_ell, l_lo, n_l, rank, n_chunk;
+  int n_walk, N_tr, NI, n_h, N_k, N_ell, l_lo, n_l, rank, n_chunk, n_total, chunk0;
   const int* off;
   const int* idx;
 };

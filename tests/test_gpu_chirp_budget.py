@@ -210,3 +210,51 @@ def test_mixed_step_between_calls_that_do_not_fit():
         assert {"basis head", "chirp fwd f32"} <= _routes(ctx, lambda: ctx.compute_cl(S.SWCL_SPLIT_BF16))
     check(step(ctx, S.SWCL_SPLIT_BF16))
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", ["bf16x9", "fp64"])
+def test_partial_sums_that_do_not_all_fit(prec):
+    """600 multipoles of two tracers, whose partial sums take more memory than 250 multipoles of Delta and
+    Delta bar: just below the budget that holds them all beside 8 multipoles, longer chunks are planned
+    with one partial sum per row.  In the mixed form no FP32 sum may cover more than 16 multipoles:
+    the transpose then runs in groups, several launches per Delta bar."""
+    import paper_2505_22718_gb300 as S
+    p = S.PRECISIONS[prec]
+    w, rng = _case(1024, 512, 600, n_tr=2)
+    Cb = rng.standard_normal((600, 2, 2))
+    free = lib_context(w)
+    C = free.compute_cl(p)
+    P, A, W = free.vjp(Cb, p)
+    most = free.query(S.SWCL_Q_WORKSPACE_BYTES)
+    free.close()
+
+    def run(budget):
+        """(results, chunks of multipoles, launches of the transpose) or None"""
+        ctx = _context(w, budget)
+        if ctx is None:
+            return None
+        got = []
+        try:
+            if _over_budget(lambda: got.append(ctx.compute_cl(p))):
+                return None
+            S.swcl_profile_enable(ctx.ptr, True)
+            if _over_budget(lambda: got.extend(ctx.vjp(Cb, p))):
+                return None
+            n = S.swcl_profile_read(ctx.ptr)
+            assert ctx.query(S.SWCL_Q_WORKSPACE_BYTES) <= budget
+            k = "fp64" if prec == "fp64" else "f32"
+            return got, n["delta_bar " + k][0], n.get("chirp adj " + k, (0,))[0]
+        finally:
+            ctx.close()
+
+    least = _smallest_budget(lambda b: run(b) is not None, most + (64 << 20))
+    groups = 0
+    for b in np.linspace(least, most, 12).astype(int):   # from 8 multipoles to all, one partial sum to all
+        got, n_delta, n_adj = run(int(b))
+        if prec == "fp64":   # the direct sums at the smallest budgets
+            _same(got, (C, P, A, W), 1e-10)
+            continue
+        assert np.array_equal(got[0], C) and np.array_equal(got[1], P) and np.array_equal(got[2], A)
+        assert max_rel(got[3], W) < 1e-5   # as in the other tests of budgets
+        groups = max(groups, n_adj - n_delta)
+    assert groups > 0 or prec == "fp64"
