@@ -28,6 +28,9 @@ int ensure(swcl_ctx* c, DevBuf& b, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (b.p && b.bytes >= bytes) return SWCL_OK;
   size_t freed = b.p ? b.bytes : 0;
+  // the chirp transpose's partial sums, which take what room there is and hold nothing between calls, give way
+  if (c->budget && c->held - freed + bytes > c->budget && &b != &c->ws_ckpart && !c->capturing)
+    release(c, c->ws_ckpart);
   if (c->budget && c->held - freed + bytes > c->budget)
     return fail(c, SWCL_ERR_OOM_BUDGET,
                 "memory budget exceeded: need " + std::to_string(c->held - freed + bytes) +
@@ -760,7 +763,9 @@ static int check_ready(swcl_ctx* c, int precision) {
 // Dbar (and, in basis mode, the per-call GEMM operands) for every multipole at once.  Then the
 // forward pass contracts and integrates chunk by chunk, and the VJP recomputes each chunk's
 // Delta before its reverse mode.  Returns 0 when not even 8 multipoles fit.
-static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need, bool whole_part) {
+// part: the partial sums of the transpose to make room for.
+enum class Part { none, one, all };
+static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need, Part part) {
   // n_need: the multipoles that take the FFTLog path (all but the Limber rows)
   if (n_need <= 0) return c->N_ell;
   const int N_ell = c->N_ell;
@@ -781,7 +786,7 @@ static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need, bool whole_par
                  + swcl::delta_bar_scratch_bytes(c->n_walk, c->N_k, N_ell)
                  + sizeof(double) * (nw * c->N_k + nrow);
   if (basis) fixed += swcl::basis_fixed_bytes(c);
-  fixed += swcl::chirp_part_bytes(c, precision, n_need, whole_part);
+  if (part != Part::none) fixed += swcl::chirp_part_bytes(c, precision, n_need, part == Part::all);
   const DevBuf* ws[] = {&c->ws_coef, &c->ws_delta, &c->ws_U, &c->ws_C, &c->ws_cbar, &c->ws_dbar,
                         &c->ws_Cbar, &c->ws_outP, &c->ws_outA, &c->ws_outW, &c->ws_pbpart,
                         &c->ws_qpart, &c->ws_ckpart, &c->bt_eimg_f, &c->bt_eimg_a, &c->bt_gdf, &c->bt_g32, &c->bt_kmu,
@@ -796,16 +801,16 @@ static int plan_ell_chunk(swcl_ctx* c, int precision, int n_need, bool whole_par
 }
 
 // The same with the tables of the chirp transforms built first.  Where the budget has no room for 8
-// multipoles beside them, their partial sums are planned at the least; then the FP64 form gives them up,
-// until other grids or tracers are set.
-static int plan_chunk(swcl_ctx* c, int precision, int n_need, int& n_lc) {
+// multipoles beside them, the least of the partial sums asked for is planned (one per row where a
+// transpose may follow); then the FP64 form gives the tables up, until other grids or tracers are set.
+static int plan_chunk(swcl_ctx* c, int precision, int n_need, Part part, int& n_lc) {
   SWCL_TRY(swcl::chirp_prepare(c, precision));
-  n_lc = plan_ell_chunk(c, precision, n_need, true);
+  n_lc = plan_ell_chunk(c, precision, n_need, part);
   if (n_lc == 0 && swcl::chirp_use(c, precision)) {
-    n_lc = plan_ell_chunk(c, precision, n_need, false);
+    if (part == Part::all) n_lc = plan_ell_chunk(c, precision, n_need, Part::one);
     if (n_lc == 0 && precision == SWCL_FP64) {
       SWCL_TRY(swcl::chirp_drop(c));
-      n_lc = plan_ell_chunk(c, precision, n_need, true);
+      n_lc = plan_ell_chunk(c, precision, n_need, part);
       if (n_lc == 0) c->ck_off = false;   // of no use: a smaller call may have room for them
     }
   }
@@ -923,7 +928,7 @@ int swcl_compute_cl(swcl_ctx* c, int precision, double* C_out) {
   swcl::LimberTable lt;
   if (lim.n_lim > 0) SWCL_TRY(limber_prepare(c, lim, nw, lt));
   int n_lc = 0;
-  SWCL_TRY(plan_chunk(c, precision, n_fft, n_lc));
+  SWCL_TRY(plan_chunk(c, precision, n_fft, c->fwd_only ? Part::one : Part::all, n_lc));
   SWCL_TRY(swcl::ensure(c, c->ws_coef, sizeof(cplx) * nrow * N_I * n_h));
   SWCL_TRY(swcl::ensure(c, c->ws_delta, nrow * n_lc * N_k * (fp64 ? sizeof(double) : sizeof(float))));
   SWCL_TRY(swcl::ensure(c, c->ws_U, sizeof(double) * nw * (size_t)N_ell * N_tr * N_tr));
@@ -1188,7 +1193,9 @@ static int batched_body(swcl_ctx* c, int precision, double* C_out, const double*
     if (e != cudaSuccess) return swcl::cuda_fail(c, e, "unpack cotangent");
   }
   c->overlap = overlap;
+  c->fwd_only = C_bar == nullptr;
   int st = swcl_compute_cl(c, precision, C_out);
+  c->fwd_only = false;
   const int64_t n_fwd = c->last_launches;
   if (st == SWCL_OK && C_bar) {
     st = swcl_vjp(c, precision, C_bar, P_bar, amp_bar, W_bar);
@@ -1489,7 +1496,7 @@ int swcl_jvp(swcl_ctx* c, int precision, int n_dir, const double* P_dot, const d
       ~KeepOff() { c->ck_off = off; }
     } keep{c, c->ck_off};
     int n_lc = 0;
-    SWCL_TRY(plan_chunk(c, precision, n_fft, n_lc));
+    SWCL_TRY(plan_chunk(c, precision, n_fft, Part::none, n_lc));
     c->ell_chunk = n_lc;
     c->ell_fft = n_fft;
     SWCL_TRY(swcl::ensure(c, c->ws_coef, sizeof(cplx) * nw2 * N_tr * N_I * n_h));

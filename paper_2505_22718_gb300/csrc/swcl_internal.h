@@ -263,6 +263,7 @@ struct swcl_ctx {
   unsigned char* stage = nullptr;
   size_t stage_off = 0;
   cudaEvent_t ev_stage = nullptr;   // after the last copy out of `stage`
+  bool fwd_only = false;     // the forward pass of a batched call without a cotangent
   int last_fwd_precision = -1;
   int ell_chunk = 0;         // multipoles per Delta chunk of the last forward pass (N_ell = whole)
   int ell_fft = 0;           // multipoles on the FFTLog path in the last forward pass (Limber after)

@@ -258,3 +258,63 @@ def test_partial_sums_that_do_not_all_fit(prec):
         assert max_rel(got[3], W) < 1e-5   # as in the other tests of budgets
         groups = max(groups, n_adj - n_delta)
     assert groups > 0 or prec == "fp64"
+
+
+def test_forward_mode_pays_for_no_transpose():
+    """Forward mode of the FP64 form has no transpose: the smallest budget under which its multipoles stay in
+    one chunk is what it holds, the cotangent's arrays that every plan counts, and no partial sums
+    (44 MB here)."""
+    import paper_2505_22718_gb300 as S
+    n_ell, n_dir, n_tr, N, n_k = 600, 8, 2, 1024, 512
+    w, rng = _case(N, n_k, n_ell, n_tr=n_tr)
+    W_dot = rng.standard_normal((n_dir,) + w.W.shape[1:]) * w.W[0]
+    free = lib_context(w)
+    J = free.jvp(W_dot=W_dot)
+    most = free.query(S.SWCL_Q_WORKSPACE_BYTES)
+    free.close()
+
+    def run(budget):
+        ctx = _context(w, budget)
+        if ctx is None:
+            return None
+        try:
+            got = []
+            if _over_budget(lambda: got.append(ctx.jvp(W_dot=W_dot))) or ctx.query(S.SWCL_Q_RECOMPUTE):
+                return None
+            return got[0]
+        finally:
+            ctx.close()
+
+    b = _smallest_budget(lambda x: run(x) is not None, most + (256 << 20))
+    assert np.array_equal(run(b), J)
+    nw, n_h = 1 + n_dir, N // 2 + 1
+    rows = nw * n_tr
+    counted = (8 * rows * n_ell * n_k            # Delta bar
+               + 16 * rows * n_h                 # cbar
+               + 8 * nw * n_k * n_ell            # the parts of P_bar
+               + 3 * 8 * nw * n_ell * n_tr ** 2  # U and the cotangent of every walker, the staging of C
+               + 8 * nw * n_ell * 2 * 3          # pair sums of the quadrature, of every walker
+               + 8 * (rows * N + nw * n_k + rows))
+    assert b < most + counted + (4 << 20)
+
+
+def test_partial_sums_give_way():
+    """A VJP whose partial sums (10 MB) fill the budget, then a call that needs 2 MB more: it has them, and
+    the VJP after it works with what is left."""
+    import paper_2505_22718_gb300 as S
+    w, rng = _case(1024, 512, 600, n_tr=2)
+    Cb, X = rng.standard_normal((600, 2, 2)), rng.standard_normal((50, 600, 2, 2))
+    modes, noise = np.ones(600), np.full(2, 1e-8)
+    free = lib_context(w)
+    C = free.compute_cl(S.SWCL_FP64)
+    g = free.vjp(Cb, S.SWCL_FP64)
+    held = free.query(S.SWCL_Q_WORKSPACE_BYTES)
+    F = free.gaussian_fisher(X, modes, noise)
+    free.close()
+    ctx = lib_context(w, budget=held + (1 << 20))
+    for _ in range(2):
+        _same([ctx.compute_cl(S.SWCL_FP64)], [C], 1e-10)
+        _same(ctx.vjp(Cb, S.SWCL_FP64), g, 1e-10)
+        _same([ctx.gaussian_fisher(X, modes, noise)], [F], 1e-9)
+    assert ctx.query(S.SWCL_Q_WORKSPACE_BYTES) <= held + (1 << 20)
+    ctx.close()
