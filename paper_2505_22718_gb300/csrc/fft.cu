@@ -482,9 +482,9 @@ k_fftlog_adj_cl(double* __restrict__ W_bar, const cplx* __restrict__ cbar,
 }
 
 // The cluster form serves few rows (fewer than a quarter of the SMs' worth) of a length the
-// four-step split supports.
+// four-step split supports and whose eight arrays per CTA fit 48 KB of shared memory (N <= 4096).
 bool use_cluster(long rows, int N) {
-  return rows * kCl <= 2L * 152 && N >= 256 && N / 2 / kCl <= 2 * kClThreads;
+  return rows * kCl <= 2L * 152 && N >= 256 && 8 * (N / 2 / kCl) * sizeof(cplx) <= 48 * 1024;
 }
 
 }  // namespace
