@@ -322,6 +322,12 @@ class Context:
             n *= d
         return n
 
+    def _points(self, n_walk):
+        """New inputs for n_walk points; as many as before keep their multipole lists, as in the library."""
+        if n_walk != self.n_walk:
+            self.n_walk = n_walk
+            self.n_out = n_walk * self.n_ell
+
     def close(self):
         if self.ptr:
             swcl_destroy(self.ptr)
@@ -348,8 +354,7 @@ class Context:
         _need(D, self._shape(self.n_knots, self.N), "D [N_knots][N]")
         _need(B, self._shape(self.n_tr, self.n_knots, self.N), "B [N_tr][N_knots][N]")
         swcl_set_windows(self.ptr, n_walk, W, D, B)
-        self.n_walk = n_walk
-        self.n_out = n_walk * self.n_ell
+        self._points(n_walk)
 
     def set_window_samples(self, W):
         """New window samples for the same walkers, keeping D and B (no host wait)."""
@@ -361,8 +366,7 @@ class Context:
         _need(P, self._shape(n_walk, self.n_k), "P [n_walk][N_k]")
         _need(amp, self._shape(n_walk, self.n_tr), "amp [n_walk][N_tr]")
         swcl_set_power(self.ptr, n_walk, P, amp)
-        self.n_walk = n_walk
-        self.n_out = n_walk * self.n_ell
+        self._points(n_walk)
 
     def set_ell_lists(self, lists=None):
         if lists is None:
