@@ -43,6 +43,7 @@ WORKLOAD_LARGE = ("large: 30 tracers (20 Gaussian clustering bins, sigma_z=0.03 
 
 # measured peaks (MEASURED_PEAKS.json written by the pool driver); FP64 derived below
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12   # 2 DFMA/clk/SM (FMA-loop probe: 1.19 TF/s at 2070 MHz)
+FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12  # 128 FP32 FMA/clk/SM (derived)
 TF32_OVER_BF16 = 1.1 / 2.25                      # nominal dense ratio
 
 
@@ -129,7 +130,21 @@ def algorithmic_work(w, walkers, rank, n_ell_useful=None):
     contraction = 4.0 * n_h * ntr * nk * ell_units
     rows = rank if rank else ni                                 # FFT rows per tracer
     fft = 2.5 * N * np.log2(N) * ntr * rows * walkers           # real FFT of length N per row
+    transforms = ell_units * ntr * (rank if rank else min(ni, 4))
+
+    def chirp(n_in, n_out):
+        m = max(512, 1 << (n_in + n_out - 2).bit_length())
+        return transforms * (10.0 * m * np.log2(m) + 6.0 * (n_in + m + n_out))
+
+    pairs = ell_units * nk * float(ntr + ntr * (ntr + 1))
     return {
+        "chirp fwd fp64": ("alu", chirp(n_h - 1, nk), 1),
+        "chirp adj fp64": ("alu", chirp(nk, n_h), 1),
+        "chirp fwd f32": ("alu32", chirp(n_h - 64, nk), 1),
+        "chirp adj f32": ("alu32", chirp(nk, n_h), 1),
+        "basis head": ("tensor", 4.0 * 64 * nk * transforms, 6),
+        "k-quadrature fp64": ("alu", pairs, 1),
+        "k-quadrature f32": ("alu32", pairs, 1),
         "contract fp64": ("alu", contraction, 1),
         "contract adj fp64": ("alu", contraction, 1),
         "contract tc": ("tensor", contraction, None),
@@ -143,7 +158,9 @@ def algorithmic_work(w, walkers, rank, n_ell_useful=None):
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of a kernel at the
 # benchmark workload (one walker), from the ncu capture summarised in profiles/, valid only for
-# the kernel source it was taken from (sha256 of the file; otherwise reported as null).
+# the kernel source it was taken from (sha256 of the file; otherwise reported as null).  These are captures
+# of the GEMMs over all frequencies, which the benchmark workload runs with SWCL_BASIS_GEMM=1 only, from an
+# earlier state of the file.
 TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture per (kernel, tile code), one
     # walker, N5K-shaped workload (profiles/basis_gemm_n5k_bf16.md); valid while basis_tc.cu is
@@ -236,7 +253,8 @@ def roofline(stats, w, walkers, precision, peaks, src, rank, workload="n5k", ste
     if flops is None:
         return {"kernel": name, "bound": None, "avg_ms": ms / launches, "note": "no algorithmic count"}
     per_step = launches / steps if steps else 1.0
-    reps = 2 if recompute and name in ("basis gemm fwd", "contract fp64") else 1
+    reps = 2 if recompute and name in ("basis gemm fwd", "contract fp64", "basis head", "chirp fwd f32",
+                                       "chirp fwd fp64") else 1
     flops = flops * reps / per_step
     useful = flops / avg_s / 1e12
     if bound == "tensor":
@@ -255,7 +273,10 @@ def roofline(stats, w, walkers, precision, peaks, src, rank, workload="n5k", ste
                 "products": products, "traffic": traffic_for(name, walkers, workload, tiles),
                 "avg_ms": ms / launches, "launches": launches, "peak_source": note,
                 "work": "4 n_h N_tr N_k N_ell useful flops per evaluation (%.3g per launch)" % flops}
-    if peaks.get("fp64_tflops"):
+    if bound == "alu32":
+        peak = FP32_PEAK_TFLOPS
+        note = "FP32 FMA pipes: 152 SMs x 128 FMA/clk x 2 flop x 2.07 GHz (derived)"
+    elif peaks.get("fp64_tflops"):
         peak = peaks["fp64_tflops"]
         note = "FP64 dense rate measured in this run (cuBLAS DGEMM); derived DFMA pipe %.2f TF/s" % FP64_PEAK_TFLOPS
     else:
@@ -938,7 +959,8 @@ def main():
                  "3xtf32": "tf32x3 tensor-core contraction (f32 accumulate) + f64 FFT/Gamma/k-sum",
                  "tf32x6": "tf32x6 tensor-core contraction (f32 accumulate) + f64 FFT/Gamma/k-sum",
                  "bf16x9": "split-bf16 tensor-core contraction (3+3 planes, 6 products in basis mode; "
-                           "f32 accumulate) + f64 FFT/Gamma/k-sum"}[args.precision]
+                           "f32 accumulate), on k grids uniform in ln k of the lowest 64 to 256 frequencies, "
+                           "with f32 chirp FFTs of the rest + f64 FFT/Gamma + f32 k-sum, compensated"}[args.precision]
         line = {"metric": METRIC, "value": out["value"], "unit": "evals/s", "n_gpus": world,
                 "steps": args.steps, "warmup": args.warmup, "ms_per_step": out["ms_per_step"],
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": dtype,
