@@ -282,7 +282,7 @@ def roofline(stats, w, walkers, precision, peaks, src, rank, workload="n5k", ste
     else:
         peak = FP64_PEAK_TFLOPS
         note = "FP64 FMA pipe: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz (derived)"
-    return {"kernel": name, "bound": "alu", "achieved": useful, "peak": peak, "unit": "TFLOP/s",
+    return {"kernel": name, "bound": bound, "achieved": useful, "peak": peak, "unit": "TFLOP/s",
             "frac": useful / peak, "traffic": traffic_for(name, walkers, workload, tiles),
             "avg_ms": ms / launches, "launches": launches, "peak_source": note,
             "work": "%.3g useful flops per launch" % flops}
