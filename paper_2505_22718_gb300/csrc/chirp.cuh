@@ -29,7 +29,7 @@
 // FP32: bound by shared-memory and table accesses (1750 wavefronts of the load/store pipe per row of
 // 2048 points) and, close behind, by instruction issue: about 2070 clocks per row and SM with four
 // resident CTAs (16 warps).  1545 such rows 19 us forward and 20 us transposed; 287 100 rows (256 walkers
-// with ragged lists) 1.89 and 1.85 ms; 89 970 rows of 8192 points 3.78 and 3.28 ms.  The GEMMs over all
+// with ragged lists) 1.89 and 1.80 ms; 89 970 rows of 8192 points 3.74 and 3.21 ms.  The GEMMs over all
 // frequencies took 56 and 58 us, 7.9 and 12.3 ms, 14.6 and 11.9 ms, with another 23 us, 1.7 ms and
 // 1.5 ms for their operand images.  Errors against 64 bits (N5K shape): Delta 1.3e-7 (GEMMs 1.9e-7),
 // normalised C 2.7e-5 (3.1e-5), W_bar 4.2e-7 (9.7e-7); white-noise windows 1.6e-7 (1.4e-7), 5.9e-5
@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "f32x2.cuh"
 #include "swcl_internal.h"
 
 namespace swcl {
@@ -53,26 +54,8 @@ template <class V> __device__ __forceinline__ V add(V a, V b) { a.x += b.x; a.y 
 template <class V> __device__ __forceinline__ V sub(V a, V b) { a.x -= b.x; a.y -= b.y; return a; }
 // FP32: both components in one instruction (the same two roundings); 2.12 -> 1.96 ms forward and 2.22 ->
 // 1.89 ms transposed for 287 100 rows of 2048 points, together with the constant offsets below
-__device__ __forceinline__ unsigned long long pk(float2 a) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
-  return r;
-}
-__device__ __forceinline__ float2 upk(unsigned long long a) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
-  return r;
-}
-template <> __device__ __forceinline__ float2 add<float2>(float2 a, float2 b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pk(a)), "l"(pk(b)));
-  return upk(r);
-}
-template <> __device__ __forceinline__ float2 sub<float2>(float2 a, float2 b) {
-  unsigned long long r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pk(a)), "l"(pk(b)));
-  return upk(r);
-}
+template <> __device__ __forceinline__ float2 add<float2>(float2 a, float2 b) { return f2_add(a, b); }
+template <> __device__ __forceinline__ float2 sub<float2>(float2 a, float2 b) { return f2_sub(a, b); }
 // a + c b and a - c b with a real constant c
 template <class V, class T> __device__ __forceinline__ V axpy(T c, V b, V a) {
   a.x = fma(c, b.x, a.x);
@@ -80,9 +63,7 @@ template <class V, class T> __device__ __forceinline__ V axpy(T c, V b, V a) {
   return a;
 }
 template <> __device__ __forceinline__ float2 axpy<float2, float>(float c, float2 b, float2 a) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pk(make_float2(c, c))), "l"(pk(b)), "l"(pk(a)));
-  return upk(r);
+  return f2_fma(make_float2(c, c), b, a);
 }
 // a b, and a conj(b)
 template <class V> __device__ __forceinline__ V mul(V a, V b) {
@@ -150,7 +131,9 @@ __host__ __device__ constexpr double sin32(int j) { return cos32(j + 24); }   //
 // e^{2 pi i S J / 32} = tw_scale(J) i^(S k) (1 + i S t), k the nearest quarter turn and t the tangent of the
 // rest, |t| <= 1: tw_tan is the product without the scale, one FMA per component, and the scale goes
 // into the FMAs of the additions that follow.  A 4-point DFT with three constant factors so takes 22
-// operations instead of 28: 16-point passes 144 and not 160, 8-point ones 52 and not 56.
+// operations instead of 28: 16-point passes 144 and not 160, 8-point ones 52 and not 56.  (A published way
+// to fit FFTs to multiply-add units: Linzer and Feig, IEEE Trans. Signal Process. 41, 1993; Goedecker, SIAM J.
+// Sci. Comput. 18, 1997.)
 __host__ __device__ constexpr int tw_quarter(int J) { return ((J & 31) + 4) >> 3; }
 __host__ __device__ constexpr int tw_rest(int J) { return (J & 31) - 8 * tw_quarter(J); }   // -4 .. 3
 __host__ __device__ constexpr double tw_scale(int J) { return cos32(tw_rest(J)); }
