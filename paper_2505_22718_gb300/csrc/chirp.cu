@@ -8,10 +8,13 @@
 namespace swcl {
 
 // ln k_q = x0 + q d to rounding: the line through the end points (their logarithms in extended
-// precision), with no point further off than a few rounding errors of ln k.  The phases
-// e^{-i eta_n ln k_q} of the line then differ from those of the grid by no more than a
-// double-precision ln k does.  Grids that geomspace, logspace or an exponential of a linspace give
-// pass; one rounded to seven digits, or perturbed by 1e-12, does not (tests/test_gpu_chirp.py).
+// precision), with no point further off than 4 eps max(4, |ln k|), eight times the largest rounding error of
+// ln k itself.  A grid as geomspace, logspace or an exponential of a linspace give it, whose points carry the
+// roundings of an exponent and of a power, lies within 1.4 of those 4 (ranges from 1e-12 to 1e6, 150 to
+// 1024 points); the phases e^{-i eta_n ln k_q} of the line differ from those of such a grid about as much as
+// rounding ln k changes them, and by a few times that at the bound: at most 5e-12 at N = 2048, where the results
+// are held to 1e-10.  A grid rounded to seven digits, or perturbed by 1e-12, does not pass
+// (tests/test_gpu_chirp.py).
 void chirp_fit_grid(swcl_ctx* c) {
   c->ck_uniform = false;
   c->ck_off = false;
@@ -68,15 +71,22 @@ bool chirp_use(const swcl_ctx* c, int precision) {
   if (r <= 0 || !mf || !ma) return false;
   // FP64 operations: about 75 per point and pair of FFTs, against 2 per (frequency, k point) of the
   // direct sum (four profile rows cost four transforms but one direct sum).  Both sides are bound by
-  // the FP64 pipe: forward + VJP at N = 2048, N_k = 1024, 103 multipoles, 15 tracers 1.01 ms against
+  // the FP64 pipe: forward + VJP at N = 2048, N_k = 1024, 103 multipoles, 15 tracers 0.95 ms against
   // 12.8 ms; N = N_k = 256, 20 multipoles, 2 tracers (three quarters of the line) 0.24 against 0.79 ms.
+  // Just inside the line the transforms are the faster side by far (20 multipoles, N_k = 152, one row: 0.11 against
+  // 0.65 ms at N = 256, 0.13 against 4.5 ms at N = 2048; N = 8192, N_k = 80 0.56 against 17.7 ms), since the direct
+  // sums also run on too few CTAs there.  The line is where the operations are equal, not where the times are.
   if (precision == SWCL_FP64) return 75.0 * r * (double)(1 << std::max(mf, ma)) < 2.0 * c->n_h * (double)c->N_k;
   // the mixed form: beside the basis-mode GEMMs, unless tiles or products of theirs are asked for
   if (precision != SWCL_SPLIT_BF16 || !c->lr_basis || c->bt_disabled || c->bt_asked) return false;
-  // From N = 1024 on: 15 tracers, 103 multipoles, N = 2048, N_k = 1024 forward + VJP 83 us a step
-  // against 136 us with the GEMMs over all frequencies, 256 such points with ragged lists 11.7 against
-  // 25.1 ms, N = N_k = 4096 with 30 tracers and 2999 multipoles 13.9 against 32.2 ms; at N = 512,
-  // N_k = 333, 7 tracers, 37 multipoles, three points both take 62 us.
+  // From N = 1024 on: 15 tracers, 103 multipoles, N = 2048, N_k = 1024 forward + VJP 59 us a step
+  // against 136 us with the GEMMs over all frequencies, 256 such points with ragged lists 7.5 against
+  // 25.1 ms, N = N_k = 4096 with 30 tracers and 2999 multipoles 11.6 against 32.2 ms; at N = 512,
+  // N_k = 333, 7 tracers, 37 multipoles, three points both take 62 us.  Few k points do not move the line: 64 of
+  // them, 7 tracers, 103 multipoles, one and 16 points 70 and 159 us against 82 and 205 us at N = 1024, 90 and 423
+  // against 142 and 564 us at N = 4096, 256 and 902 against 365 and 1025 us at N = 8192.  The GEMMs win, forward
+  // alone, where all rows keep 256 frequencies (k_head) and those are half of them: N = 1024 with sigma_z = 0.02
+  // above z = 0.6, finer than that grid resolves, 78 against 64 us, and equal at N = 2048.
   return c->N >= 1024;
 }
 
