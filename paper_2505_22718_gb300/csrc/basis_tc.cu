@@ -1806,7 +1806,7 @@ __global__ void __maxnreg__(32) k_dimg(uint8_t* __restrict__ img, const float* _
 // choice of rounds), 89 970 columns x 4096 k 2.0 ms at 1 to 4 rounds a row (0.81 ms with one); the GEMM kernels
 // with their H image took 24 us, 3.6 ms and 1.9 ms for the K of one round.
 // Warps: 0 copies, 1 MMA and TMEM, 2-9 form H, then drain (two warps per 32-lane quarter, 32 columns
-// each) and store, 10-11 find the rounds of the tile's rows during the first one.  Columns: each half of a
+// each) and store, 10-11 find the rounds of the tile's rows while the first one's H is formed.  Columns: each half of a
 // tile holds 32/r whole groups of r profile rows.
 constexpr int kHeadNT = 64;
 constexpr int kHeadKb = 2 * kChirpHead / kK;               // 4 K-blocks a round
@@ -1993,8 +1993,12 @@ k_head(float* __restrict__ delta, const uint8_t* __restrict__ aimg, const float4
         store_planes<kPlanes>(bsm + kb * kHeadB, kHeadNT * kRow, off64(row, ch * 16), v);
       }
       fence_proxy_async();
-    } else if (warp >= 10 && rd == 0) {
-      // rounds of each row of the tile, one warp a row.  A row's columns are neighbours
+    }
+    if (warp >= 2 && rd == 0) {
+      // Rounds of each row of the tile, one warp a row: the first two by warps 10 and 11 while H is formed,
+      // further ones (few multipoles per row) by all ten: 48 points of 15 tracers, one multipole each, forward
+      // 141 us with two warps, 113 us so (94 us with 64 frequencies for every row).  A row's columns are
+      // neighbours
       const int gh = 32 / sh.r;
       auto row_of = [&](int half) {   // walker N_tr + tracer of column 32 half + lane (-1: no column)
         const int gi = lane / sh.r, g = (2 * ct + half) * gh + gi;
@@ -2009,7 +2013,7 @@ k_head(float* __restrict__ delta, const uint8_t* __restrict__ aimg, const float4
         int wi;
         if (f0) { wi = __shfl_sync(0xffffffffu, w0, __ffs(f0) - 1); f0 &= f0 - 1; }
         else { wi = __shfl_sync(0xffffffffu, w1, __ffs(f1) - 1); f1 &= f1 - 1; }
-        if ((k & 1) != warp - 10) continue;
+        if ((k + 8) % 10 != warp - 2) continue;
         const int need = head_rounds(F + (size_t)wi * sh.NI * sh.n_h, sh.r, sh.n_h, lane);
         if (w0 == wi) colrd[lane] = need;
         if (w1 == wi) colrd[32 + lane] = need;
