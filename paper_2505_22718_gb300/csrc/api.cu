@@ -1398,6 +1398,8 @@ int swcl_step_host(swcl_ctx* c, int precision, const double* W, const double* P,
     c->hgraph_key.alloc_gen = gen;
     for (int t = 0; t < 8; ++t) c->hgraph_key.ptrs[t] = ptrs[t];
     c->hgraph_launches = c->last_launches;
+    c->hgraph_chunk = c->ell_chunk;
+    c->hgraph_fft = c->ell_fft;
   }
   SWCL_TRY_CUDA(c, cudaGraphLaunch(c->hgraph_exec, c->stream), "graph launch");
   // wait by polling an event: a sampler's step is short (a fraction of a millisecond), and a
@@ -1412,6 +1414,9 @@ int swcl_step_host(swcl_ctx* c, int precision, const double* W, const double* P,
   }
   c->last_launches = c->hgraph_launches;
   c->last_fwd_precision = precision;
+  // Delta lies in the chunks of this step, whatever calls came between its capture and its replay
+  c->ell_chunk = c->hgraph_chunk;
+  c->ell_fft = c->hgraph_fft;
   const int h = *c->hs_status;
   if (h) {
     *c->hs_status = 0;

@@ -288,6 +288,7 @@ struct swcl_ctx {
     int64_t alloc_gen = -1;
   } hgraph_key;
   int64_t hgraph_launches = 0;
+  int hgraph_chunk = 0, hgraph_fft = 0;   // ell_chunk and ell_fft of the captured step
   swcl::DevBuf hs_C, hs_Cb, hs_Pb, hs_Ab, hs_Wb;   // device side of the step's arrays
   int* hs_status = nullptr;                        // page-locked copy of the status word
   cudaEvent_t ev_host = nullptr;                   // end of the step, polled by the host
